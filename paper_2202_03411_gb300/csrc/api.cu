@@ -179,6 +179,7 @@ void scatman_destroy(scatman_handle *h) {
     cudaFree(h->d_tail);
     cudaFree(h->d_H);
     cudaFree(h->d_uq_qz);
+    cudaFree(h->d_fg);
     cudaFree(h->d_uq_qrow);
     cudaFree(h->d_adj_part);
     cudaFree(h->d_gmax);
@@ -266,6 +267,22 @@ static bool check_param_shape(const scatman_shape *s, std::string *why) {
     return true;
 }
 
+// q of the detector's pixels into d_q.
+static int fill_detector_q(scatman_handle *h) {
+    const scatman_config &c = h->cfg;
+    return check_cuda(h, h->uniform_q ? launch_detector_q_uniform(c.det_nx, c.det_ny, c.theta_max_deg, h->k0, h->d_q,
+                                                                  h->stream)
+                                      : launch_detector_q(c.det_nx, c.det_ny, c.theta_max_deg, h->k0, h->d_q, h->stream),
+                      "detector q");
+}
+
+// The same for a handle whose forward pass does without it (the sample grid).
+static int need_q(scatman_handle *h) {
+    if (h->d_q) return SCATMAN_OK;
+    const int rc = alloc_dev(h, (void **)&h->d_q, (size_t)h->n_pix * 3 * sizeof(double), "q buffer");
+    return rc ? rc : fill_detector_q(h);
+}
+
 int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle **out) {
     if (!out) return SCATMAN_ERR_ARG;
     *out = nullptr;
@@ -309,13 +326,14 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
     // device
     if (cudaGetDevice(&h->device) != cudaSuccess)
         return fail(set_error(h, SCATMAN_ERR_UNSUPPORTED, "no CUDA device"));
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, h->device) != cudaSuccess)
+    int major = 0, minor = 0;
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, h->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, h->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
         return fail(set_error(h, SCATMAN_ERR_UNSUPPORTED, "cannot query the CUDA device"));
-    if (!(prop.major == 10 && prop.minor == 3))
+    if (!(major == 10 && minor == 3))
         return fail(set_error(h, SCATMAN_ERR_UNSUPPORTED,
                               "this library is built for sm_103a (compute capability 10.3) only"));
-    h->sm_count = prop.multiProcessorCount;
 
     if (h->tensor_core) {
         h->Nxp = (int)round_up(c.nx, 16);
@@ -341,7 +359,8 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
     const size_t npix = (size_t)h->n_pix;
     const bool f64 = (h->precision == SCATMAN_FP64);
     int rc;
-    if ((rc = alloc_dev(h, (void **)&h->d_q, npix * 3 * sizeof(double), "q buffer"))) return fail(rc);
+    h->on_grid = use_field_grid(*cfg, &h->fg);
+    if (!h->on_grid && (rc = alloc_dev(h, (void **)&h->d_q, npix * 3 * sizeof(double), "q buffer"))) return fail(rc);
     if ((rc = alloc_dev(h, (void **)&h->d_chi, nvox * sizeof(float), "occupancy buffer"))) return fail(rc);
     // per-slice occupied boxes (every mode skips the empty parts of each
     // slice), then the tensor-core kernel's occupied-slice list
@@ -357,12 +376,20 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
     if ((rc = alloc_dev(h, &h->d_A, npix * cx, "field buffer"))) return fail(rc);
     if ((rc = alloc_dev(h, &h->d_I, npix * (f64 ? 8 : 4), "intensity buffer"))) return fail(rc);
     if ((rc = alloc_dev(h, (void **)&h->d_err, kStatusBytes, "status block"))) return fail(rc);
-    if (h->uniform_q && (rc = alloc_dev(h, (void **)&h->d_uq_qz, npix * sizeof(float2), "q_z table")))
+    if (h->on_grid) {
+        if ((rc = alloc_dev(h, (void **)&h->d_fg, field_grid_layout(&h->fg, h->tensor_core, h->Nxp, nullptr),
+                            "field sample grid")))
+            return fail(rc);
+        field_grid_layout(&h->fg, h->tensor_core, h->Nxp, h->d_fg);
+    }
+    if (h->uniform_q && !h->on_grid && (rc = alloc_dev(h, (void **)&h->d_uq_qz, npix * sizeof(float2), "q_z table")))
         return fail(rc);
     if (h->uniform_tc &&
         (rc = alloc_dev(h, (void **)&h->d_uq_qrow, (size_t)c.det_ny * 3 * sizeof(double), "detector row q")))
         return fail(rc);
-    if (h->uniform_tc) {
+    if (h->on_grid) {
+        // (its sums live in the grid's own buffers)
+    } else if (h->uniform_tc) {
         const size_t hb = uq_tc_h_bytes(c.nx, c.nz, c.det_ny);
         // (zeroed by each forward before the y-sum writes its occupied part)
         if ((rc = alloc_dev(h, &h->d_H, hb, "y-contracted slices"))) return fail(rc);
@@ -384,13 +411,10 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
                         "q upload");
         if (rc) return fail(rc);
         if ((rc = check_cuda(h, cudaStreamSynchronize(h->stream), "q upload"))) return fail(rc);
+    } else if (h->on_grid) {
+        if ((rc = check_cuda(h, launch_field_grid_tables(h->fg, h->stream), "field sample grid"))) return fail(rc);
     } else {
-        rc = check_cuda(h, h->uniform_q ? launch_detector_q_uniform(c.det_nx, c.det_ny, c.theta_max_deg, h->k0,
-                                                                    h->d_q, h->stream)
-                                         : launch_detector_q(c.det_nx, c.det_ny, c.theta_max_deg, h->k0, h->d_q,
-                                                             h->stream),
-                        "detector q");
-        if (rc) return fail(rc);
+        if ((rc = fill_detector_q(h))) return fail(rc);
     }
     if (h->tensor_core) {
         std::string why;
@@ -398,7 +422,7 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
             return fail(set_error(h, SCATMAN_ERR_CUDA, why));
         h->have_tmap = true;
     }
-    if (h->uniform_q &&
+    if (h->uniform_q && !h->on_grid &&
         (rc = check_cuda(h, launch_uq_qz_table(h->d_q, h->n_pix, h->k0, h->d_uq_qz, h->stream), "q_z table")))
         return fail(rc);
     if (h->uniform_tc &&
@@ -669,7 +693,15 @@ int scatman_forward(scatman_handle *h, void *I_dev, void *A_dev) {
     const scatman_config &c = h->cfg;
     const double str_re = h->str_re, str_im = h->str_im;     // set by voxelise
     cudaError_t e;
-    if (h->uniform_tc) {
+    if (h->on_grid && h->tensor_core) {
+        e = launch_rows_y_tc(h->tmap_B, h->fg.qrow, 2 * h->fg.Hs, c.nx, c.ny, c.nz, h->Nxp, h->Nyp, c.voxel, h->split,
+                             h->s_bf16, h->d_bounds, (float2 *)h->fg.H, h->d_err, h->sm_count, h->stream);
+        if (e == cudaSuccess)
+            e = launch_field_grid_tc(h->fg, h->Nxp, h->d_bounds, geom_chunk_y(h->d_bounds, c.nz), str_re, str_im,
+                                     (float2 *)h->d_A, (float *)I_dev, h->sm_count, h->stream);
+    } else if (h->on_grid) {
+        e = launch_field_grid(h->fg, h->d_s, h->d_bounds, str_re, str_im, h->d_A, I_dev, h->sm_count, h->stream);
+    } else if (h->uniform_tc) {
         // the y sum writes only occupied slices and x spans: the rest of H is zero
         e = cudaMemsetAsync(h->d_H, 0, uq_tc_h_bytes(c.nx, c.nz, c.det_ny), h->stream);
         if (e == cudaSuccess) {
@@ -871,6 +903,15 @@ int scatman_contraction_flops(scatman_handle *h, double *issued, double *dense) 
                         "slice geometry download");
     if (rc) return rc;
     if ((rc = scatman_sync(h))) return rc;
+    if (h->on_grid) {
+        // the y-sum of the sample grid's rows: on the tensor cores as issued, else
+        // four flops a folded term (dense: the direct sums over the detector's pixels)
+        const FieldGrid &f = h->fg;
+        *dense = 8.0 * dense_pairs * (h->split ? 2.0 : 1.0);
+        *issued = h->tensor_core ? tc_issued_flops(b.data(), c.nz, h->Nxp, h->Nyp, 2 * f.Hs, h->split)
+                                 : 8.0 * (double)f.Hs * f.Ky * c.nx * c.nz;
+        return SCATMAN_OK;
+    }
     if (!h->tensor_core) {
         *dense = 8.0 * dense_pairs;
         *issued = h->uniform_q ? *dense : simt_issued_flops(b.data(), c.nz, c.ny, h->n_pix, h->precision == SCATMAN_FP64);
@@ -883,7 +924,9 @@ int scatman_contraction_flops(scatman_handle *h, double *issued, double *dense) 
 
 int scatman_get_q(scatman_handle *h, double *q_host) {
     if (!h || !q_host) return SCATMAN_ERR_ARG;
-    int rc = check_cuda(h, cudaMemcpyAsync(q_host, h->d_q, (size_t)h->n_pix * 3 * sizeof(double),
+    int rc = need_q(h);
+    if (rc) return rc;
+    rc = check_cuda(h, cudaMemcpyAsync(q_host, h->d_q, (size_t)h->n_pix * 3 * sizeof(double),
                                            cudaMemcpyDeviceToHost, h->stream),
                         "q download");
     if (rc) return rc;
@@ -1013,7 +1056,8 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
     const scatman_config &c = h->cfg;
     const bool f64 = h->precision == SCATMAN_FP64;
     const size_t nvox = (size_t)c.nx * c.ny * c.nz;
-    int rc;
+    int rc = need_q(h);
+    if (rc) return rc;
     if (!h->d_S) {
         if ((rc = alloc_dev(h, &h->d_S, nvox * (f64 ? sizeof(double2) : sizeof(float2)), "adjoint field")))
             return rc;

@@ -169,6 +169,25 @@ struct SliceOut {
     int *chunk_y;                   // per slice and 8-column chunk [y_lo | y_hi] (see above), or null
 };
 
+// The field's sample grid on the Ewald sphere (field_grid.cu): sizes, then
+// device buffers in one allocation.  Passed to its kernels by value.
+struct FieldGrid {
+    int uniform = 0;                // uniform-q detector (rows fix s) instead of the flat one (columns fix t)
+    int elem = 4;                   // bytes of a real number
+    int nx = 0, ny = 0, nz = 0, det_nx = 0, det_ny = 0;
+    int Hs = 0, Ht = 0;             // half the points in s and t
+    int H1 = 0, H2 = 0, n1 = 0;     // per-column (per-row) direction: its half points and half pixels; per-pixel direction
+    int Kx = 0, Ky = 0, U = 0, V = 0;   // half sides of the grid and the detector, rounded up
+    int jc = 0;                     // slice chunks of the x/z sum
+    double sm = 0, tm = 0;          // largest |s|, |t|
+    double k0 = 0, voxel = 0, top = 0;  // top: tan or sin of theta_max
+    void *ty = nullptr, *tx = nullptr, *tz = nullptr;   // phases of the sums
+    void *node2 = nullptr, *w1 = nullptr, *pix = nullptr;   // interpolation: points, weights, pixels
+    double *qrow = nullptr, *point_s = nullptr, *point_t = nullptr;
+    void *H = nullptr, *Q = nullptr, *B = nullptr;      // y-sums, samples, per-column interpolants
+    size_t bytes = 0;
+};
+
 }  // namespace scm
 
 struct scatman_handle {
@@ -234,6 +253,9 @@ struct scatman_handle {
     size_t mindex_cap = 0;
     double str_re = 0, str_im = 0;  // global strength factor of s: n^2 - 1, or the map's index scale
     double map_index_max = 0;       // max |delta|, |beta| over a volume map's cells
+    bool on_grid = false;           // the field goes through its sample grid
+    scm::FieldGrid fg;
+    unsigned char *d_fg = nullptr;  // its buffers
     int splits = 1;
     long long device_bytes = 0;
     scm::TcMaps tmap_B;
@@ -307,10 +329,27 @@ struct UqStore {
     uint16_t *Ht;
     int Jp, Rg, Kx;
     bool bf16;                  // H's 16-bit type
+    float2 *H32 = nullptr;      // FP32 sums instead of the planes (launch_rows_y_tc)
 };
 cudaError_t launch_uq_y_tc_mma(const TcMaps &maps, const double *qrow, int det_ny, int nx, int ny, int nz, int Nxp,
                                int Nyp, double voxel, bool split, bool bf16, int *geom,
                                const UqStore &store, int *err, int sm_count, cudaStream_t st);
+// The same with the rows' sums kept in FP32: H[row][j][x], rows of Nxp, written
+// in the occupied 8-column chunks.
+cudaError_t launch_rows_y_tc(const TcMaps &maps, const double *qrow, int rows, int nx, int ny, int nz, int Nxp,
+                             int Nyp, double voxel, bool split, bool bf16, int *geom, float2 *H, int *err,
+                             int sm_count, cudaStream_t st);
+// The field through its sample grid (field_grid.cu).  plan: whether the
+// detector and box allow it, and its sizes; layout: buffer offsets from base.
+bool plan_field_grid(const scatman_config &c, bool fp64, FieldGrid *f);
+bool use_field_grid(const scatman_config &c, FieldGrid *f);
+size_t field_grid_layout(FieldGrid *f, bool tensor_core, int Nxp, unsigned char *base);
+cudaError_t launch_field_grid_tables(const FieldGrid &f, cudaStream_t st);
+// Forward from the slices (FP32 or FP64), or from the tensor-core y-sums in f.H.
+cudaError_t launch_field_grid(const FieldGrid &f, const void *s, const int *bounds, double str_re, double str_im,
+                              void *A, void *I, int sm_count, cudaStream_t st);
+cudaError_t launch_field_grid_tc(const FieldGrid &f, int Nxp, const int *bounds, const int *chunk_y, double str_re,
+                                 double str_im, float2 *A, float *I, int sm_count, cudaStream_t st);
 // Real flops one contraction launch issues for the recorded slice geometry
 // (a host copy of the first 4 nz + 2 kGeomChunks nz ints of the buffer).
 double tc_issued_flops(const int *geom_host, int nz, int Nxp, int Nyp, long long n_pix, bool split);

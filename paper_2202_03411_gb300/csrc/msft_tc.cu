@@ -93,6 +93,7 @@ struct TcParams {
     // [-Im | Re | Im] of H at rows (3 (v / h_Rg) + plane) h_Jg + (v % h_Rg) h_Jp + j
     uint16_t *Ht;
     int h_Jp, h_Jg, h_Rg, h_Kx, h_bf16;
+    float2 *H32;                // or, when set, FP32 sums at [(m nz + j) Nxp + x]
 };
 
 // Unit word: first chunk c_lo | chunks nch << 5 | shift << 10 | K-step mask << 11.
@@ -499,7 +500,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     tmem_ld8(lane_base + col, gr);
                     tmem_ld8(lane_base + col + nr, gi);
                     tmem_ld_wait8(gr, gi);
-                    if (valid) {
+                    if (valid && P.H32) {
+                        float4 *dst = reinterpret_cast<float4 *>(P.H32 + ((size_t)v * P.nz + t) * P.Nxp + 8 * c);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            dst[e] = make_float4(gr[2 * e], gi[2 * e], gr[2 * e + 1], gi[2 * e + 1]);
+                    } else if (valid) {
                         uint32_t re[4], im[4], mi[4];
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
@@ -798,7 +804,8 @@ static cudaError_t launch_tc(const TcMaps &maps, const double *q, long long n_pi
     P.h_Rg = store ? store->Rg : 1;
     P.h_Kx = store ? store->Kx : 0;
     P.h_bf16 = store && store->bf16 ? 1 : 0;
-    if (store && (store->Kx < Nxp || store->Kx % 8 != 0 || store->Jp < nz)) return cudaErrorInvalidValue;
+    P.H32 = store ? store->H32 : nullptr;
+    if (store && !store->H32 && (store->Kx < Nxp || store->Kx % 8 != 0 || store->Jp < nz)) return cudaErrorInvalidValue;
     const size_t smem = (split ? 2 : 1) * tc_a_bytes(Nyp) + ring + tc_fixed_bytes();
     // The attribute is per function and shared by every thread of the process:
     // always raise it to the largest size any launch uses, never to this
@@ -846,6 +853,16 @@ cudaError_t launch_uq_y_tc_mma(const TcMaps &maps, const double *qrow, int det_n
                                int *err, int sm_count, cudaStream_t st) {
     return launch_tc(maps, qrow, det_ny, nx, ny, nz, Nxp, Nyp, voxel, 1.0, 0.0, split, bf16, geom, nullptr,
                      nullptr, err, sm_count, st, &store, nullptr);
+}
+
+cudaError_t launch_rows_y_tc(const TcMaps &maps, const double *qrow, int rows, int nx, int ny, int nz, int Nxp,
+                             int Nyp, double voxel, bool split, bool bf16, int *geom, float2 *H, int *err,
+                             int sm_count, cudaStream_t st) {
+    UqStore store{};
+    store.H32 = H;
+    store.Rg = 1;
+    return launch_tc(maps, qrow, rows, nx, ny, nz, Nxp, Nyp, voxel, 1.0, 0.0, split, bf16, geom, nullptr, nullptr,
+                     err, sm_count, st, &store, nullptr);
 }
 
 }  // namespace scm

@@ -353,6 +353,9 @@ long long scatman_footprint_bytes(const scatman_config *c) {
     } else {
         b += round_2mib(256LL * 128 * 4 * 8);   // last wave's partial fields (< 256 SMs, <= 4 parts)
     }
+    FieldGrid fg;
+    if (use_field_grid(*c, &fg))                // the field's sample grid: phases, sums, weights
+        b += round_2mib((long long)field_grid_layout(&fg, tc, (c->nx + 15) / 16 * 16, nullptr));
     b += round_2mib(nvox * cx);                 // adjoint field (backward)
     if (tc) {
         // adjoint partial fields (<= 8), scale, pixel table, y-phase operand tiles
