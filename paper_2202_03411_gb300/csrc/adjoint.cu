@@ -423,6 +423,14 @@ static size_t grad_voxel_smem(const ShapeParams &sp) {
     return (size_t)(kGradThreads / 32) * (size_t)(n_geom_params(sp.kind, sp.lmax) - 1) * 32 * sizeof(float);
 }
 
+// The dynamic shared memory attribute of the FP32 kernels, per function and shared by every
+// thread of the process: always the most a shape of this function's degree bound needs,
+// never one launch's size (a concurrent launch of a higher degree would be refused).
+static int grad_voxel_smem_most(const ShapeParams &sp) {
+    const int l = sp.kind == SCATMAN_SPHHARM && sp.lmax > 6 ? SCATMAN_MAX_LMAX : 6;
+    return (kGradThreads / 32) * (n_geom_params(SCATMAN_SPHHARM, l) - 1) * 32 * (int)sizeof(float);
+}
+
 template <typename R>
 using GradVoxelFn = void (*)(ShapeParams, GridParams, const typename Cx<R>::T *, double *);
 
@@ -465,7 +473,7 @@ int grad_voxel_blocks(bool fp64, const ShapeParams &sp, const GridParams &gp, in
     } else {
         const auto fn = grad_voxel_fn<float>(sp, gp);
         const size_t smem = grad_voxel_smem(sp);
-        ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+        ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, grad_voxel_smem_most(sp)) == cudaSuccess &&
              cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kGradThreads, smem) == cudaSuccess;
     }
     if (!ok) {
@@ -487,7 +495,7 @@ cudaError_t launch_grad_voxels(bool fp64, const ShapeParams &sp, const GridParam
     }
     const auto fn = grad_voxel_fn<float>(sp, gp);
     const size_t smem = grad_voxel_smem(sp);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, grad_voxel_smem_most(sp));
     if (e != cudaSuccess) return e;
     fn<<<n_blocks, kGradThreads, smem, st>>>(sp, gp, (const float2 *)S, partials);
     return cudaGetLastError();

@@ -126,3 +126,20 @@ def test_served_gradient_matches_oracle():
     ref = oracle.gradient(s, g, 2 * (res["I"].astype(np.float64) - target.astype(np.float64)), A, width=0.5)
     assert np.linalg.norm(res["grad"] - ref) / np.linalg.norm(ref) < 1e-6
     assert abs(res["loss"][0] - ((I - target) ** 2).sum()) < 1e-6 * res["loss"][0]
+
+
+def test_concurrent_gradients_of_mixed_degrees():
+    """Shapes without harmonics and of the highest degree of one voxel-gradient
+    kernel share it on concurrent streams: every request succeeds."""
+    from paper_2202_03411_gb300.serving import Server
+    g = Geometry(24, 24, 24, 1.0, 6.0, 45.0, 32, 32)
+    rng = np.random.default_rng(3)
+    shapes = [Shape(SPHERE, r=7.0, delta=0.01, beta=0.001),
+              Shape(SPHHARM, R0=7.0, lmax=6, alm=random_alm(rng, 6), delta=0.01, beta=0.001),
+              Shape(SPHHARM, R0=7.0, lmax=2, alm=random_alm(rng, 2), delta=0.01, beta=0.001)]
+    target = np.zeros(g.n_pix, dtype=np.float32)
+    srv = Server(budget_bytes=8 << 30, slots=8, precision="tc_bf16_split")
+    tickets = [srv.submit(g, shapes[i % 3], target)[0] for i in range(600)]
+    status = [srv.wait(t)[0] for t in tickets]
+    srv.close()
+    assert status == [0] * len(status)
