@@ -180,6 +180,7 @@ void scatman_destroy(scatman_handle *h) {
     cudaFree(h->d_H);
     cudaFree(h->d_uq_qz);
     cudaFree(h->d_fg);
+    cudaFree(h->d_fga);
     cudaFree(h->d_uq_qrow);
     cudaFree(h->d_adj_part);
     cudaFree(h->d_gmax);
@@ -283,6 +284,16 @@ static int need_q(scatman_handle *h) {
     return rc ? rc : fill_detector_q(h);
 }
 
+// The sample grid's buffers and tables.
+static int need_field_grid(scatman_handle *h) {
+    if (h->d_fg) return SCATMAN_OK;
+    int rc = alloc_dev(h, (void **)&h->d_fg, field_grid_layout(&h->fg, h->tensor_core, h->Nxp, nullptr),
+                       "field sample grid");
+    if (rc) return rc;
+    field_grid_layout(&h->fg, h->tensor_core, h->Nxp, h->d_fg);
+    return check_cuda(h, launch_field_grid_tables(h->fg, h->stream), "field sample grid");
+}
+
 int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle **out) {
     if (!out) return SCATMAN_ERR_ARG;
     *out = nullptr;
@@ -359,6 +370,7 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
     const size_t npix = (size_t)h->n_pix;
     const bool f64 = (h->precision == SCATMAN_FP64);
     int rc;
+    h->adj_on_grid = use_field_grid_adjoint(*cfg, &h->fg);
     h->on_grid = use_field_grid(*cfg, &h->fg);
     if (!h->on_grid && (rc = alloc_dev(h, (void **)&h->d_q, npix * 3 * sizeof(double), "q buffer"))) return fail(rc);
     if ((rc = alloc_dev(h, (void **)&h->d_chi, nvox * sizeof(float), "occupancy buffer"))) return fail(rc);
@@ -376,12 +388,7 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
     if ((rc = alloc_dev(h, &h->d_A, npix * cx, "field buffer"))) return fail(rc);
     if ((rc = alloc_dev(h, &h->d_I, npix * (f64 ? 8 : 4), "intensity buffer"))) return fail(rc);
     if ((rc = alloc_dev(h, (void **)&h->d_err, kStatusBytes, "status block"))) return fail(rc);
-    if (h->on_grid) {
-        if ((rc = alloc_dev(h, (void **)&h->d_fg, field_grid_layout(&h->fg, h->tensor_core, h->Nxp, nullptr),
-                            "field sample grid")))
-            return fail(rc);
-        field_grid_layout(&h->fg, h->tensor_core, h->Nxp, h->d_fg);
-    }
+    if (h->on_grid && (rc = need_field_grid(h))) return fail(rc);
     if (h->uniform_q && !h->on_grid && (rc = alloc_dev(h, (void **)&h->d_uq_qz, npix * sizeof(float2), "q_z table")))
         return fail(rc);
     if (h->uniform_tc &&
@@ -411,9 +418,7 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
                         "q upload");
         if (rc) return fail(rc);
         if ((rc = check_cuda(h, cudaStreamSynchronize(h->stream), "q upload"))) return fail(rc);
-    } else if (h->on_grid) {
-        if ((rc = check_cuda(h, launch_field_grid_tables(h->fg, h->stream), "field sample grid"))) return fail(rc);
-    } else {
+    } else if (!h->on_grid) {
         if ((rc = fill_detector_q(h))) return fail(rc);
     }
     if (h->tensor_core) {
@@ -1056,8 +1061,7 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
     const scatman_config &c = h->cfg;
     const bool f64 = h->precision == SCATMAN_FP64;
     const size_t nvox = (size_t)c.nx * c.ny * c.nz;
-    int rc = need_q(h);
-    if (rc) return rc;
+    int rc;
     if (!h->d_S) {
         if ((rc = alloc_dev(h, &h->d_S, nvox * (f64 ? sizeof(double2) : sizeof(float2)), "adjoint field")))
             return rc;
@@ -1072,7 +1076,19 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
         if ((rc = alloc_dev(h, (void **)&h->d_part, need * sizeof(double), "gradient partials"))) return rc;
         h->part_count = need;
     }
-    if (h->tensor_core && adjoint_tc_supported(c.nx, c.ny)) {
+    if (h->adj_on_grid) {
+        if ((rc = need_field_grid(h))) return rc;
+        if (!h->d_fga) {
+            if ((rc = alloc_dev(h, (void **)&h->d_fga, field_grid_adjoint_layout(h->fg, &h->fga, nullptr),
+                                "adjoint sample grid")))
+                return rc;
+            field_grid_adjoint_layout(h->fg, &h->fga, h->d_fga);
+        }
+        rc = check_cuda(h, launch_field_grid_adjoint(h->fg, h->fga, h->d_A, dLdI_dev, h->d_S, h->stream),
+                        "adjoint field");
+        if (rc) return rc;
+    } else if (h->tensor_core && adjoint_tc_supported(c.nx, c.ny)) {
+        if ((rc = need_q(h))) return rc;
         // adjoint contraction on the tensor cores (per slice, or per Jacobi-Anger order)
         if (h->adj_orders < 0 && (rc = plan_adjoint(h))) return rc;
         const int N = h->adj_orders;
@@ -1106,6 +1122,7 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
                                       "adjoint slices from orders")))
             return rc;
     } else {
+        if ((rc = need_q(h))) return rc;
         rc = check_cuda(h, launch_adjoint_field(f64, h->d_A, dLdI_dev, h->d_q, h->n_pix, c.nx, c.ny, c.nz, c.voxel,
                                                 h->d_S, h->stream),
                         "adjoint field");

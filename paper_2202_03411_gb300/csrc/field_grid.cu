@@ -31,6 +31,7 @@
 #include <complex>
 
 #include "internal.cuh"
+#include "field_grid.cuh"
 
 namespace scm {
 
@@ -72,7 +73,6 @@ static int plan_points(double k0, double top, double along, double across, doubl
 // points of 32 columns in shared memory: 131 KB in FP32, 200 KB in FP64).
 static int fg_max_half(bool fp64) { return fp64 ? 96 : 128; }
 constexpr int kFgMaxSide = 512;          // grid side in x and y
-constexpr int kFgSlices = 16;            // slices of one x/z block
 
 bool plan_field_grid(const scatman_config &c, bool fp64, FieldGrid *f) {
     *f = FieldGrid();
@@ -145,6 +145,12 @@ bool use_field_grid(const scatman_config &c, FieldGrid *f) {
     return plan_field_grid(c, c.precision == SCATMAN_FP64, f);
 }
 
+bool use_field_grid_adjoint(const scatman_config &c, FieldGrid *f) {
+    const bool plain = c.precision == SCATMAN_FP64 || c.precision == SCATMAN_FP32;
+    if (c.q_list || !plain || (double)c.det_nx * c.det_ny < 128.0) return false;
+    return plan_field_grid(c, c.precision == SCATMAN_FP64, f);
+}
+
 static size_t up256(size_t b) { return (b + 255) / 256 * 256; }
 
 // Lays the grid's buffers out from `base` (null: sizes only); returns the bytes.
@@ -177,13 +183,6 @@ size_t field_grid_layout(FieldGrid *f, bool tensor_core, int Nxp, unsigned char 
 // Tables (once per handle)
 // ---------------------------------------------------------------------------
 
-struct alignas(16) FgDouble4 {
-    double x, y, z, w;
-};
-template <typename R> struct Fg;
-template <> struct Fg<float> { using C = float2; using V4 = float4; };
-template <> struct Fg<double> { using C = double2; using V4 = FgDouble4; };
-
 __device__ __forceinline__ double fg_angle(int a, int H) { return (2 * a + 1) * kPi / (4.0 * H); }   // N = 2H points
 
 // cos and sin of a phase held in double; FP32 tables reduce it in FP64 first.
@@ -200,19 +199,6 @@ __device__ __forceinline__ double2 fg_cs(double ph, double) {
 }
 __device__ __forceinline__ double fg_coord(int k, int n) { return (n & 1) ? (double)k : k + 0.5; }
 
-// 1 / (x^2 - x_a^2) from the squares as pairs; the pole at a point itself is
-// cut off far below the distances that arise, where the weights have long
-// become 1 at that point and 0 elsewhere.
-__device__ __forceinline__ float fg_recip(float xh, float xl, float nh, float nl) {
-    float d = (xh - nh) + (xl - nl);
-    d = fabsf(d) < 1e-12f ? 1e-12f : d;
-    return __fdividef(1.0f, d);
-}
-__device__ __forceinline__ double fg_recip(double xh, double, double nh, double) {
-    double d = xh - nh;
-    d = fabs(d) < 1e-30 ? 1e-30 : d;
-    return 1.0 / d;
-}
 template <typename R>
 __device__ __forceinline__ typename Fg<R>::V4 fg_square(double x, R third, R fourth) {
     const double q = x * x;
@@ -387,43 +373,6 @@ cudaError_t launch_field_grid_tables(const FieldGrid &f, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------------------
-// The folded sums.  A block of 256 threads computes two real products
-//   out[row][col] = sum_k T[k][row] S[k][col]
-// side by side: threads 0-127 the cosines with the even parts, 128-255 the
-// sines with the odd parts.  64 columns, 8 kRpt rows; a thread holds rows
-// bg + 8 i and columns 4 cg .. 4 cg + 3, K runs in tiles of kFgK staged in
-// shared memory.  Per K value a warp reads 5 + kRpt shared-memory wavefronts
-// for 4 kRpt FMAs per thread.
-// ---------------------------------------------------------------------------
-constexpr int kFgThreads = 256;
-constexpr int kFgK = 32;
-constexpr int kFgCols = 64;
-constexpr int kFgColStride = kFgCols + 4;      // 16-byte stores of neighbouring K values fall in different banks
-
-template <typename R, int kRpt>
-struct FgTile {
-    alignas(32) R S[2][kFgK][kFgColStride];    // even, odd parts
-    alignas(16) R T[2][kFgK][8 * kRpt];        // cosines, sines
-};
-
-template <typename R, int kRpt>
-__device__ __forceinline__ void fg_multiply(const FgTile<R, kRpt> &t, int grp, int bg, int cg, int kn, R (&acc)[kRpt][4]) {
-    using V4 = typename Fg<R>::V4;
-#pragma unroll 4
-    for (int k = 0; k < kn; ++k) {
-        const V4 s = *reinterpret_cast<const V4 *>(&t.S[grp][k][4 * cg]);
-#pragma unroll
-        for (int i = 0; i < kRpt; ++i) {
-            const R w = t.T[grp][k][bg + 8 * i];
-            acc[i][0] = fma(w, s.x, acc[i][0]);
-            acc[i][1] = fma(w, s.y, acc[i][1]);
-            acc[i][2] = fma(w, s.z, acc[i][2]);
-            acc[i][3] = fma(w, s.w, acc[i][3]);
-        }
-    }
-}
-
 // Rows per thread whose tiles of 8 kRpt waste least on n rows.
 static int fg_rows_per_thread(int n) {
     int best = 3, waste = 1 << 30;
@@ -436,10 +385,6 @@ static int fg_rows_per_thread(int n) {
     }
     return best;
 }
-
-// The two mirror voxels of half-coordinate k on a side of n.
-__device__ __forceinline__ int fg_plus(int k, int n) { return n / 2 + k; }
-__device__ __forceinline__ int fg_minus(int k, int n) { return (n - 1) / 2 - k; }
 
 // H[a][even, odd][j][x] = sum over y' of cos (q_a y') even s, -i sin (q_a y') odd s.
 // Block: 32 columns x of one slice.  Slices and columns outside the occupied
@@ -767,11 +712,6 @@ __global__ void __launch_bounds__(128) fg_pixels_out_kernel(FieldGrid f, R str_r
 // ---------------------------------------------------------------------------
 // Forward launches
 // ---------------------------------------------------------------------------
-
-template <typename K>
-static cudaError_t fg_smem(K kernel, size_t bytes) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
 
 template <typename R, int kRpt>
 static cudaError_t fg_run_y(const FieldGrid &f, const void *s, const int *bounds, cudaStream_t st) {

@@ -188,6 +188,12 @@ struct FieldGrid {
     size_t bytes = 0;
 };
 
+// Buffers of the adjoint through the grid (field_grid_adjoint.cu), one allocation.
+struct FieldGridAdjoint {
+    int chunks = 0;                 // of the per-pixel direction
+    void *B = nullptr, *G = nullptr, *T = nullptr;      // pixels gathered along it; onto the grid; x/z sums
+};
+
 }  // namespace scm
 
 struct scatman_handle {
@@ -256,6 +262,9 @@ struct scatman_handle {
     bool on_grid = false;           // the field goes through its sample grid
     scm::FieldGrid fg;
     unsigned char *d_fg = nullptr;  // its buffers
+    bool adj_on_grid = false;       // the adjoint goes through the grid
+    scm::FieldGridAdjoint fga;
+    unsigned char *d_fga = nullptr; // its buffers (from the first backward on)
     int splits = 1;
     long long device_bytes = 0;
     scm::TcMaps tmap_B;
@@ -350,6 +359,12 @@ cudaError_t launch_field_grid(const FieldGrid &f, const void *s, const int *boun
                               void *A, void *I, int sm_count, cudaStream_t st);
 cudaError_t launch_field_grid_tc(const FieldGrid &f, int Nxp, const int *bounds, const int *chunk_y, double str_re,
                                  double str_im, float2 *A, float *I, int sm_count, cudaStream_t st);
+// Whether a handle of this configuration runs its adjoint through the grid.
+bool use_field_grid_adjoint(const scatman_config &c, FieldGrid *f);
+// The adjoint field (field_grid_adjoint.cu); layout: buffer offsets from base, returns the bytes.
+size_t field_grid_adjoint_layout(const FieldGrid &f, FieldGridAdjoint *a, unsigned char *base);
+cudaError_t launch_field_grid_adjoint(const FieldGrid &f, const FieldGridAdjoint &ad, const void *A, const void *w,
+                                      void *S, cudaStream_t st);
 // Real flops one contraction launch issues for the recorded slice geometry
 // (a host copy of the first 4 nz + 2 kGeomChunks nz ints of the buffer).
 double tc_issued_flops(const int *geom_host, int nz, int Nxp, int Nyp, long long n_pix, bool split);

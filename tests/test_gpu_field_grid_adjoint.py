@@ -1,0 +1,89 @@
+"""The adjoint through the sample grid of scattering directions against the direct sums.
+
+The same pixels as an explicit list of q take the direct adjoint, so the two
+paths of one precision mode are compared on the same shape.  The upstream
+gradient is positive, so sum_p w_p I_p has no cancellation against a target;
+tolerances (relative L2 of the gradient vector): FP64 1e-9 (the plan leaves
+1e-12 of sum |w A|, a few hundred times |S|), FP32 2e-5 (field, adjoint and
+voxel sums each within a few 1e-6 of 64 bits).
+"""
+import numpy as np
+import pytest
+
+from workloads import (DETECTOR_UNIFORM_Q, ELLIPSOID, SPHERE, SPHHARM, Geometry, Shape, random_alm)
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"fp64": 1e-9, "fp32": 2e-5}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def _grad(g, s, prec, w, q_list=None):
+    import torch
+    import paper_2202_03411_gb300 as sm
+    h = sm.scatman_create(g, prec, soft=True, soft_width=0.6 * g.voxel, q_list=q_list)
+    real = torch.float64 if prec == "fp64" else torch.float32
+    I = torch.empty(sm.scatman_n_pix(h), dtype=real, device="cuda")
+    sm.scatman_voxelise(h, s)
+    sm.scatman_forward(h, I)
+    up = torch.as_tensor(w, device="cuda").to(real)
+    grad, again = sm.scatman_backward(h, up), sm.scatman_backward(h, up)
+    q = sm.scatman_get_q(h)
+    h.close()
+    assert np.array_equal(grad, again, equal_nan=True)
+    return grad, q
+
+
+# grids and detectors off every tile: odd and even sides, one row, one column,
+# one slice, more points than a thread's share, several chunks of pixels
+GEOMETRIES = [
+    Geometry(21, 19, 23, 1.0, 7.0, 50.0, 45, 37),
+    Geometry(64, 30, 17, 1.0, 6.0, 60.0, 33, 64),
+    Geometry(20, 72, 1, 0.7, 5.0, 75.0, 131, 1),
+    Geometry(35, 3, 40, 1.3, 9.0, 20.0, 1, 140),
+    Geometry(140, 24, 33, 1.0, 5.0, 55.0, 40, 600),
+    Geometry(24, 27, 30, 1.0, 5.0, 40.0, 70, 65, DETECTOR_UNIFORM_Q),
+    Geometry(22, 26, 20, 1.0, 6.0, 44.5, 631, 40, DETECTOR_UNIFORM_Q),    # just inside the sphere's rim
+    Geometry(24, 24, 24, 1.0, 5.0, 60.0, 64, 64, DETECTOR_UNIFORM_Q),     # off-sphere corners: direct
+]
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("k", range(len(GEOMETRIES)))
+def test_plain_modes(k, prec):
+    g = GEOMETRIES[k]
+    rng = np.random.default_rng(k)
+    lo = g.voxel * min(g.nx, g.ny, g.nz)
+    shapes = [Shape(ELLIPSOID, a=0.3 * g.nx * g.voxel, b=0.25 * g.ny * g.voxel + 0.4, c=0.3 * g.nz * g.voxel + 0.4,
+                    delta=0.02, beta=0.004, latitude=-88, longitude=4, rotation=3, cx=0.1 * g.nx * g.voxel,
+                    cy=-0.1 * g.ny * g.voxel)]
+    if lo > 12:
+        shapes.append(Shape(SPHHARM, R0=0.3 * lo, lmax=3, alm=random_alm(rng, 3, 0.08), delta=0.02, beta=0.003,
+                            latitude=20, longitude=70, rotation=-30))
+    for s in shapes:
+        w = 0.5 + rng.random(g.n_pix)
+        got, q = _grad(g, s, prec, w)
+        flat = Geometry(g.nx, g.ny, g.nz, g.voxel, g.wavelength, g.theta_max_deg, g.det_nx, g.det_ny)
+        if g.detector == DETECTOR_UNIFORM_Q:
+            k0 = 2 * np.pi / g.wavelength
+            w = w * ((q[:, 0] ** 2 + q[:, 1] ** 2) / k0 ** 2 <= 1.0)
+        ref, _ = _grad(flat, s, prec, w, q_list=q)
+        err = np.linalg.norm(got - ref) / np.linalg.norm(ref)
+        assert err < TOL[prec], (g, prec, s.kind, err)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_not_a_number_upstream_reaches_the_gradient(prec):
+    g = Geometry(20, 22, 18, 1.0, 5.0, 45.0, 30, 26)
+    w = np.ones(g.n_pix)
+    w[77] = np.nan
+    grad, _ = _grad(g, Shape(SPHERE, r=6.0, delta=0.02, beta=0.003), prec, w)
+    assert np.all(np.isnan(grad))
