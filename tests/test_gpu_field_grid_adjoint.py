@@ -87,3 +87,35 @@ def test_not_a_number_upstream_reaches_the_gradient(prec):
     w[77] = np.nan
     grad, _ = _grad(g, Shape(SPHERE, r=6.0, delta=0.02, beta=0.003), prec, w)
     assert np.all(np.isnan(grad))
+
+
+@pytest.mark.parametrize("shape,peak", [
+    (Shape(SPHERE, r=30.0, delta=0.01, beta=0.001), 0.15),
+    (Shape(ELLIPSOID, a=14.0, b=30.0, c=33.0, delta=0.01, beta=0.001, latitude=20, longitude=50), 0.3),
+    (Shape(ELLIPSOID, a=3.0, b=30.0, c=33.0, delta=0.01, beta=0.001, latitude=20, longitude=50), 1.0),
+])
+def test_fit_handles_keep_the_peak_direct(shape, peak):
+    """With soft occupancy the pixels around the forward direction carry the direct
+    sums' values (up to the order of at most four partial sums, 4 x 2^-24 in the
+    field), the others the grid's."""
+    import torch
+    import paper_2202_03411_gb300 as sm
+    g = Geometry(96, 96, 80, 1.0, 10.0, 45.0, 201, 230)
+    h = sm.scatman_create(g, "fp32")
+    q = sm.scatman_get_q(h)
+    h.close()
+    out = []
+    for ql in (None, q):
+        h = sm.scatman_create(g, "tc_bf16_split", soft=True, soft_width=0.5, q_list=ql)
+        I = torch.empty(g.n_pix, device="cuda")
+        sm.scatman_voxelise(h, shape)
+        sm.scatman_forward(h, I)
+        sm.scatman_sync(h)
+        out.append(I.cpu().double().numpy().reshape(g.det_ny, g.det_nx))
+        h.close()
+    x = np.abs((2 * np.arange(g.det_nx) + 1 - g.det_nx) / g.det_nx)
+    y = np.abs((2 * np.arange(g.det_ny) + 1 - g.det_ny) / g.det_ny)
+    at = np.ix_(y <= peak, x <= peak)
+    d = np.linalg.norm(out[0][at] - out[1][at]) / np.linalg.norm(out[1][at])
+    assert d < 5e-7, d
+    assert np.linalg.norm(out[0] - out[1]) / np.linalg.norm(out[1]) < 1e-4
