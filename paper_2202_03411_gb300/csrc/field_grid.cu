@@ -145,10 +145,15 @@ bool use_field_grid(const scatman_config &c, FieldGrid *f) {
     return plan_field_grid(c, c.precision == SCATMAN_FP64, f);
 }
 
+// Whether the adjoint runs through the grid.  In the tensor-core modes it pays
+// once three products over the grid's directions and the gather are less work
+// than one product over the pixels.
 bool use_field_grid_adjoint(const scatman_config &c, FieldGrid *f) {
-    const bool plain = c.precision == SCATMAN_FP64 || c.precision == SCATMAN_FP32;
-    if (c.q_list || !plain || (double)c.det_nx * c.det_ny < 128.0) return false;
-    return plan_field_grid(c, c.precision == SCATMAN_FP64, f);
+    const double pixels = (double)c.det_nx * c.det_ny;
+    if (c.q_list || pixels < 128.0) return false;
+    const bool tc = c.precision != SCATMAN_FP64 && c.precision != SCATMAN_FP32 && adjoint_tc_supported(c.nx, c.ny);
+    if (!plan_field_grid(c, c.precision == SCATMAN_FP64, f)) return false;
+    return !tc || 12.0 * f->Hs * f->Ht + 8192.0 < pixels;
 }
 
 static size_t up256(size_t b) { return (b + 255) / 256 * 256; }

@@ -89,6 +89,25 @@ def test_not_a_number_upstream_reaches_the_gradient(prec):
     assert np.all(np.isnan(grad))
 
 
+@pytest.mark.parametrize("prec", ["tc_f16_split", "tc_bf16_split", "tc_f16"])
+@pytest.mark.parametrize("g", [
+    Geometry(40, 36, 44, 1.0, 7.0, 45.0, 150, 141),
+    Geometry(96, 128, 3, 1.0, 9.0, 40.0, 256, 257),           # three slices: one product sum per slice
+    Geometry(140, 40, 36, 1.0, 8.0, 45.0, 160, 130),          # wider than the tensor-core adjoint takes
+])
+def test_tensor_core_modes(g, prec):
+    """The same slices on both sides.  5e-5: the direct tensor-core adjoint rounds
+    its operands to FP16 (2^-12 each, independent over 20000 pixels and more), the
+    fields of the two sides differ by a few 1e-6; the grid's split operands add less."""
+    s = Shape(ELLIPSOID, a=0.3 * g.nx, b=0.3 * g.ny, c=0.3 * g.nz + 0.3, delta=0.02, beta=0.004, latitude=-80,
+              longitude=4, rotation=3, cy=-0.05 * g.ny)
+    w = 0.5 + np.random.default_rng(g.nx).random(g.n_pix)
+    got, q = _grad(g, s, prec, w)
+    ref, _ = _grad(g, s, prec, w, q_list=q)
+    err = np.linalg.norm(got - ref) / np.linalg.norm(ref)
+    assert err < 5e-5, (g, prec, err)
+
+
 @pytest.mark.parametrize("shape,peak", [
     (Shape(SPHERE, r=30.0, delta=0.01, beta=0.001), 0.15),
     (Shape(ELLIPSOID, a=14.0, b=30.0, c=33.0, delta=0.01, beta=0.001, latitude=20, longitude=50), 0.3),
