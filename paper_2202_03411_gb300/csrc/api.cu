@@ -502,6 +502,60 @@ static void set_radius_band(const scatman_shape *s, ShapeParams *sp, bool fp64) 
     if (!(sp->band_hi > 0.f)) sp->band_lo = sp->band_hi = 0.f;
 }
 
+// Where the FP32 occupancy test of a binary shape decides.  Coordinates up to
+// `far` lose 1e-7 of it each, a few times over in the rotation.  Harmonics: with u =
+// 2^-24 a term of degree l is off by at most (6 l + 10) u of its bound
+// |a_lm| sqrt((2l+1)/(4 pi)), the direction by 6 u (times the slope, below l + 1 times
+// the same bounds), the distance by 6 u of its size; sh_margin is four times the sum.
+// The margins of sphere and ellipsoid (1e-4 of r^2) and of the maps (4e-3 voxel)
+// cover their FP32 error for the sizes that fp32_first asks for; the FP64 mode takes
+// the FP32 test first only there.
+static void set_fp32_test(const scatman_config &c, ShapeParams *sp) {
+    const double far = 0.5 * std::max(c.nx, std::max(c.ny, c.nz)) * c.voxel +
+                       std::fmax(std::fabs(sp->cx), std::fmax(std::fabs(sp->cy), std::fabs(sp->cz)));
+    const bool scale = c.voxel > 1e-9 && c.voxel < 1e9;
+    if (sp->kind == SCATMAN_SPHERE) {
+        sp->fp32_first = scale && sp->r > 0.03 * far;
+    } else if (sp->kind == SCATMAN_ELLIPSOID) {
+        sp->fp32_first = scale && std::fmin(sp->a, std::fmin(sp->b, sp->c)) > 0.03 * far;
+    } else if (sp->kind == SCATMAN_SPHHARM) {
+        double b = 0.0;
+        for (int l = 1; l <= sp->lmax; ++l)
+            for (int m = -l; m <= l; ++m)
+                b += (12.0 * l + 16.0) * std::fabs(sp->alm[l * l + l + m]) * std::sqrt((2.0 * l + 1.0) / (4.0 * kPi));
+        const double err = 5.97e-8 * (sp->R0 * (b + 6.0) + 12.0 * far);
+        sp->sh_margin = (float)std::fmin(4.0 * err, 1e30);
+        sp->fp32_first = scale && far < 512.0 * c.voxel && err < 0.02 * c.voxel;
+    } else {
+        sp->fp32_first = scale && far < 512.0 * c.voxel &&
+                         (sp->kind != SCATMAN_RADIALMAP || sp->band_hi < 256.0 * c.voxel);
+    }
+}
+
+// The radius table of a binary harmonics shape.  The radius changes by at most
+// R0 sum_l |a_l| sqrt(l(l+1)(2l+1)/(4 pi)) per radian (Cauchy-Schwarz with
+// sum_m |grad Y_lm|^2 = l(l+1)(2l+1)/(4 pi)), and no direction of a cell is
+// farther than sqrt(2)/n from its centre.  n balances the table's 6 n^2 radii
+// against the shell of voxels it leaves undecided, 4 pi R0^2 x 2 slack.
+static void set_radius_table(const scatman_config &c, ShapeParams *sp) {
+    sp->rtab_n = 0;
+    if (sp->kind != SCATMAN_SPHHARM || sp->soft || sp->lmax < 2 || !(sp->band_hi > 0.f)) return;
+    double S = 0.0;
+    for (int l = 1; l <= sp->lmax; ++l) {
+        double n2 = 0.0;
+        for (int m = -l; m <= l; ++m) n2 += sp->alm[l * l + l + m] * sp->alm[l * l + l + m];
+        S += std::sqrt(n2 * l * (l + 1.0) * (2.0 * l + 1.0) / (4.0 * kPi));
+    }
+    S *= sp->R0;
+    const double v = c.voxel, best = std::cbrt(3.0 * sp->R0 * sp->R0 * S / (v * v * v));
+    const int n = std::min(kRtabMax, std::max(8, (int)(std::fmin(best, 1e6) / 8.0 + 0.5) * 8));
+    // the cell's extent, an FP32 direction's rounding, and the FP32 radius' and distance's margins
+    const double slack = S * (1.41422 / n + 1e-5) + sp->sh_margin + 1e-3 * v + 1e-5 * sp->band_hi;
+    if (!(slack < 0.3 * ((double)sp->band_hi - sp->band_lo))) return;       // settles too little beyond the band
+    sp->rtab_n = n;
+    sp->rtab_slack = (float)slack;
+}
+
 // Copies a map shape's arrays to the device (grown buffers owned by the handle)
 // and fills the map fields of the shape parameters.
 static int upload_maps(scatman_handle *h, const scatman_shape *s, ShapeParams *sp) {
@@ -665,6 +719,8 @@ int scatman_voxelise(scatman_handle *h, const scatman_shape *s) {
     int rc = upload_maps(h, s, &sp);
     if (rc) return rc;
     set_radius_band(s, &sp, h->precision == SCATMAN_FP64);
+    set_fp32_test(c, &sp);
+    if (h->precision != SCATMAN_FP64 || sp.fp32_first) set_radius_table(c, &sp);
 
     const GridParams gp = make_grid(c.nx, c.ny, c.nz, c.voxel, h->k0, s->delta, s->beta);
     SliceOut so;
@@ -678,6 +734,9 @@ int scatman_voxelise(scatman_handle *h, const scatman_shape *s) {
     so.chi = h->d_chi;
     so.bounds = h->d_bounds;
     so.chunk_y = h->tensor_core ? geom_chunk_y(h->d_bounds, c.nz) : nullptr;
+    so.table = geom_table(h->d_bounds, c.nz);
+    so.stage = geom_stage(h->d_bounds, c.nz);
+    so.rtab = geom_rtab(h->d_bounds, c.nz);
     double strength = std::fmax(std::fabs(s->delta), std::fabs(s->beta));
     if (sp.varn) strength = std::fmax(strength, h->map_index_max);
     h->scan_fp64 = c.scan_fp64 || (h->k0 * c.voxel * c.nz * strength > 5.0);
@@ -1361,6 +1420,7 @@ extern "C" int scatman_forward_noalloc(const scatman_config *cfg, const scatman_
         for (int k = 0; k < (s->lmax + 1) * (s->lmax + 1); ++k) sp.alm[k] = s->alm[k];
     finish_shape_params(&sp);
     set_radius_band(s, &sp, false);   // CUDA-core FP32 path
+    set_fp32_test(c, &sp);
     const GridParams gp = make_grid(c.nx, c.ny, c.nz, c.voxel, k0, s->delta, s->beta);
     SliceOut so;
     so.layout = kLayoutC32;
@@ -1369,6 +1429,9 @@ extern "C" int scatman_forward_noalloc(const scatman_config *cfg, const scatman_
     so.chi = d_chi;
     so.bounds = nullptr;
     so.chunk_y = nullptr;
+    so.table = nullptr;
+    so.stage = nullptr;
+    so.rtab = nullptr;
     const double strength = std::fmax(std::fabs(s->delta), std::fabs(s->beta));
     const bool scan_fp64 = c.scan_fp64 || (k0 * c.voxel * c.nz * strength > 5.0);
     e = launch_voxelise(sp, gp, so, scan_fp64, false, st);

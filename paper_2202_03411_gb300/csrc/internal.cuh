@@ -97,6 +97,17 @@ struct ShapeParams {
     // |p| below band_lo is inside (soft: chi = 1), above band_hi outside
     // (chi = 0) (band_hi = 0: no band)
     float band_lo, band_hi;
+    // FP64 mode, binary shapes: the FP32 test's margins hold for these sizes, so
+    // it may settle voxels before the FP64 one
+    int fp32_first;
+    // binary harmonics: the voxeliser tabulates the radius at the centres of
+    // rtab_n^2 cells on each face of a cube of directions; anywhere in a cell it
+    // is within rtab_slack of that (rtab_n = 0: no table)
+    int rtab_n;
+    float rtab_slack;
+    // binary harmonics: the FP32 test decides where the radius and the distance
+    // differ by more than this (four times a bound on their FP32 error)
+    float sh_margin;
 };
 
 // Soft occupancy cut of the FP32 modes: chi = 1 / (1 + e^{-t}) with
@@ -150,11 +161,22 @@ struct TcMaps {
 //   [4 nz, 68 nz)        occupied y range of every 8-column chunk of every slice,
 //                        [y_lo | y_hi] x [nz][kGeomChunks] (tensor-core grids, nx <= 256)
 //   then                 the tensor-core kernel's work-unit list (uint2, kMaxUnitsPerSlice nz + 1)
+//   then                 T of 0 .. nz full voxels (16 bytes each), for binary shapes
+//   then                 harmonics shapes: their coefficients as the voxeliser stages
+//                        them (kShStageInts), and the radius table (floats)
+constexpr int kRtabMax = 64;        // cells along a cube face's edge
+constexpr int kShStageInts = 1536;
 constexpr int kGeomChunks = 32;
 constexpr int kMaxUnitsPerSlice = 4;
-inline size_t slice_geom_ints(int nz) {
-    return 4 * (size_t)nz + 2 * (size_t)kGeomChunks * nz + 2 * ((size_t)kMaxUnitsPerSlice * nz + 1);
+inline size_t geom_table_at(int nz) {
+    return (4 * (size_t)nz + 2 * (size_t)kGeomChunks * nz + 2 * ((size_t)kMaxUnitsPerSlice * nz + 1) + 3) / 4 * 4;
 }
+inline size_t geom_stage_at(int nz) { return geom_table_at(nz) + 4 * ((size_t)nz + 1); }
+inline size_t geom_rtab_at(int nz) { return geom_stage_at(nz) + kShStageInts; }
+inline void *geom_stage(int *g, int nz) { return g + geom_stage_at(nz); }
+inline size_t slice_geom_ints(int nz) { return geom_rtab_at(nz) + 6 * (size_t)kRtabMax * kRtabMax; }
+inline void *geom_table(int *g, int nz) { return g + geom_table_at(nz); }
+inline float *geom_rtab(int *g, int nz) { return reinterpret_cast<float *>(g + geom_rtab_at(nz)); }
 inline int *geom_chunk_y(int *g, int nz) { return g + 4 * (size_t)nz; }
 inline uint2 *geom_units(int *g, int nz) {
     return reinterpret_cast<uint2 *>(g + 4 * (size_t)nz + 2 * (size_t)kGeomChunks * nz);
@@ -167,6 +189,9 @@ struct SliceOut {
     float *chi;                     // occupancy [z][x][y]
     int *bounds;                    // per slice [x_lo | x_hi | y_lo | y_hi] of chi != 0 (nz each), or null
     int *chunk_y;                   // per slice and 8-column chunk [y_lo | y_hi] (see above), or null
+    void *table;                    // T of 0 .. nz full voxels (with bounds)
+    void *stage;                    // staged coefficients of harmonics shapes (with bounds)
+    float *rtab;                    // their radius table
 };
 
 // A rectangle of the detector's pixels (w = 0: all of them).

@@ -106,6 +106,74 @@ __device__ __forceinline__ T sh_radius_unclipped(const ShapeParams &sp, T px, T 
     return tb.R0 * ((T)1 + sum);
 }
 
+// FP32 radius for the binary voxeliser.  With (x, y, z) = p / |p| the harmonics
+// of order m are P_l^m(z) times the real and imaginary part of (x + i y)^m (the
+// sine's powers ride along, so neither the azimuth nor its distance from the axis
+// is formed); per order the terms a P and b P are summed first, five operations a
+// term.  The loops are rolled over coefficients in shared memory, one 16-byte
+// load a term: order m starts at m (L + 1) - m (m - 1) / 2 with
+// (a_lm, -a_lm b_lm, alm of +m, alm of -m) for l = m .. L.
+constexpr int kShTerms = (SCATMAN_MAX_LMAX + 1) * (SCATMAN_MAX_LMAX + 2) / 2;
+struct alignas(16) ShTerms {
+    float4 t[kShTerms];
+    float d[SCATMAN_MAX_LMAX + 4];
+};
+
+// By all threads of a block.
+__device__ __forceinline__ void sh_stage_terms(const ShapeParams &sp, ShTerms &tab) {
+    const int L = sp.lmax;
+    for (int k = threadIdx.x; k < (L + 1) * (L + 1); k += blockDim.x) {
+        const int m = k / (L + 1), l = k % (L + 1), i = l * (l + 1) / 2 + m;
+        if (l < m) continue;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (l == m + 1) v.x = sp.sh_ef[m];
+        if (l > m + 1) {
+            v.x = sp.sh_af[i];
+            v.y = (float)(-sp.sh_a[i] * sp.sh_b[i]);
+        }
+        if (l > 0) {                                     // a_00 is not a coefficient
+            v.z = sp.almf[l * l + l + m];
+            if (m > 0) v.w = sp.almf[l * l + l - m];
+        }
+        tab.t[m * (L + 1) - m * (m - 1) / 2 + l - m] = v;
+    }
+    for (int m = threadIdx.x; m <= L; m += blockDim.x) tab.d[m] = sp.sh_df[m];
+}
+
+// Radius along body direction p (not normalised) with 1 / |p| = inv, clipped.
+__device__ __forceinline__ float sh_radius_f(const ShapeParams &sp, const ShTerms &tab, float px, float py, float pz,
+                                             float inv) {
+    const float x = px * inv, y = py * inv, z = pz * inv;
+    const int L = sp.lmax;
+    const float4 *t = tab.t;
+    // (x + i y)^m times the diagonal factors, sqrt(2) and 1 / sqrt(4 pi)
+    float er = 0.28209479177387814347f, ei = 0.f, sum = 0.f;
+#pragma unroll 1
+    for (int m = 0; m <= L; ++m) {
+        if (m > 0) {
+            const float d = m == 1 ? 1.41421356237309504880f * tab.d[1] : tab.d[m];
+            const float xr = er * x - ei * y;
+            ei = d * (er * y + ei * x);
+            er = d * xr;
+        }
+        float4 v = *t++;
+        float p2 = 0.f, p1 = 1.f, a = v.z, b = v.w;
+#pragma unroll 4
+        for (int l = m + 1; l <= L; ++l) {
+            v = *t++;
+            const float p = fmaf(v.x * z, p1, v.y * p2);
+            p2 = p1;
+            p1 = p;
+            a = fmaf(v.z, p, a);
+            b = fmaf(v.w, p, b);
+        }
+        sum = fmaf(a, er, fmaf(b, ei, sum));
+    }
+    float r = sp.R0f * (1.f + sum);
+    r = r < sp.rminf ? sp.rminf : r;
+    return r > sp.rmaxf ? sp.rmaxf : r;
+}
+
 // The same radius clipped to [rmin, rmax].
 template <typename T>
 __device__ __forceinline__ T sh_radius(const ShapeParams &sp, T px, T py, T pz, T rr) {
@@ -235,13 +303,14 @@ __device__ __forceinline__ void sh_stage_tables(const ShapeParams &sp, double *t
 }
 
 // The FP64 binary decision of one harmonics voxel by a whole warp (call with
-// all 32 lanes; every lane gets the result): the body coordinates and |p| as in
+// all 32 lanes; every lane gets the result): the body coordinates and |p|^2 as in
 // occupancy_binary_fp64, then lane m (m <= lmax) sums the terms of orders +m
-// and -m over l = m..lmax with the recurrences of real_sh_all, and the warp
-// adds the lanes' sums.  GB300 runs FP64 at a small fraction of its FP32 rate,
-// so the warp's instruction count, not its lane count, sets the cost of the
-// near-surface decisions: splitting the orders over lanes cuts it about three-fold.
-// Only the summation order differs from occupancy_binary_fp64 (both decide in
+// and -m over l = m..lmax, and the warp adds the lanes' sums.  GB300 runs FP64 at
+// a small fraction of its FP32 rate, so the warp's chain of dependent operations
+// sets the cost of the near-surface decisions: the orders are split over the
+// lanes, and with the sine's powers kept in (x + i y)^m (see sh_radius_f) one
+// reciprocal square root replaces a root and four divisions.
+// Only the operations' order differs from occupancy_binary_fp64 (both decide in
 // FP64; the oracle evaluates the radius by yet another route).
 static __device__ __noinline__ double sh_binary_fp64_warp(const ShapeParams &sp, const GridParams &gp, int ix, int iy,
                                                          int iz, const double *tab) {
@@ -249,50 +318,34 @@ static __device__ __noinline__ double sh_binary_fp64_warp(const ShapeParams &sp,
     double px, py, pz;
     body_coords(sp, gp, ix, iy, iz, px, py, pz);
     const double p2 = __dadd_rn(__dadd_rn(__dmul_rn(px, px), __dmul_rn(py, py)), __dmul_rn(pz, pz));
-    const double rr = sqrt(p2);
-    double ct = 1.0, st = 0.0, cphi = 1.0, sphi = 0.0;
-    if (rr > 0.0) {
-        ct = pz / rr;
-        const double rho = sqrt(px * px + py * py);
-        st = rho / rr;
-        if (rho > 0.0) {
-            cphi = px / rho;
-            sphi = py / rho;
-        }
+    double inv = 0.0, z = 1.0;                            // p = 0 takes the body's +z direction
+    if (p2 > 0.0) {
+        inv = rsqrt(p2);
+        z = pz * inv;
     }
+    // (the root rounds to nearest: a voxel exactly on a clipped radius is inside)
+    const double rr = sqrt(p2), x = px * inv, y = py * inv;
     const int L = sp.lmax, m = threadIdx.x & 31;
     double part = 0.0;
     if (m <= L) {
-        double pmm = 0.28209479177387814347, cm = 1.0, sm = 0.0;
+        double er = m == 0 ? 0.28209479177387814347 : 0.28209479177387814347 * 1.41421356237309504880, ei = 0.0;
         for (int k = 1; k <= m; ++k) {
-            pmm = td[k] * st * pmm;
-            const double c2 = cm * cphi - sm * sphi, s2 = sm * cphi + cm * sphi;
-            cm = c2;
-            sm = s2;
+            const double xr = er * x - ei * y, d = td[k];
+            ei = d * (er * y + ei * x);
+            er = d * xr;
         }
-        const double kSqrt2 = 1.41421356237309504880;
-        const double wc = m == 0 ? 1.0 : kSqrt2 * cm, ws = kSqrt2 * sm;
-        double q2 = 0.0, q1 = pmm;
-        for (int l = m; l <= L; ++l) {
-            double p;
-            if (l == m) {
-                p = pmm;
-            } else if (l == m + 1) {
-                p = te[m] * ct * pmm;
-            } else {
-                const int i = l * (l + 1) / 2 + m;
-                p = ta[i] * (ct * q1 - tb[i] * q2);
-            }
-            if (l > m) {
-                q2 = q1;
-                q1 = p;
-            }
-            if (l == 0) continue;                     // a_00 is not a coefficient
-            if (m == 0)
-                part += talm[l * l + l] * p;
-            else
-                part += talm[l * l + l + m] * (p * wc) + talm[l * l + l - m] * (p * ws);
+        double q2 = 0.0, q1 = 1.0;
+        double a = m == 0 ? 0.0 : talm[m * m + 2 * m], b = m == 0 ? 0.0 : talm[m * m];     // (a_00 is not a coefficient)
+        for (int l = m + 1; l <= L; ++l) {
+            const int i = l * (l + 1) / 2 + m;
+            const double c = l == m + 1 ? te[m] : ta[i];
+            const double p = c * (z * q1 - (l == m + 1 ? 0.0 : tb[i]) * q2);
+            q2 = q1;
+            q1 = p;
+            a += talm[l * l + l + m] * p;
+            if (m > 0) b += talm[l * l + l - m] * p;
         }
+        part = a * er + b * ei;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
@@ -333,18 +386,54 @@ __device__ __forceinline__ int vmap_cell(const ShapeParams &sp, const GridParams
     return vmap_cell_fp64(sp, px, py, pz);
 }
 
-// Occupancy of one voxel.  Binary decisions are the FP64 ones above; the
-// FP32 modes first evaluate the same quantity in FP32 and only fall back to
-// FP64 when the margin is within a bound well above the FP32 error
-// (1e-4 relative for sphere and ellipsoid, 4e-3 voxel for harmonics), so the
-// decision always equals the FP64 one.  Soft occupancy is the logistic of
-// the signed distance to the surface along the ray from the centre; the FP32
-// modes set it to zero where the logistic is below 2^-24 (soft_zero()), the
-// FP64 mode keeps the exact logistic everywhere.
+// FP32 form of the binary decision (1 or 0), or -1 where the margin is within a
+// bound well above the FP32 error (1e-4 relative for sphere and ellipsoid,
+// sp.sh_margin for harmonics, 4e-3 voxel for radii maps): the caller then takes the FP64 decision,
+// so the result always equals it.
 // kMaps: compiled for the map kinds (radii and volume maps); the parametric
 // kinds' instantiation carries none of their code.
-// kDefer (FP32 modes): a binary voxel the FP32 test cannot settle returns -1
-// instead of taking the FP64 path here, so the caller can batch those voxels.
+template <bool kMaps>
+__device__ __forceinline__ float occupancy_binary_f(const ShapeParams &sp, const GridParams &gp, const ShTerms &tab,
+                                                    int ix, int iy, int iz) {
+    if (kMaps && sp.kind == SCATMAN_VOLUMEMAP) {
+        const int cell = vmap_cell<false>(sp, gp, ix, iy, iz);
+        return (cell >= 0 && sp.vmap[cell] != 0) ? 1.f : 0.f;
+    }
+    const float vox = gp.voxf;
+    const float dx = ((float)ix - 0.5f * (float)(gp.nx - 1)) * vox - sp.cxf;
+    const float dy = ((float)iy - 0.5f * (float)(gp.ny - 1)) * vox - sp.cyf;
+    const float dz = ((float)iz - 0.5f * (float)(gp.nz - 1)) * vox - sp.czf;
+    float m, margin;
+    if (!kMaps && sp.kind == SCATMAN_SPHERE) {
+        const float r2 = sp.r2f;
+        m = r2 - (dx * dx + dy * dy + dz * dz);
+        margin = 1e-4f * r2 + 1e-6f;
+    } else {
+        const float px = sp.Rf[0] * dx + sp.Rf[3] * dy + sp.Rf[6] * dz;
+        const float py = sp.Rf[1] * dx + sp.Rf[4] * dy + sp.Rf[7] * dz;
+        const float pz = sp.Rf[2] * dx + sp.Rf[5] * dy + sp.Rf[8] * dz;
+        if (!kMaps && sp.kind == SCATMAN_ELLIPSOID) {
+            const float u = px * sp.inv_af, v = py * sp.inv_bf, w = pz * sp.inv_cf;
+            m = 1.f - (u * u + v * v + w * w);
+            margin = 1e-4f;
+        } else {
+            const float rr2 = px * px + py * py + pz * pz, inv = rr2 > 0.f ? rsqrtf(rr2) : 0.f;
+            const float rr = kMaps ? sqrtf(rr2) : rr2 * inv;
+            const float rs = kMaps ? rmap_radius_f(sp, px, py, pz) : sh_radius_f(sp, tab, px, py, pz, inv);
+            m = rs - rr;
+            margin = kMaps ? 4e-3f * vox : sp.sh_margin;
+            // radii map: angles to ~2e-6 rad (worse near the centre) times the
+            // map's steepest slope, plus rounding
+            if (kMaps) margin += 1e-6f * (fabsf(rs) + rr) + sp.rm_slope * (2e-6f + 2e-5f / fmaxf(rr, vox));
+        }
+    }
+    return fabsf(m) > margin ? (m > 0.f ? 1.f : 0.f) : -1.f;
+}
+
+// Soft occupancy of one voxel, the logistic of the signed distance to the
+// surface along the ray from the centre; the FP32 modes set it to zero where the
+// logistic is below 2^-24 (soft_zero()), the FP64 mode keeps the exact logistic
+// everywhere.  A volume map has no surface radius: binary there.
 // Soft occupancy cut of the FP32 modes (kSoftCutT): without the cut every voxel of the grid has chi > 0 (the logistic never
 // vanishes) and the contraction cannot skip the empty part of a slice.  The
 // dropped voxels change the field by at most |n^2 - 1| times their summed
@@ -353,51 +442,11 @@ __device__ __forceinline__ int vmap_cell(const ShapeParams &sp, const GridParams
 // it stays the derivative of the function the forward computes.
 __device__ __forceinline__ bool soft_zero(float t) { return t < -kSoftCutT; }
 
-template <bool kFp64, bool kMaps = false, bool kDefer = false,
-          typename OccT = typename std::conditional<kFp64, double, float>::type>
+template <bool kFp64, bool kMaps = false, typename OccT = typename std::conditional<kFp64, double, float>::type>
 __device__ __forceinline__ OccT occupancy(const ShapeParams &sp, const GridParams &gp, int ix, int iy, int iz) {
     if (kMaps && sp.kind == SCATMAN_VOLUMEMAP) {
-        // binary in both modes: a volume map has no surface radius
         const int cell = vmap_cell<kFp64>(sp, gp, ix, iy, iz);
         return (cell >= 0 && sp.vmap[cell] != 0) ? (OccT)1 : (OccT)0;
-    }
-    if (!sp.soft) {
-        if (!kFp64) {
-            const float vox = gp.voxf;
-            const float dx = ((float)ix - 0.5f * (float)(gp.nx - 1)) * vox - sp.cxf;
-            const float dy = ((float)iy - 0.5f * (float)(gp.ny - 1)) * vox - sp.cyf;
-            const float dz = ((float)iz - 0.5f * (float)(gp.nz - 1)) * vox - sp.czf;
-            if (sp.kind == SCATMAN_SPHERE) {
-                const float r2 = sp.r2f;
-                const float m = r2 - (dx * dx + dy * dy + dz * dz);
-                if (fabsf(m) > 1e-4f * r2 + 1e-6f) return m > 0.f ? (OccT)1 : (OccT)0;
-            } else {
-                const float px = sp.Rf[0] * dx + sp.Rf[3] * dy + sp.Rf[6] * dz;
-                const float py = sp.Rf[1] * dx + sp.Rf[4] * dy + sp.Rf[7] * dz;
-                const float pz = sp.Rf[2] * dx + sp.Rf[5] * dy + sp.Rf[8] * dz;
-                if (sp.kind == SCATMAN_ELLIPSOID) {
-                    const float u = px * sp.inv_af, v = py * sp.inv_bf, w = pz * sp.inv_cf;
-                    const float m = 1.f - (u * u + v * v + w * w);
-                    if (fabsf(m) > 1e-4f) return m > 0.f ? (OccT)1 : (OccT)0;
-                } else if (kMaps && sp.kind == SCATMAN_RADIALMAP) {
-                    const float rr = sqrtf(px * px + py * py + pz * pz);
-                    const float rs = rmap_radius_f(sp, px, py, pz);
-                    const float m = rs - rr;
-                    // FP32 error bound: angles to ~2e-6 rad (worse near the
-                    // centre) times the map's steepest slope, plus rounding
-                    const float margin = 4e-3f * vox + 1e-6f * (fabsf(rs) + rr) +
-                                         sp.rm_slope * (2e-6f + 2e-5f / fmaxf(rr, vox));
-                    if (fabsf(m) > margin) return m > 0.f ? (OccT)1 : (OccT)0;
-                } else {
-                    const float rr = sqrtf(px * px + py * py + pz * pz);
-                    const float rs = sh_radius<float>(sp, px, py, pz, rr);
-                    const float m = rs - rr;
-                    if (fabsf(m) > 4e-3f * vox) return m > 0.f ? (OccT)1 : (OccT)0;
-                }
-            }
-        }
-        if (kDefer && !kFp64) return (OccT)-1;
-        return (OccT)occupancy_binary_fp64(sp, gp, ix, iy, iz);
     }
     if constexpr (kFp64) {
         double px, py, pz;

@@ -48,14 +48,13 @@ constexpr int kVoxThreads = 256;
 constexpr int kMaxRun = 16;         // z values per lane: nz <= 512 (256 in the FP64 mode)
 constexpr int kVoxQueue = 512;      // binary voxels per CTA whose FP64 decision is batched
 
-// s_j = chi_j T_j with T_j = exp(i k0 dz (n-1) C_j) = e^{-k0 dz beta C} e^{-i k0 dz delta C}.
+// s_j = chi_j T_j with T_j = exp(i k0 dz (n-1) C_j) = e^{-k0 dz beta C} e^{-i k0 dz delta C},
+// for soft occupancy and for maps with an index per cell (binary shapes of one
+// index: voxelise_binary_kernel below).
 // A warp takes one (x, y) line at a time; its lanes take 32 consecutive z per
-// step, so neighbouring lanes hold neighbouring voxels (and binary shapes can
-// skip the surface radius where the whole step is clearly inside or outside).
-// Pass 1 renders chi into shared memory for all of the CTA's lines; in the
-// FP32 modes the few binary voxels too close to the surface for the FP32 test
-// are queued and decided in FP64 afterwards by whole warps (a lone lane in
-// the FP64 path would hold its warp for the full FP64 radius).  Pass 2 forms
+// step, so neighbouring lanes hold neighbouring voxels (and shapes with a radius
+// band skip the surface radius where the whole step is clearly inside or outside).
+// Pass 1 renders chi into shared memory for all of the CTA's lines.  Pass 2 forms
 // the exclusive prefix C_j with a warp scan per step plus the running total
 // of earlier steps, then T_j and s_j.  Tiles are [line][z] with a padded row,
 // so both the z-walk and the line-fastest output loop are free of bank
@@ -80,10 +79,6 @@ __global__ void __launch_bounds__(kVoxThreads, 3) voxelise_scan_kernel(ShapePara
     using Re = typename std::conditional<kFp64, double, float>::type;
     Cx *s_tile = reinterpret_cast<Cx *>(smem);                                // [32][zs]
     float *chi_tile = reinterpret_cast<float *>(smem + sizeof(Cx) * zs * kLinesPerCta);
-    int *queue = reinterpret_cast<int *>(chi_tile + (size_t)zs * kLinesPerCta);   // (line << 16) | z
-    __shared__ int s_qn;
-    if (threadIdx.x == 0) s_qn = 0;
-    __syncthreads();
 
     const int ix = blockIdx.x;
     const int y0 = blockIdx.y * kLinesPerCta;
@@ -131,15 +126,7 @@ __global__ void __launch_bounds__(kVoxThreads, 3) voxelise_scan_kernel(ShapePara
                         const int cell = vmap_cell<kFp64>(sp, gp, ix, iy, iz);
                         c = (cell >= 0 && sp.vmap[cell] != 0) ? (Re)1 : (Re)0;
                     } else {
-                        c = (Re)occupancy<kFp64, kMaps, true>(sp, gp, ix, iy, iz);
-                        if (!kFp64 && c < (Re)0) {
-                            // too close to the surface for FP32: queue it (inline when full)
-                            const int slot = atomicAdd(&s_qn, 1);
-                            if (slot < kVoxQueue)
-                                queue[slot] = (yl << 16) | iz;
-                            else
-                                c = (Re)occupancy_binary_fp64(sp, gp, ix, iy, iz);
-                        }
+                        c = (Re)occupancy<kFp64, kMaps>(sp, gp, ix, iy, iz);
                     }
                 }
                 if (kFp64) srow[iz].x = c;                                // exact copy until pass 2
@@ -148,34 +135,6 @@ __global__ void __launch_bounds__(kVoxThreads, 3) voxelise_scan_kernel(ShapePara
         }
     }
     __syncthreads();
-    if (!kFp64) {
-        // the queued voxels' FP64 decisions: harmonics one voxel per warp (its
-        // lanes split the orders; coefficient tables staged in the slice tile,
-        // which the FP32 modes leave unused until pass 2, when it is large
-        // enough), other kinds one voxel per thread
-        const int qn = min(s_qn, kVoxQueue);
-        const bool warp_sh = !kMaps && sp.kind == SCATMAN_SPHHARM &&
-                             sizeof(Cx) * (size_t)zs * kLinesPerCta >= kShTabDoubles * sizeof(double);
-        if (warp_sh && qn > 0) {
-            double *tab = reinterpret_cast<double *>(s_tile);
-            sh_stage_tables(sp, tab);
-            __syncthreads();
-            for (int k = warp; k < qn; k += kVoxThreads / 32) {
-                const int e = queue[k];
-                const int yl = e >> 16, iz = e & 0xffff;
-                const double in = sh_binary_fp64_warp(sp, gp, ix, y0 + yl, iz, tab);
-                if (lane == 0) chi_tile[(size_t)yl * zs + iz] = (float)in;
-            }
-        } else {
-            for (int k = threadIdx.x; k < qn; k += kVoxThreads) {
-                const int e = queue[k];
-                const int yl = e >> 16, iz = e & 0xffff;
-                chi_tile[(size_t)yl * zs + iz] = (float)occupancy_binary_fp64(sp, gp, ix, y0 + yl, iz);
-            }
-        }
-        __syncthreads();
-    }
-
     for (int yl = warp; yl < kLinesPerCta; yl += kVoxThreads / 32) {
         const int iy = y0 + yl;
         if (iy >= gp.ny) break;
@@ -310,34 +269,418 @@ __global__ void __launch_bounds__(kVoxThreads, 3) voxelise_scan_kernel(ShapePara
     }
 }
 
-__global__ void bounds_init_kernel(int *b, int nz, int *cy) {
+// T after C full voxels of the beam's path, (Re, Im) in the slices' precision.
+template <typename ScanT, typename Cx>
+__device__ __forceinline__ Cx full_voxels_T(const VoxConst &vc, int C) {
+    const ScanT mag = exp(-vc_pick<ScanT>(vc.att, vc.att_f) * (ScanT)C);
+    ScanT sn, cs;
+    sincos(vc_pick<ScanT>(vc.ph, vc.ph_f) * (ScanT)C, &sn, &cs);
+    Cx v;
+    v.x = mag * cs;
+    v.y = -(mag * sn);
+    return v;
+}
+
+// ---------------------------------------------------------------------------
+// Binary shapes of one index.  A voxel is a bit, C_j is a count of bits, and T
+// takes only the nz + 1 values of a table, so nothing of the scan runs per
+// voxel: a line of 32 z is one ballot, its prefix a popcount, its transmission a
+// load.  The FP64 modes settle a voxel in FP32 where the margin allows it, as
+// the FP32 modes do (the decision is the FP64 one either way).
+//
+// A CTA owns kLines y lines at one x, a warp takes whole lines.  What is left
+// is the surface radius near the surface: harmonics cost several hundred instructions
+// a voxel, so first the radius band and then a table of radii over a cube of
+// directions (6 x 64^2 for a radius of 48 voxels, good to the shape's steepest
+// slope times half a cell, about 1.4 voxels there) settle what they can, and the
+// voxels left are queued and evaluated by full warps.  Stores are 16 bytes per
+// thread and plane.  Few lines per CTA keep the SMs evenly loaded (planes
+// through the middle carry most of the surface): 16, and 8 where 16 would leave
+// SMs without a CTA.
+// ---------------------------------------------------------------------------
+constexpr int kBitSteps = kMaxRun + 1;       // padded row of a line's bit words
+
+// Coefficients staged in memory for the voxeliser: ShTerms, then the FP64 tables.
+// (Kernel parameters serve one address at a time, so reading them by lane is slow:
+// once per launch, not per CTA.)
+static_assert(sizeof(ShTerms) + kShTabDoubles * sizeof(double) <= kShStageInts * sizeof(int) &&
+                  sizeof(ShTerms) % 16 == 0,
+              "staged coefficients");
+__device__ __forceinline__ void block_copy(void *dst, const void *src, size_t bytes) {
+    for (int k = threadIdx.x; k < (int)(bytes / 8); k += blockDim.x)
+        reinterpret_cast<uint2 *>(dst)[k] = reinterpret_cast<const uint2 *>(src)[k];
+}
+
+// (relative error below 1e-6)
+__device__ __forceinline__ float sqrt_approx(float x) {
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Cell of direction p in the radius table: cube face, then the two tangents.
+__device__ __forceinline__ int rtab_cell(float px, float py, float pz, int n) {
+    const float ax = fabsf(px), ay = fabsf(py), az = fabsf(pz);
+    int face;
+    float m, a, b;
+    if (ax >= ay && ax >= az) {
+        face = 0;
+        m = px;
+        a = py;
+        b = pz;
+    } else if (ay >= az) {
+        face = 2;
+        m = py;
+        a = pz;
+        b = px;
+    } else {
+        face = 4;
+        m = pz;
+        a = px;
+        b = py;
+    }
+    if (m < 0.f) ++face;
+    const float s = __fdividef(0.5f * (float)n, fabsf(m)), h = 0.5f * (float)n;
+    const int i = min(n - 1, max(0, (int)fmaf(a, s, h))), j = min(n - 1, max(0, (int)fmaf(b, s, h)));
+    return (face * n + i) * n + j;
+}
+
+// Radius at the centre of cell k (see rtab_cell).
+__device__ __forceinline__ float rtab_radius(const ShapeParams &sp, const ShTerms &tab, int k) {
+    const int n = sp.rtab_n, face = k / (n * n), i = (k / n) % n, j = k % n;
+    const float m = (face & 1) ? -1.f : 1.f, a = (2 * i + 1) / (float)n - 1.f, b = (2 * j + 1) / (float)n - 1.f;
+    const float px = face < 2 ? m : face < 4 ? b : a, py = face < 2 ? a : face < 4 ? m : b;
+    const float pz = face < 2 ? b : face < 4 ? a : m;
+    return sh_radius_f(sp, tab, px, py, pz, rsqrtf(px * px + py * py + pz * pz));
+}
+
+template <bool kFp64, typename ScanT, bool kMaps, int kLines>
+__global__ void __launch_bounds__(kVoxThreads, 3) voxelise_binary_kernel(ShapeParams sp, GridParams gp, SliceOut out,
+                                                                         VoxConst vc) {
+    using Cx = typename std::conditional<kFp64, double2, float2>::type;
+    extern __shared__ __align__(16) unsigned char smem[];
+    Cx *T = reinterpret_cast<Cx *>(smem);                                     // [nz + 1]
+    __shared__ __align__(16) double s_tab[kMaps ? 1 : kShTabDoubles];
+    __shared__ uint32_t s_bits[kLines][kBitSteps];
+    __shared__ int s_base[kLines][kBitSteps];
+    uint16_t *near = reinterpret_cast<uint16_t *>(T + gp.nz + 1);             // [kLines nz]: (line << 9) | z
+    __shared__ int s_queue[kVoxQueue];                                        // the same, for the FP64 test
+    __shared__ int s_nn, s_qn;
+    __shared__ ShTerms s_sh;
+    if (threadIdx.x == 0) s_nn = s_qn = 0;
+    if (!kMaps && sp.kind == SCATMAN_SPHHARM) {
+        if (out.stage)
+            block_copy(&s_sh, out.stage, sizeof(ShTerms));
+        else
+            sh_stage_terms(sp, s_sh);
+    }
+    __syncthreads();
+    const int nz = gp.nz, steps = (nz + 31) / 32, ix = blockIdx.x, y0 = blockIdx.y * kLines;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const float vox = gp.voxf;
+    const float xo = ((float)ix - 0.5f * (float)(gp.nx - 1)) * vox - sp.cxf;
+    const bool band = sp.band_hi > 0.f, rtab = !kMaps && sp.rtab_n > 0 && out.rtab != nullptr;
+    const bool fp64_only = kFp64 && !sp.fp32_first;
+    // shapes with a costly surface queue their undecided voxels
+    const bool dense = sp.kind == SCATMAN_SPHHARM || sp.kind == SCATMAN_RADIALMAP || fp64_only;
+
+    constexpr int kU = 4;                        // steps whose table loads are in flight together
+    for (int yl = warp; yl < kLines; yl += kVoxThreads / 32) {
+        const int iy = y0 + yl;
+        const float yo = ((float)iy - 0.5f * (float)(gp.ny - 1)) * vox - sp.cyf;
+        const float r2xy = xo * xo + yo * yo;
+        const float rim = sp.band_hi * 1.0001f + 2e-3f * vox;
+        if (iy >= gp.ny || (band && r2xy > rim * rim)) {
+            // no voxel of the line (the band's margins are within the rim's)
+            if (lane < steps) s_bits[yl][lane] = 0u;
+            continue;
+        }
+#pragma unroll 1
+        for (int st0 = 0; st0 < steps; st0 += kU) {
+            bool in[kU], ask[kU];
+            float d[kU], r[kU];
+#pragma unroll
+            for (int q = 0; q < kU; ++q) {
+                const int iz = 32 * (st0 + q) + lane;
+                in[q] = false;
+                ask[q] = iz < nz;
+                d[q] = r[q] = 0.f;
+                if (ask[q] && band) {
+                    // |p| = |d|: the rotation keeps lengths; margins cover FP32 rounding
+                    const float zo = ((float)iz - 0.5f * (float)(nz - 1)) * vox - sp.czf;
+                    d[q] = sqrt_approx(r2xy + zo * zo);
+                    const float m = 1e-3f * vox + 1e-5f * d[q];
+                    in[q] = d[q] + m < sp.band_lo;
+                    ask[q] = !in[q] && d[q] - m <= sp.band_hi;
+                    if (!kMaps && ask[q] && rtab) {
+                        const float px = sp.Rf[0] * xo + sp.Rf[3] * yo + sp.Rf[6] * zo;
+                        const float py = sp.Rf[1] * xo + sp.Rf[4] * yo + sp.Rf[7] * zo;
+                        const float pz = sp.Rf[2] * xo + sp.Rf[5] * yo + sp.Rf[8] * zo;
+                        r[q] = __ldg(&out.rtab[rtab_cell(px, py, pz, sp.rtab_n)]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < kU; ++q) {
+                const int st = st0 + q, iz = 32 * st + lane;
+                if (st >= steps) break;
+                if (!kMaps && rtab && ask[q]) {
+                    const float over = r[q] - d[q];
+                    in[q] = over > sp.rtab_slack;
+                    ask[q] = fabsf(over) <= sp.rtab_slack;
+                }
+                if (!dense && ask[q]) {
+                    // (a few instructions each: no queue)
+                    const float c = occupancy_binary_f<kMaps>(sp, gp, s_sh, ix, iy, iz);
+                    in[q] = c > 0.f;
+                    if (c < 0.f) {
+                        const int slot = atomicAdd(&s_qn, 1);
+                        if (slot < kVoxQueue)
+                            s_queue[slot] = (yl << 9) | iz;
+                        else
+                            in[q] = occupancy_binary_fp64(sp, gp, ix, iy, iz) != 0.0;
+                    }
+                }
+                const uint32_t word = __ballot_sync(0xffffffffu, in[q]);
+                if (lane == 0) s_bits[yl][st] = word;
+                const uint32_t asking = __ballot_sync(0xffffffffu, dense && ask[q]);
+                if (asking) {
+                    int at = 0;
+                    if (lane == 0) at = atomicAdd(&s_nn, __popc(asking));
+                    at = __shfl_sync(0xffffffffu, at, 0);
+                    if (dense && ask[q]) near[at + __popc(asking & ((1u << lane) - 1u))] = (uint16_t)((yl << 9) | iz);
+                }
+            }
+        }
+    }
+    for (int k = threadIdx.x; k <= nz; k += kVoxThreads)
+        T[k] = out.table ? reinterpret_cast<const Cx *>(out.table)[k] : full_voxels_T<ScanT, Cx>(vc, k);
+    __syncthreads();
+    if (dense) {
+        for (int k = threadIdx.x; k < s_nn; k += kVoxThreads) {
+            const int e = near[k], yl = e >> 9, iz = e & 511, iy = y0 + yl;
+            bool in = false;
+            if (fp64_only) {
+                in = occupancy_binary_fp64(sp, gp, ix, iy, iz) != 0.0;
+            } else {
+                const float c = occupancy_binary_f<kMaps>(sp, gp, s_sh, ix, iy, iz);
+                in = c > 0.f;
+                if (c < 0.f) {
+                    // too close to the surface for FP32: queue it (inline when full)
+                    const int slot = atomicAdd(&s_qn, 1);
+                    if (slot < kVoxQueue)
+                        s_queue[slot] = e;
+                    else
+                        in = occupancy_binary_fp64(sp, gp, ix, iy, iz) != 0.0;
+                }
+            }
+            if (in) atomicOr(&s_bits[yl][iz >> 5], 1u << (iz & 31));
+        }
+        __syncthreads();
+    }
+    const int qn = min(s_qn, kVoxQueue);
+    if (qn > 0) {
+        // the queued voxels' FP64 decisions: harmonics one voxel per warp, other kinds one per thread
+        const bool warps = !kMaps && sp.kind == SCATMAN_SPHHARM;
+        if (warps) {
+            if (out.stage)
+                block_copy(s_tab, reinterpret_cast<const unsigned char *>(out.stage) + sizeof(ShTerms), sizeof(s_tab));
+            else
+                sh_stage_tables(sp, s_tab);
+            __syncthreads();
+        }
+        for (int k = warps ? warp : threadIdx.x; k < qn; k += warps ? kVoxThreads / 32 : kVoxThreads) {
+            const int yl = s_queue[k] >> 9, iz = s_queue[k] & 511;
+            const bool in = (warps ? sh_binary_fp64_warp(sp, gp, ix, y0 + yl, iz, s_tab)
+                                   : occupancy_binary_fp64(sp, gp, ix, y0 + yl, iz)) != 0.0;
+            if (in && !(warps && lane > 0)) atomicOr(&s_bits[yl][iz >> 5], 1u << (iz & 31));
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x < kLines) {
+        int n = 0;
+        for (int st = 0; st < steps; ++st) {
+            s_base[threadIdx.x][st] = n;
+            n += __popc(s_bits[threadIdx.x][st]);
+        }
+    }
+    if (out.bounds) {
+        // occupied box of each slice (order-independent min/max): lane b of step
+        // st collects slice 32 st + b's bits of all lines
+        for (int st = kVoxThreads / 32 - 1 - warp; st < steps; st += kVoxThreads / 32) {
+            const uint32_t w = lane < kLines ? s_bits[lane][st] : 0u;
+            uint32_t mine = 0;
+#pragma unroll
+            for (int b = 0; b < 32; ++b) {
+                const uint32_t m = __ballot_sync(0xffffffffu, (w >> b) & 1u);
+                if (lane == b) mine = m;
+            }
+            const int iz = 32 * st + lane;
+            if (mine) {
+                const int lo = y0 + __ffs(mine) - 1, hi = y0 + 32 - __clz(mine);
+                atomicMin(&out.bounds[iz], ix);
+                atomicMax(&out.bounds[nz + iz], ix + 1);
+                atomicMin(&out.bounds[2 * nz + iz], lo);
+                atomicMax(&out.bounds[3 * nz + iz], hi);
+                if (out.chunk_y) {
+                    // y range of this slice's 8-column chunk (tensor-core grids: ix < 8 kGeomChunks)
+                    const int c = iz * kGeomChunks + (ix >> 3);
+                    atomicMin(&out.chunk_y[c], lo);
+                    atomicMax(&out.chunk_y[kGeomChunks * nz + c], hi);
+                }
+            }
+        }
+    }
+    __syncthreads();
+
+    const long long nxy = (long long)gp.nx * gp.ny;
+    if (out.layout == kLayoutC64 || out.layout == kLayoutC32) {
+        for (int it = threadIdx.x; it < nz * kLines; it += kVoxThreads) {
+            const int iz = it / kLines, yl = it % kLines, iy = y0 + yl;
+            if (iy >= gp.ny) continue;
+            const uint32_t w = s_bits[yl][iz >> 5], below = w & ((1u << (iz & 31)) - 1u);
+            const bool in = (w >> (iz & 31)) & 1u;
+            Cx v;
+            v.x = v.y = 0;
+            if (in) v = T[s_base[yl][iz >> 5] + __popc(below)];
+            const long long at = iz * nxy + (long long)ix * gp.ny + iy;
+            out.chi[at] = in ? 1.f : 0.f;
+            reinterpret_cast<Cx *>(out.s)[at] = v;
+        }
+        return;
+    }
+    if constexpr (!kFp64) {
+        // tensor-core slice operand (planes -Im, Re, Im; see voxelise_scan_kernel): a
+        // thread packs 8 consecutive y of one slice.  Rows run to Kp, a multiple of
+        // 16, so the store past ny falls into the padding, which stays zero.
+        constexpr int kGroups = kLines / 8;
+        const bool f16 = out.layout == kLayoutTcF16, wide = (gp.ny & 3) == 0;
+        for (int it = threadIdx.x; it < nz * kGroups; it += kVoxThreads) {
+            const int iz = it / kGroups, yg = 8 * (it % kGroups), iy = y0 + yg;
+            if (iy >= gp.ny) continue;
+            float re[8], im[8], chi[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const uint32_t w = s_bits[yg + k][iz >> 5], below = w & ((1u << (iz & 31)) - 1u);
+                const bool in = (w >> (iz & 31)) & 1u;
+                float2 v = make_float2(0.f, 0.f);
+                if (in) v = T[s_base[yg + k][iz >> 5] + __popc(below)];
+                re[k] = v.x;
+                im[k] = v.y;
+                chi[k] = in ? 1.f : 0.f;
+            }
+            uint32_t pr[4], pi[4], pn[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (f16) {
+                    const __half2 a = __floats2half2_rn(re[2 * k], re[2 * k + 1]);
+                    const __half2 b = __floats2half2_rn(im[2 * k], im[2 * k + 1]);
+                    const __half2 c = __floats2half2_rn(-im[2 * k], -im[2 * k + 1]);
+                    pr[k] = *reinterpret_cast<const uint32_t *>(&a);
+                    pi[k] = *reinterpret_cast<const uint32_t *>(&b);
+                    pn[k] = *reinterpret_cast<const uint32_t *>(&c);
+                } else {
+                    const __nv_bfloat162 a = __floats2bfloat162_rn(re[2 * k], re[2 * k + 1]);
+                    const __nv_bfloat162 b = __floats2bfloat162_rn(im[2 * k], im[2 * k + 1]);
+                    const __nv_bfloat162 c = __floats2bfloat162_rn(-im[2 * k], -im[2 * k + 1]);
+                    pr[k] = *reinterpret_cast<const uint32_t *>(&a);
+                    pi[k] = *reinterpret_cast<const uint32_t *>(&b);
+                    pn[k] = *reinterpret_cast<const uint32_t *>(&c);
+                }
+            }
+            uint16_t *row = reinterpret_cast<uint16_t *>(out.s) + ((size_t)iz * 3 * out.Nxp + ix) * out.Kp + iy;
+            const size_t plane = (size_t)out.Nxp * out.Kp;
+            *reinterpret_cast<uint4 *>(row) = make_uint4(pn[0], pn[1], pn[2], pn[3]);
+            *reinterpret_cast<uint4 *>(row + plane) = make_uint4(pr[0], pr[1], pr[2], pr[3]);
+            *reinterpret_cast<uint4 *>(row + 2 * plane) = make_uint4(pi[0], pi[1], pi[2], pi[3]);
+            float *x = out.chi + iz * nxy + (long long)ix * gp.ny + iy;
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                if (wide && iy + 4 * g + 4 <= gp.ny) {
+                    *reinterpret_cast<float4 *>(x + 4 * g) =
+                        make_float4(chi[4 * g], chi[4 * g + 1], chi[4 * g + 2], chi[4 * g + 3]);
+                } else {
+#pragma unroll
+                    for (int k = 4 * g; k < 4 * g + 4; ++k)
+                        if (iy + k < gp.ny) x[k] = chi[k];
+                }
+            }
+        }
+    }
+}
+
+// Empty bounds, the transmission table (table: the T of 0 .. nz full voxels, or
+// null), and in the blocks from `first` on the radius table, after a block that
+// stages the coefficients.
+template <typename ScanT, typename Cx>
+__global__ void voxelise_init_kernel(ShapeParams sp, int *b, int nz, int *cy, Cx *table, VoxConst vc, int first,
+                                     void *stage, float *rtab) {
+    if ((int)blockIdx.x == first) {
+        sh_stage_terms(sp, *reinterpret_cast<ShTerms *>(stage));
+        sh_stage_tables(sp, reinterpret_cast<double *>(reinterpret_cast<unsigned char *>(stage) + sizeof(ShTerms)));
+        return;
+    }
+    if ((int)blockIdx.x > first) {
+        __shared__ ShTerms s_sh;
+        sh_stage_terms(sp, s_sh);
+        __syncthreads();
+        const int k = (blockIdx.x - first - 1) * blockDim.x + threadIdx.x;
+        if (k < 6 * sp.rtab_n * sp.rtab_n) rtab[k] = rtab_radius(sp, s_sh, k);
+        return;
+    }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < 4 * nz) {
         const int part = i / nz;
         b[i] = (part == 0 || part == 2) ? 0x7fffffff : 0;     // lo parts start high, hi parts low
     }
     if (cy && i < 2 * kGeomChunks * nz) cy[i] = i < kGeomChunks * nz ? 0x7fffffff : 0;
+    const int last = first * blockDim.x - 1 - i;          // the last threads: neither bounds nor many chunks
+    if (table && last <= nz) table[last] = full_voxels_T<ScanT, Cx>(vc, last);
+}
+
+template <bool kFp64, typename ScanT>
+static cudaError_t run_voxelise(const ShapeParams &sp, const GridParams &gp, const SliceOut &out, const VoxConst &vc,
+                                cudaStream_t st) {
+    using Cx = typename std::conditional<kFp64, double2, float2>::type;
+    const bool maps = sp.kind == SCATMAN_RADIALMAP || sp.kind == SCATMAN_VOLUMEMAP;
+    const bool binary = !sp.soft && !sp.varn;
+    if (out.bounds) {
+        const int first = (2 * kGeomChunks * gp.nz + 255) / 256;
+        const int cells = binary ? 6 * sp.rtab_n * sp.rtab_n : 0;
+        const int more = binary && sp.kind == SCATMAN_SPHHARM ? 1 + (cells + 255) / 256 : 0;
+        voxelise_init_kernel<ScanT, Cx><<<first + more, 256, 0, st>>>(
+            sp, out.bounds, gp.nz, out.chunk_y, binary ? (Cx *)out.table : nullptr, vc, first, out.stage, out.rtab);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    if (binary) {
+        // CTAs of 8 lines where 16 leave fewer than two per SM of a 152-SM part
+        const bool small = (long long)gp.nx * ((gp.ny + 15) / 16) < 304;
+        const int lines = small ? 8 : 16;
+        const size_t smem = sizeof(Cx) * ((size_t)gp.nz + 1) + sizeof(uint16_t) * (size_t)lines * gp.nz;
+        const dim3 grid(gp.nx, (gp.ny + lines - 1) / lines);
+        auto k = small ? (maps ? voxelise_binary_kernel<kFp64, ScanT, true, 8> : voxelise_binary_kernel<kFp64, ScanT, false, 8>)
+                       : (maps ? voxelise_binary_kernel<kFp64, ScanT, true, 16>
+                               : voxelise_binary_kernel<kFp64, ScanT, false, 16>);
+        k<<<grid, kVoxThreads, smem, st>>>(sp, gp, out, vc);
+        return cudaGetLastError();
+    }
+    const dim3 grid(gp.nx, (gp.ny + kLinesPerCta - 1) / kLinesPerCta);
+    const size_t smem = (sizeof(Cx) + sizeof(float)) * (size_t)(gp.nz + 1) * kLinesPerCta;
+    // per-function attribute shared by all threads: set it to the largest size
+    // (nz = 256) so a concurrent launch from another thread is never rejected
+    const int smem_max = (int)((sizeof(Cx) + sizeof(float)) * ((kFp64 ? 256 : 32 * kMaxRun) + 1) * kLinesPerCta);
+    auto k = maps ? voxelise_scan_kernel<kFp64, ScanT, true> : voxelise_scan_kernel<kFp64, ScanT, false>;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+    if (e != cudaSuccess) return e;
+    k<<<grid, kVoxThreads, smem, st>>>(sp, gp, out, vc);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_voxelise(const ShapeParams &sp, const GridParams &gp, const SliceOut &out, bool scan_fp64,
                             bool fp64_mode, cudaStream_t st) {
     if (gp.nz > 32 * kMaxRun || (fp64_mode && gp.nz > 256)) return cudaErrorInvalidValue;
     if (out.chunk_y && (out.bounds == nullptr || gp.nx > 8 * kGeomChunks)) return cudaErrorInvalidValue;
-    if (out.bounds)
-        bounds_init_kernel<<<(2 * kGeomChunks * gp.nz + 255) / 256, 256, 0, st>>>(out.bounds, gp.nz, out.chunk_y);
-    dim3 grid(gp.nx, (gp.ny + kLinesPerCta - 1) / kLinesPerCta);
-    size_t cx = fp64_mode ? sizeof(double2) : sizeof(float2);
-    size_t smem = (cx + sizeof(float)) * (size_t)(gp.nz + 1) * kLinesPerCta + kVoxQueue * sizeof(int);
-    // per-function attribute shared by all threads: set it to the largest size
-    // (nz = 256) so a concurrent launch from another thread is never rejected
-    const int smem_max = (int)((cx + sizeof(float)) * ((fp64_mode ? 256 : 32 * kMaxRun) + 1) * kLinesPerCta +
-                               kVoxQueue * sizeof(int));
-    const bool maps = sp.kind == SCATMAN_RADIALMAP || sp.kind == SCATMAN_VOLUMEMAP;
-    auto k = fp64_mode   ? (maps ? voxelise_scan_kernel<true, double, true> : voxelise_scan_kernel<true, double, false>)
-             : scan_fp64 ? (maps ? voxelise_scan_kernel<false, double, true> : voxelise_scan_kernel<false, double, false>)
-                         : (maps ? voxelise_scan_kernel<false, float, true> : voxelise_scan_kernel<false, float, false>);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
-    if (e != cudaSuccess) return e;
     VoxConst vc;
     vc.att = gp.k0 * gp.voxel * gp.beta;
     vc.ph = gp.k0 * gp.voxel * gp.delta;
@@ -347,8 +690,9 @@ cudaError_t launch_voxelise(const ShapeParams &sp, const GridParams &gp, const S
     vc.ph_f = (float)vc.ph;
     vc.kdz_f = (float)vc.kdz;
     vc.inv_scale_f = (float)vc.inv_scale;
-    k<<<grid, kVoxThreads, smem, st>>>(sp, gp, out, vc);
-    return cudaGetLastError();
+    return fp64_mode   ? run_voxelise<true, double>(sp, gp, out, vc, st)
+           : scan_fp64 ? run_voxelise<false, double>(sp, gp, out, vc, st)
+                       : run_voxelise<false, float>(sp, gp, out, vc, st);
 }
 
 }  // namespace scm
