@@ -758,13 +758,14 @@ int scatman_voxelise(scatman_handle *h, const scatman_shape *s) {
 }
 
 // The pixels around the forward direction that hold a parametric shape's central
-// peak, |q| r < 3.3 with r its smallest half-width (outside, a sphere's
-// intensity is below 2 % of the peak's); none for a map.  A fit's loss is the
-// difference between the pattern and a measured one that nearly equals it,
-// twenty times smaller and more, and its value is set in the peak: there the
-// 16-bit phase pairs' rounding, 1e-6 of the intensity and another for the grid's
-// directions than for the pixel's own, would move the loss by 4e-5 (measured,
-// 96^3 on 256^2; with the peak's sums direct 1e-6).
+// peak, |q| r < 4.5 with r its smallest half-width (up to a sphere's first zero;
+// beyond it its intensity is below 0.8 % of the peak's); none for a map.  A fit's
+// loss is the difference between the pattern and a measured one that nearly equals
+// it, twenty times smaller and more, and its value and gradient are set in the
+// peak: there the 16-bit phase pairs' rounding, 1e-6 of the intensity and another
+// for the grid's directions than for the pixel's own, would move the loss by 4e-5
+// (measured, 96^3 on 256^2; with the peak's sums direct 1e-6), and a nearly
+// cancelling gradient by as much already from a rim at 3.3 (7 % of the peak).
 static PixelRect peak_pixels(const scatman_handle *h) {
     const scatman_config &c = h->cfg;
     const scatman_shape &s = h->shape;
@@ -774,7 +775,7 @@ static PixelRect peak_pixels(const scatman_handle *h) {
     if (s.kind == SCATMAN_SPHHARM) r = s.R0;
     PixelRect p;
     if (!(r > 0.0)) return p;
-    const double sn = 3.3 / (r * 2.0 * h->k0);                   // sin(theta / 2) at the rim
+    const double sn = 4.5 / (r * 2.0 * h->k0);                   // sin(theta / 2) at the rim
     const double X = sn < 0.7 ? std::tan(2.0 * std::asin(sn)) / std::tan(c.theta_max_deg * kPi / 180.0) : 1.0;
     auto margin = [&](int n) { return X < 1.0 ? (int)std::floor(0.5 * ((n - 1) - X * n)) : 0; };
     p.u0 = std::max(0, margin(c.det_nx));
