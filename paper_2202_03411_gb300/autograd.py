@@ -33,7 +33,11 @@ def params_of(shape: Shape) -> np.ndarray:
 
 def shape_with(template: Shape, params) -> Shape:
     p = np.asarray(params, dtype=np.float64)
-    s = copy.deepcopy(template)
+    s = copy.copy(template)
+    for name, v in vars(template).items():
+        # (a deep copy of the whole object walks its two dozen numbers too)
+        if not isinstance(v, (int, float, type(None))) and not (name == "alm" and s.kind not in (SPHERE, ELLIPSOID)):
+            setattr(s, name, copy.deepcopy(v))
     if s.kind == SPHERE:
         s.r = float(p[0])
     elif s.kind == ELLIPSOID:

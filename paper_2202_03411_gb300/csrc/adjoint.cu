@@ -535,6 +535,37 @@ cudaError_t launch_grad_pixels(bool fp64, const void *A, const void *dLdI, long 
     return cudaGetLastError();
 }
 
+// The partial sums over blocks, one block per value: the ng + 2 voxel sums, the
+// pixel sum, and the handle's error word, so that one small copy brings all that
+// the host needs.
+__global__ void __launch_bounds__(128) grad_totals_kernel(const double *__restrict__ part, int nvb, int nv, int npb,
+                                                          const int *__restrict__ err, double *__restrict__ out) {
+    __shared__ double red[128];
+    const int k = blockIdx.x;
+    double s = 0.0;
+    if (k < nv) {
+        for (int b = threadIdx.x; b < nvb; b += 128) s += part[(size_t)b * nv + k];
+    } else {
+        for (int b = threadIdx.x; b < npb; b += 128) s += part[(size_t)nvb * nv + b];
+    }
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = 64; o > 0; o >>= 1) {
+        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        out[k] = red[0];
+        if (k == nv) out[nv + 1] = (double)*err;
+    }
+}
+
+cudaError_t launch_grad_totals(const double *part, int nvb, int nv, int npb, const int *err, double *out,
+                               cudaStream_t st) {
+    grad_totals_kernel<<<nv + 1, 128, 0, st>>>(part, nvb, nv, npb, err, out);
+    return cudaGetLastError();
+}
+
 }  // namespace scm
 
 namespace scm {

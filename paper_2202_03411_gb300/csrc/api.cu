@@ -192,8 +192,11 @@ void scatman_destroy(scatman_handle *h) {
     cudaFree(h->d_rmap);
     cudaFree(h->d_rmapf);
     cudaFree(h->d_vmap);
-    cudaFree(h->d_mdelta);
-    cudaFree(h->d_mbeta);
+    cudaFree(h->d_mdelta);           // (with d_mbeta behind it)
+    for (auto &m : h->map_stage) {
+        cudaFreeHost(m.p);
+        if (m.ev) cudaEventDestroy(m.ev);
+    }
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     if (dev_prev >= 0) cudaSetDevice(dev_prev);
     delete h;
@@ -371,7 +374,7 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
     const size_t npix = (size_t)h->n_pix;
     const bool f64 = (h->precision == SCATMAN_FP64);
     int rc;
-    h->adj_on_grid = use_field_grid_adjoint(*cfg, &h->fg);
+    h->adj_on_grid = use_field_grid_adjoint(*cfg, &h->fg);      // (the same plan)
     h->on_grid = use_field_grid(*cfg, &h->fg);
     h->peak_direct = h->on_grid && h->tensor_core && c.soft;
     const bool direct = !h->on_grid || h->peak_direct;          // some pixels' sums run over their own q
@@ -475,11 +478,23 @@ static void set_radius_band(const scatman_shape *s, ShapeParams *sp, bool fp64) 
         lo = std::fmin(std::fmax(s->R0 * (1.0 - b), sp->rmin), sp->rmax);
         hi = std::fmin(std::fmax(s->R0 * (1.0 + b), sp->rmin), sp->rmax);
     } else if (s->kind == SCATMAN_RADIALMAP) {
-        lo = hi = s->radial_map[0];
-        for (long long k = 1; k < (long long)s->map_ntheta * s->map_nphi; ++k) {
-            lo = std::fmin(lo, s->radial_map[k]);
-            hi = std::fmax(hi, s->radial_map[k]);
+        const size_t n = (size_t)s->map_ntheta * s->map_nphi;
+        constexpr size_t kL = 8;                                    // independent extrema: vector code
+        double los[kL], his[kL];
+        for (size_t i = 0; i < kL; ++i) los[i] = his[i] = s->radial_map[0];
+        size_t k = 0;
+        for (; k + kL <= n; k += kL)
+            for (size_t i = 0; i < kL; ++i) {
+                const double r = s->radial_map[k + i];
+                los[i] = r < los[i] ? r : los[i];
+                his[i] = r > his[i] ? r : his[i];
+            }
+        for (; k < n; ++k) {
+            los[0] = std::fmin(los[0], s->radial_map[k]);
+            his[0] = std::fmax(his[0], s->radial_map[k]);
         }
+        lo = *std::min_element(los, los + kL);
+        hi = *std::max_element(his, his + kL);
     } else if (sp->soft && s->kind == SCATMAN_SPHERE) {
         lo = hi = s->r;                 // binary spheres and ellipsoids decide cheaply without it
     } else if (sp->soft && s->kind == SCATMAN_ELLIPSOID) {
@@ -556,9 +571,92 @@ static void set_radius_table(const scatman_config &c, ShapeParams *sp) {
     sp->rtab_slack = (float)slack;
 }
 
+// Pinned staging for a map upload of `bytes`, kept by the handle: the copies then
+// run beside the host, which waits only for the upload before the last one.
+// A captured upload reads its staging at every replay: memory of its own, kept until
+// the handle goes (map_staged then records nothing).
+static int map_staging(scatman_handle *h, size_t bytes, unsigned char **out) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    int rc = check_cuda(h, cudaStreamIsCapturing(h->stream, &cap), "map staging");
+    if (rc) return rc;
+    h->map_captured = cap != cudaStreamCaptureStatusNone;
+    if (h->map_captured) {
+        h->captured_maps.emplace_back((bytes + 7) / 8);
+        *out = (unsigned char *)h->captured_maps.back().data();
+        return SCATMAN_OK;
+    }
+    scatman_handle::MapStage &m = h->map_stage[h->map_turn ^= 1];
+    if (!m.ev && (rc = check_cuda(h, cudaEventCreateWithFlags(&m.ev, cudaEventDisableTiming), "map staging"))) return rc;
+    if ((rc = check_cuda(h, cudaEventSynchronize(m.ev), "map staging"))) return rc;
+    if (m.cap < bytes) {
+        cudaFreeHost(m.p);
+        m.p = nullptr;
+        m.cap = 0;
+        if ((rc = check_cuda(h, cudaHostAlloc((void **)&m.p, bytes, cudaHostAllocDefault), "map staging"))) return rc;
+        m.cap = bytes;
+    }
+    *out = m.p;
+    return SCATMAN_OK;
+}
+
+// After the upload's copies.
+static int map_staged(scatman_handle *h) {
+    return h->map_captured ? SCATMAN_OK
+                           : check_cuda(h, cudaEventRecord(h->map_stage[h->map_turn].ev, h->stream), "map staging");
+}
+
+// A volume map's index values into `dl` and `bt` (the shape's where an array is
+// absent), in one pass: their largest |n^2 - 1| squared and magnitude, and whether
+// all are finite.
+struct MapScan {
+    double scale2 = 0.0, imax = 0.0;
+    bool finite = true;
+};
+static MapScan scan_map_index(const scatman_shape *s, size_t n, double *dl, double *bt) {
+    constexpr size_t kL = 8;                                        // independent lanes: vector code
+    double scale[kL] = {}, imax[kL] = {}, zero[kL] = {};
+    const double *md = s->map_delta, *mb = s->map_beta;
+    const double d0[kL] = {s->delta, s->delta, s->delta, s->delta, s->delta, s->delta, s->delta, s->delta};
+    const double b0[kL] = {s->beta, s->beta, s->beta, s->beta, s->beta, s->beta, s->beta, s->beta};
+    auto lanes = [&](const double *vd, const double *vb, size_t k, size_t m) {
+        for (size_t i = 0; i < m; ++i) {
+            const double d = vd[i], b = vb[i];
+            dl[k + i] = d;
+            bt[k + i] = b;
+            const double re = -2.0 * d + d * d - b * b, im = 2.0 * b - 2.0 * d * b, q = re * re + im * im;
+            const double ad = std::fabs(d), ab = std::fabs(b), a = ad > ab ? ad : ab;
+            scale[i] = q > scale[i] ? q : scale[i];
+            imax[i] = a > imax[i] ? a : imax[i];
+            zero[i] += 0.0 * d + 0.0 * b;                           // not a number once a value is not finite
+        }
+    };
+    size_t k = 0;
+    for (; k + kL <= n; k += kL) lanes(md ? md + k : d0, mb ? mb + k : b0, k, kL);
+    lanes(md ? md + k : d0, mb ? mb + k : b0, k, n - k);
+    MapScan r;
+    for (size_t i = 0; i < kL; ++i) {
+        r.scale2 = std::fmax(r.scale2, scale[i]);
+        r.imax = std::fmax(r.imax, imax[i]);
+        r.finite = r.finite && zero[i] == 0.0;
+    }
+    return r;
+}
+
+// Whether all n values are finite (their exponents, so that the loop is vector code).
+static bool all_finite(const double *v, size_t n) {
+    uint64_t bad = 0;
+    for (size_t k = 0; k < n; ++k) {
+        uint64_t b;
+        std::memcpy(&b, v + k, 8);
+        bad |= (uint64_t)((b & 0x7ff0000000000000ull) == 0x7ff0000000000000ull);
+    }
+    return bad == 0;
+}
+
 // Copies a map shape's arrays to the device (grown buffers owned by the handle)
 // and fills the map fields of the shape parameters.
-static int upload_maps(scatman_handle *h, const scatman_shape *s, ShapeParams *sp) {
+static int upload_maps(scatman_handle *h, const scatman_shape *s, unsigned char *stage, const MapScan &scan,
+                       ShapeParams *sp) {
     int rc;
     sp->varn = 0;
     sp->nscale = 1.0;
@@ -576,22 +674,26 @@ static int upload_maps(scatman_handle *h, const scatman_shape *s, ShapeParams *s
             if ((rc = alloc_dev(h, (void **)&h->d_rmapf, n * sizeof(float), "radial map"))) return rc;
             h->rmap_cap = n;
         }
-        std::vector<float> f(n);
+        double *rd = (double *)stage;
+        float *f = (float *)(rd + n);
         double slope_t = 0.0, slope_p = 0.0;
-        for (int i = 0; i < nt; ++i)
+        for (int i = 0; i < nt; ++i) {
+            const double *row = s->radial_map + (size_t)i * np, *next = s->radial_map + (size_t)((i + 1) % nt) * np;
             for (int k = 0; k < np; ++k) {
-                const double r = s->radial_map[(size_t)i * np + k];
+                const double r = row[k], dt = std::fabs(next[k] - r), dp = std::fabs(row[k + 1 < np ? k + 1 : 0] - r);
+                rd[(size_t)i * np + k] = r;
                 f[(size_t)i * np + k] = (float)r;
-                slope_t = std::fmax(slope_t, std::fabs(s->radial_map[(size_t)((i + 1) % nt) * np + k] - r));
-                slope_p = std::fmax(slope_p, std::fabs(s->radial_map[(size_t)i * np + (k + 1) % np] - r));
+                slope_t = dt > slope_t ? dt : slope_t;
+                slope_p = dp > slope_p ? dp : slope_p;
             }
-        if ((rc = check_cuda(h, cudaMemcpyAsync(h->d_rmap, s->radial_map, n * sizeof(double), cudaMemcpyHostToDevice,
-                                                 h->stream), "radial map upload")))
+        }
+        if ((rc = check_cuda(h, cudaMemcpyAsync(h->d_rmap, rd, n * sizeof(double), cudaMemcpyHostToDevice, h->stream),
+                             "radial map upload")))
             return rc;
-        if ((rc = check_cuda(h, cudaMemcpyAsync(h->d_rmapf, f.data(), n * sizeof(float), cudaMemcpyHostToDevice,
-                                                 h->stream), "radial map upload")))
+        if ((rc = check_cuda(h, cudaMemcpyAsync(h->d_rmapf, f, n * sizeof(float), cudaMemcpyHostToDevice, h->stream),
+                             "radial map upload")))
             return rc;
-        // a copy from pageable host memory has left the staging vector when the call returns
+        if ((rc = map_staged(h))) return rc;
         sp->rmap = h->d_rmap;
         sp->rmapf = h->d_rmapf;
         sp->ntheta = nt;
@@ -611,7 +713,11 @@ static int upload_maps(scatman_handle *h, const scatman_shape *s, ShapeParams *s
             if ((rc = alloc_dev(h, (void **)&h->d_vmap, n, "volume map"))) return rc;
             h->vmap_cap = n;
         }
-        if ((rc = check_cuda(h, cudaMemcpyAsync(h->d_vmap, s->volume_map, n, cudaMemcpyHostToDevice, h->stream),
+        const bool varn = s->map_delta || s->map_beta;
+        const double *dl = (const double *)stage;                    // (with an index per cell, then its beta)
+        unsigned char *cells = stage + (varn ? 2 * n * sizeof(double) : 0);
+        std::memcpy(cells, s->volume_map, n);
+        if ((rc = check_cuda(h, cudaMemcpyAsync(h->d_vmap, cells, n, cudaMemcpyHostToDevice, h->stream),
                              "volume map upload")))
             return rc;
         sp->vmap = h->d_vmap;
@@ -620,40 +726,25 @@ static int upload_maps(scatman_handle *h, const scatman_shape *s, ShapeParams *s
         sp->mz = s->map_nz;
         sp->mdx = s->map_dx;
         sp->mdxf = (float)s->map_dx;
-        if (s->map_delta || s->map_beta) {
+        if (varn) {
             if (h->mindex_cap < n) {
                 cudaFree(h->d_mdelta);
-                cudaFree(h->d_mbeta);
                 h->d_mdelta = h->d_mbeta = nullptr;
                 h->mindex_cap = 0;
-                if ((rc = alloc_dev(h, (void **)&h->d_mdelta, n * sizeof(double), "map index"))) return rc;
-                if ((rc = alloc_dev(h, (void **)&h->d_mbeta, n * sizeof(double), "map index"))) return rc;
+                if ((rc = alloc_dev(h, (void **)&h->d_mdelta, 2 * n * sizeof(double), "map index"))) return rc;
                 h->mindex_cap = n;
             }
-            // per-cell values, the shape's where an array is absent; the scale
-            // is the largest |n^2 - 1| over the cells
-            std::vector<double> dl(n), bt(n);
-            double scale = 0.0, imax = 0.0;
-            for (size_t k = 0; k < n; ++k) {
-                dl[k] = s->map_delta ? s->map_delta[k] : s->delta;
-                bt[k] = s->map_beta ? s->map_beta[k] : s->beta;
-                const double re = -2.0 * dl[k] + dl[k] * dl[k] - bt[k] * bt[k];
-                const double im = 2.0 * bt[k] - 2.0 * dl[k] * bt[k];
-                scale = std::fmax(scale, std::sqrt(re * re + im * im));
-                imax = std::fmax(imax, std::fmax(std::fabs(dl[k]), std::fabs(bt[k])));
-            }
-            if ((rc = check_cuda(h, cudaMemcpyAsync(h->d_mdelta, dl.data(), n * sizeof(double), cudaMemcpyHostToDevice,
-                                                     h->stream), "map index upload")))
-                return rc;
-            if ((rc = check_cuda(h, cudaMemcpyAsync(h->d_mbeta, bt.data(), n * sizeof(double), cudaMemcpyHostToDevice,
+            h->d_mbeta = h->d_mdelta + n;
+            if ((rc = check_cuda(h, cudaMemcpyAsync(h->d_mdelta, dl, 2 * n * sizeof(double), cudaMemcpyHostToDevice,
                                                      h->stream), "map index upload")))
                 return rc;
             sp->mdelta = h->d_mdelta;
             sp->mbeta = h->d_mbeta;
             sp->varn = 1;
-            sp->nscale = scale > 0.0 ? scale : 1.0;
-            h->map_index_max = imax;
+            sp->nscale = scan.scale2 > 0.0 ? std::sqrt(scan.scale2) : 1.0;
+            h->map_index_max = scan.imax;
         }
+        if ((rc = map_staged(h))) return rc;
     }
     return SCATMAN_OK;
 }
@@ -667,21 +758,29 @@ int scatman_voxelise(scatman_handle *h, const scatman_shape *s) {
     if (s->kind == SCATMAN_RADIALMAP) {
         if (!s->radial_map || s->map_ntheta < 1 || s->map_nphi < 1)
             return set_error(h, SCATMAN_ERR_ARG, "radial map needs data and map_ntheta, map_nphi >= 1");
-        for (long long k = 0; k < (long long)s->map_ntheta * s->map_nphi; ++k)
-            if (!std::isfinite(s->radial_map[k])) return set_error(h, SCATMAN_ERR_ARG, "radial map values must be finite");
+        if (!all_finite(s->radial_map, (size_t)s->map_ntheta * s->map_nphi))
+            return set_error(h, SCATMAN_ERR_ARG, "radial map values must be finite");
     }
     if (s->kind == SCATMAN_VOLUMEMAP) {
         if (!s->volume_map || s->map_nx < 1 || s->map_ny < 1 || s->map_nz < 1 || !(s->map_dx > 0))
             return set_error(h, SCATMAN_ERR_ARG, "volume map needs data, map_nx/ny/nz >= 1 and map_dx > 0");
-        const long long ncell = (long long)s->map_nx * s->map_ny * s->map_nz;
-        for (const double *arr : {s->map_delta, s->map_beta})
-            if (arr)
-                for (long long k = 0; k < ncell; ++k)
-                    if (!std::isfinite(arr[k])) return set_error(h, SCATMAN_ERR_ARG, "map index values must be finite");
     }
     {
         std::string why;
         if (!check_param_shape(s, &why)) return set_error(h, SCATMAN_ERR_ARG, why);
+    }
+    // a map's arrays go to the staging memory here, where they are also looked over
+    unsigned char *stage = nullptr;
+    MapScan scan;
+    if (is_map_kind(s->kind)) {
+        const bool radii = s->kind == SCATMAN_RADIALMAP, varn = s->map_delta || s->map_beta;
+        const size_t n = radii ? (size_t)s->map_ntheta * s->map_nphi : (size_t)s->map_nx * s->map_ny * s->map_nz;
+        const int rc = map_staging(h, n * (radii ? sizeof(double) + sizeof(float) : varn ? 1 + 2 * sizeof(double) : 1), &stage);
+        if (rc) return rc;
+        if (!radii && varn) {
+            scan = scan_map_index(s, n, (double *)stage, (double *)stage + n);
+            if (!scan.finite) return set_error(h, SCATMAN_ERR_ARG, "map index values must be finite");
+        }
     }
 
     h->shape = *s;
@@ -716,7 +815,7 @@ int scatman_voxelise(scatman_handle *h, const scatman_shape *s) {
     sp.cz = s->cz;
     for (size_t k = 0; k < h->alm.size(); ++k) sp.alm[k] = h->alm[k];
     finish_shape_params(&sp);
-    int rc = upload_maps(h, s, &sp);
+    int rc = is_map_kind(s->kind) ? upload_maps(h, s, stage, scan, &sp) : SCATMAN_OK;
     if (rc) return rc;
     set_radius_band(s, &sp, h->precision == SCATMAN_FP64);
     set_fp32_test(c, &sp);
@@ -1170,7 +1269,7 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
     const GridParams gp = make_grid(c.nx, c.ny, c.nz, c.voxel, h->k0, h->shape.delta, h->shape.beta);
     const int ng = grad_param_count(h->sp);
     const int nvb = grad_voxel_blocks(f64, h->sp, gp, h->sm_count), npb = grad_pixel_blocks(h->n_pix);
-    const size_t need = (size_t)nvb * (ng + 2) + (size_t)npb;
+    const size_t need = (size_t)nvb * (ng + 2) + (size_t)npb + (size_t)ng + 4;      // and the totals
     if (h->part_count < need) {
         cudaFree(h->d_part);
         h->d_part = nullptr;
@@ -1256,18 +1355,18 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
                                           h->stream),
                     "pixel gradient");
     if (rc) return rc;
-    std::vector<double> part(need);
-    rc = check_cuda(h, cudaMemcpyAsync(part.data(), h->d_part, need * sizeof(double), cudaMemcpyDeviceToHost,
+    double *d_tot = h->d_part + (size_t)nvb * (ng + 2) + (size_t)npb;
+    rc = check_cuda(h, launch_grad_totals(h->d_part, nvb, ng + 2, npb, h->d_err, d_tot, h->stream), "gradient sums");
+    if (rc) return rc;
+    // the copy into pageable memory has finished when the call returns
+    std::vector<double> sums((size_t)ng + 4);
+    rc = check_cuda(h, cudaMemcpyAsync(sums.data(), d_tot, sums.size() * sizeof(double), cudaMemcpyDeviceToHost,
                                        h->stream),
                     "gradient download");
     if (rc) return rc;
-    if ((rc = scatman_sync(h))) return rc;
-    // fixed-order sums of the per-block partials
-    std::vector<double> sums(ng + 2, 0.0);
-    for (int b = 0; b < nvb; ++b)
-        for (int k = 0; k < ng + 2; ++k) sums[k] += part[(size_t)b * (ng + 2) + k];
-    double wI = 0.0;
-    for (int b = 0; b < npb; ++b) wI += part[(size_t)nvb * (ng + 2) + b];
+    if ((rc = check_cuda(h, cudaStreamSynchronize(h->stream), "stream synchronize"))) return rc;
+    if (sums[(size_t)ng + 3] != 0.0) return scatman_sync(h);      // reports and clears the error word
+    const double wI = sums[(size_t)ng + 2];
     // n, c = n^2 - 1 and their derivatives in delta, beta
     const double d = h->shape.delta, bb = h->shape.beta;
     const double nr = 1.0 - d, ni = bb;

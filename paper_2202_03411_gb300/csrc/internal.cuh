@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <list>
 #include <string>
 #include <vector>
 
@@ -291,6 +292,15 @@ struct scatman_handle {
     double *d_mdelta = nullptr, *d_mbeta = nullptr;
     size_t mindex_cap = 0;
     double str_re = 0, str_im = 0;  // global strength factor of s: n^2 - 1, or the map's index scale
+    // pinned staging of the last two map uploads, each free again once its event has passed
+    struct MapStage {
+        unsigned char *p = nullptr;
+        size_t cap = 0;
+        cudaEvent_t ev = nullptr;
+    } map_stage[2];
+    int map_turn = 0;
+    bool map_captured = false;      // the upload under way is being captured
+    std::list<std::vector<double>> captured_maps;
     double map_index_max = 0;       // max |delta|, |beta| over a volume map's cells
     bool on_grid = false;           // the field goes through its sample grid
     bool peak_direct = false;       // (fits in the tensor-core modes) except the pattern's peak
@@ -429,6 +439,9 @@ cudaError_t launch_grad_pixels(bool fp64, const void *A, const void *dLdI, long 
                                double *partials, int n_blocks, cudaStream_t st);
 int grad_pixel_blocks(long long n_pix);
 // Tensor-core adjoint field (adjoint_tc.cu).
+// out: nv voxel sums over nvb blocks, the pixel sum over npb, the error word (nv + 2 doubles).
+cudaError_t launch_grad_totals(const double *part, int nvb, int nv, int npb, const int *err, double *out,
+                               cudaStream_t st);
 bool adjoint_tc_supported(int nx, int ny);
 // nz: slices, or in order mode (orders != 0) the number N of Jacobi-Anger orders;
 // S receives the slices' (or orders') fields [nz][nx][ny].
