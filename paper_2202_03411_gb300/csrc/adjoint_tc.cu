@@ -66,7 +66,7 @@ struct AdjParams {
     int stages;
     int teams;                  // generator teams (1, 2 or 4; never more than stages)
     const float2 *A;            // forward field (FP32)
-    const float *w;             // dL/dI (null: 1)
+    const float *w;             // dL/dI (null: 1, and gmax_bits is the caller's)
     const unsigned *gmax_bits;  // max |w A| as float bits
     long long n_pix;
     int nx, ny, nz, Nyp;
@@ -419,7 +419,7 @@ __global__ void adj_gmax_kernel(const float2 *__restrict__ A, const float *__res
     float m = 0.f;
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
         const float2 a = A[p];
-        m = fmaxf(m, fabsf(w ? w[p] : 1.f) * sqrtf(a.x * a.x + a.y * a.y));
+        m = fmaxf(m, fabsf(w[p]) * sqrtf(a.x * a.x + a.y * a.y));
     }
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) atomicMax(gmax_bits, __float_as_uint(m));
@@ -507,9 +507,12 @@ cudaError_t launch_adjoint_tc(const float2 *A, const float *w, const float4 *tab
     P.partial = partial;
     P.nvox = (long long)nx * ny * nz;
     P.err = err;
-    cudaError_t e = cudaMemsetAsync(gmax_bits, 0, sizeof(unsigned), st);
-    if (e != cudaSuccess) return e;
-    adj_gmax_kernel<<<(unsigned)std::min<long long>((n_pix + 255) / 256, 1024), 256, 0, st>>>(A, w, n_pix, gmax_bits);
+    cudaError_t e;
+    if (w) {                                         // (with w null the caller has the largest |A|)
+        e = cudaMemsetAsync(gmax_bits, 0, sizeof(unsigned), st);
+        if (e != cudaSuccess) return e;
+        adj_gmax_kernel<<<(unsigned)std::min<long long>((n_pix + 255) / 256, 1024), 256, 0, st>>>(A, w, n_pix, gmax_bits);
+    }
     e = cudaFuncSetAttribute(adjoint_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
     if (e != cudaSuccess) return e;
     dim3 grid((nz + 1) / 2, splits);

@@ -1292,6 +1292,8 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
                 return rc;
         }
         if (tc_adjoint) {
+            if (!h->d_gmax && (rc = alloc_dev(h, (void **)&h->d_gmax, sizeof(unsigned), "adjoint scale"))) return rc;
+            h->fga.gmax = h->d_gmax;
             rc = check_cuda(h, launch_field_grid_gather(h->fg, h->fga, (const float2 *)h->d_A, (const float *)dLdI_dev,
                                                         h->stream),
                             "adjoint gather");

@@ -24,9 +24,9 @@
 // error over the whole box (plan_points below), not from the shape.
 //
 // Measured (forward pass with the voxeliser, against the direct sums): 128^3 on
-// 512^2 to 60 degrees, BF16 split phases 138 us (1798); 96^3 on 256^2, FP32
-// 51 us (5195), FP64 372 us (96705); 32^3 on 64^2, FP64 90 us (736); uniform-q
-// 30^3 on 512^2, FP32 59 us (125, the separable sums per pixel row).
+// 512^2 to 60 degrees, BF16 split phases 74 us (1798); 96^3 on 256^2, FP32
+// 28 us (5195), FP64 164 us (73600, the same ellipsoid); 32^3 on 64^2, FP64 31 us
+// (736); uniform-q 30^3 on 512^2, FP32 29 us (125, the separable sums per pixel row).
 #include <cmath>
 #include <complex>
 
@@ -131,18 +131,28 @@ bool plan_field_grid(const scatman_config &c, bool fp64, FieldGrid *f) {
 // Whether a handle of this configuration computes its field on the sample
 // grid.  Not with a list of q (no detector), nor in the single-product modes
 // and the tensor-core uniform-q detector (their 16-bit roundings belong to the
-// pixel and to the row), nor where the direct sums are as fast.  Forward pass,
-// 45 degrees, wavelength 8, grid / direct: FP32 21 / 28 us already at 16^3 voxels
-// and 12^2 pixels, 27 / 294 us at 48^3 / 128^2; FP64 60 / 303 and 103 / 5759 us.
-// Split phases on the tensor cores: 35 / 36 us at 48^3 / 128^2, 36 / 46 us at
-// 64^3 / 128^2, 45 / 39 us at 96^3 / 64^2, 48 / 277 us at 96^3 / 256^2.
+// pixel and to the row), nor where the direct sums are as fast.  FP32 and FP64:
+// already at 16^3 voxels and 12^2 pixels.  Split phases on the tensor cores (45
+// degrees, wavelength 8, ellipsoid, forward pass, grid / direct in us): 29 / 28 at
+// 48^3 on 64^2, 29 / 32 on 96^2, 29 / 34 on 128^2; 35 / 36 at 64^3 on 64^2, 33 / 46 on
+// 128^2; 48 / 47 at 96^3 on 64^2, 46 / 56 on 96^2; and where the grid has more points
+// than the detector has pixels (60 degrees, wavelength 6) 58 / 47 at 96^3 on 64^2,
+// 68 / 84 at 128^3 on 96^2.
+// Fits in the split phases keep their pattern's peak on the direct sums
+// (api.cu), and a small problem's other pixels too: the gradient of a nearly
+// cancelling loss sees their rounding (3e-5 at 64^3 on 128^2).
 bool use_field_grid(const scatman_config &c, FieldGrid *f) {
     const bool split = c.precision == SCATMAN_TC_F16_SPLIT || c.precision == SCATMAN_TC_BF16_SPLIT;
     const bool plain = c.precision == SCATMAN_FP64 || c.precision == SCATMAN_FP32;
     if (c.q_list || !(plain || (split && c.detector == SCATMAN_DETECTOR_FLAT))) return false;
     const double pixels = (double)c.det_nx * c.det_ny, terms = pixels * ((double)c.nx * c.ny * c.nz);
-    if (plain ? pixels < 128.0 : terms < 2.5e9) return false;
-    return plan_field_grid(c, c.precision == SCATMAN_FP64, f);
+    if (plain ? pixels < 128.0 : terms < (c.soft ? 2e10 : 5e8)) return false;
+    if (!plan_field_grid(c, c.precision == SCATMAN_FP64, f)) return false;
+    if (split && terms < 8e9 && pixels < 2.4 * f->Hs * f->Ht) return false;
+    // FP32 fits: a loss near its minimum shows the pattern's rounding many times
+    // larger.  Dot2 sums halve it, at ten FP32 operations a term instead of one.
+    f->dot2 = c.precision == SCATMAN_FP32 && c.soft;
+    return true;
 }
 
 // Whether the adjoint runs through the grid.  In the tensor-core modes it pays
@@ -179,7 +189,7 @@ size_t field_grid_layout(FieldGrid *f, bool tensor_core, int Nxp, unsigned char 
     const size_t row = (size_t)(tensor_core && Nxp > f->nx ? Nxp : f->nx);
     f->H = take(2 * (size_t)f->Hs * f->nz * row * 2 * e);
     f->Q = take((size_t)f->jc * f->Hs * f->Ht * 8 * e);
-    f->B = take((size_t)f->H2 * 8 * f->n1 * e);
+    f->B = take((size_t)f->H2 * 8 * ((f->n1 + 31) / 32 * 32) * e);
     f->bytes = at;
     return at;
 }
@@ -350,12 +360,12 @@ __global__ void fg_pixels_kernel(FieldGrid f) {
     }
     V4 e = fg_square<R>(x, (R)x, (R)0);
     const V4 *nd = (const V4 *)f.node2;
-    R D = (R)0;
+    R D = (R)0, low = (R)0;
     for (int a = 0; a < f.H2; ++a) {
         const V4 n = nd[a];
-        D += n.z * fg_recip(e.x, e.y, n.x, n.y);
+        fg_dot2(n.z, fg_recip(e.x, e.y, n.x, n.y), D, low);
     }
-    e.w = (R)1 / D;
+    e.w = (R)1 / (D + low);
     if (!valid) e.z = (R)__longlong_as_double(0x7ff8000000000000ll);
     ((V4 *)f.pix)[(size_t)v * f.U + i] = e;
 }
@@ -378,13 +388,19 @@ cudaError_t launch_field_grid_tables(const FieldGrid &f, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// Rows per thread whose tiles of 8 kRpt waste least on n rows.
-static int fg_rows_per_thread(int n) {
-    int best = 3, waste = 1 << 30;
-    for (int r : {6, 5, 3}) {
-        const int w = (n + 8 * r - 1) / (8 * r) * 8 * r;
-        if (w < waste) {
-            waste = w;
+// Rows per thread (tiles of 8 kRpt of n rows) on a grid of `others` blocks per row
+// tile: the fewest rounds over the SMs times a block's work, its rows and the
+// loads it makes whatever their number (worth three rows in FP32, half a row in
+// FP64, whose arithmetic takes the time).  FP64 32^3 on 64^2: 36 blocks of 24 rows
+// took 21 us, 108 of 8 rows take 8; larger grids keep five or six rows.
+static int fg_rows_per_thread(int n, long long others, bool fp64, int sm_count) {
+    int best = 3;
+    double cost = 1e300;
+    for (int r : {6, 5, 3, 2, 1}) {
+        const long long blocks = others * ((n + 8 * r - 1) / (8 * r));
+        const double c = (double)((blocks + sm_count - 1) / sm_count) * (r + (fp64 ? 0.5 : 3.0));
+        if (c < 0.95 * cost) {
+            cost = c;
             best = r;
         }
     }
@@ -401,6 +417,7 @@ __global__ void __launch_bounds__(kFgThreads) fg_y_kernel(FieldGrid f, const typ
     extern __shared__ __align__(32) unsigned char smem[];
     FgTile<R, kRpt> &t = *reinterpret_cast<FgTile<R, kRpt> *>(smem);
     const int j = blockIdx.y, x0 = blockIdx.x * 32, a0 = blockIdx.z * 8 * kRpt;
+    pdl_wait();
     const int xlo = bounds[j], xhi = bounds[f.nz + j], ylo = bounds[2 * f.nz + j], yhi = bounds[3 * f.nz + j];
     if (xlo >= xhi || x0 >= xhi || x0 + 32 <= xlo) return;
     const int grp = threadIdx.x >> 7, tt = threadIdx.x & 127, cg = tt & 15, bg = tt >> 4;
@@ -410,30 +427,51 @@ __global__ void __launch_bounds__(kFgThreads) fg_y_kernel(FieldGrid f, const typ
     const int kbeg = max(0, max(ylo - f.ny / 2, (f.ny - 1) / 2 - (yhi - 1))) & ~(kFgK - 1);
     const R *cy = (const R *)f.ty, *sy = cy + (size_t)f.Ky * f.Hs;
     R acc[kRpt][4] = {};
-    for (int k0 = kbeg; k0 < kend; k0 += kFgK) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < kFgK * 8 * kRpt; i += kFgThreads) {
-            const int k = i / (8 * kRpt), a = i % (8 * kRpt);
+    // one tile's operands on their way from memory
+    R tc[kRpt], ts[kRpt];
+    C sp[4], sm[4];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < kRpt; ++q) {
+            const int i = threadIdx.x + q * kFgThreads, k = i / (8 * kRpt), a = i % (8 * kRpt);
             const bool in = k0 + k < kend && a0 + a < f.Hs;
-            t.T[0][k][a] = in ? cy[(size_t)(k0 + k) * f.Hs + a0 + a] : (R)0;
-            t.T[1][k][a] = in ? sy[(size_t)(k0 + k) * f.Hs + a0 + a] : (R)0;
+            tc[q] = in ? cy[(size_t)(k0 + k) * f.Hs + a0 + a] : (R)0;
+            ts[q] = in ? sy[(size_t)(k0 + k) * f.Hs + a0 + a] : (R)0;
         }
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            const int xl = warp * 4 + c, x = x0 + xl, k = k0 + lane;
-            C p, m;
-            p.x = p.y = m.x = m.y = (R)0;
+            const int x = x0 + warp * 4 + c, k = k0 + lane;
+            sp[c].x = sp[c].y = sm[c].x = sm[c].y = (R)0;
             if (x < f.nx && k < kend) {
                 const C *line = s + ((size_t)j * f.nx + x) * f.ny;
                 const int ip = fg_plus(k, f.ny), im = fg_minus(k, f.ny);
-                p = line[ip];
-                if (im != ip) m = line[im];
+                sp[c] = line[ip];
+                if (im != ip) sm[c] = line[im];
             }
-            t.S[0][lane][2 * xl] = p.x + m.x;
-            t.S[0][lane][2 * xl + 1] = p.y + m.y;
-            t.S[1][lane][2 * xl] = p.x - m.x;
-            t.S[1][lane][2 * xl + 1] = p.y - m.y;
         }
+    };
+    auto store = [&]() {
+#pragma unroll
+        for (int q = 0; q < kRpt; ++q) {
+            const int i = threadIdx.x + q * kFgThreads, k = i / (8 * kRpt), a = i % (8 * kRpt);
+            t.T[0][k][a] = tc[q];
+            t.T[1][k][a] = ts[q];
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int xl = warp * 4 + c;
+            t.S[0][lane][2 * xl] = sp[c].x + sm[c].x;
+            t.S[0][lane][2 * xl + 1] = sp[c].y + sm[c].y;
+            t.S[1][lane][2 * xl] = sp[c].x - sm[c].x;
+            t.S[1][lane][2 * xl + 1] = sp[c].y - sm[c].y;
+        }
+    };
+    // (a tile's loads all in flight before the first is used; fetching the next
+    // tile under this one's products as well gained nothing)
+    for (int k0 = kbeg; k0 < kend; k0 += kFgK) {
+        load(k0);
+        __syncthreads();
+        store();
         __syncthreads();
         fg_multiply<R, kRpt>(t, grp, bg, cg, min(kFgK, kend - k0), acc);
     }
@@ -473,12 +511,22 @@ __global__ void __launch_bounds__(kFgThreads) fg_xz_kernel(FieldGrid f, int Nxp,
     extern __shared__ __align__(32) unsigned char smem[];
     FgTile<R, kRpt> &t = *reinterpret_cast<FgTile<R, kRpt> *>(smem);
     __shared__ int s_lo[kFgSlices], s_hi[kFgSlices];
+    __shared__ uint32_t s_live[kFgSlices];              // the occupied 8-column chunks, a bit each
     const int a = blockIdx.x, j0 = blockIdx.y * kFgSlices, b0 = blockIdx.z * 8 * kRpt;
     const int grp = threadIdx.x >> 7, tt = threadIdx.x & 127, cg = tt & 15, bg = tt >> 4;
+    pdl_wait();
     if (threadIdx.x < kFgSlices) {
         const int j = j0 + threadIdx.x;
         s_lo[threadIdx.x] = j < f.nz ? bounds[j] : 0x7fffffff;
         s_hi[threadIdx.x] = j < f.nz ? bounds[f.nz + j] : 0;
+    }
+    if (kPm) {
+        for (int jl = threadIdx.x >> 5; jl < kFgSlices; jl += kFgThreads / 32) {
+            const int c = (j0 + jl) * kGeomChunks + (threadIdx.x & 31);
+            const bool live = j0 + jl < f.nz && chunk_y[c] < chunk_y[kGeomChunks * f.nz + c];
+            const uint32_t m = __ballot_sync(0xffffffffu, live);
+            if ((threadIdx.x & 31) == 0) s_live[jl] = m;
+        }
     }
     __syncthreads();
     int kend = 0;
@@ -489,39 +537,58 @@ __global__ void __launch_bounds__(kFgThreads) fg_xz_kernel(FieldGrid f, int Nxp,
     const R *cx = (const R *)f.tx + (size_t)a * f.Kx * f.Ht, *sx = cx + (size_t)f.Hs * f.Kx * f.Ht;
     const C *H = (const C *)f.H;
     R acc[kRpt][4] = {};
-    for (int k0 = 0; k0 < kend; k0 += kFgK) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < kFgK * 8 * kRpt; i += kFgThreads) {
-            const int k = i / (8 * kRpt), b = i % (8 * kRpt);
+    // one tile's operands on their way from memory: the phases, and of two
+    // (slice, x') the values of both parts at +x and -x
+    R tc[kRpt], ts[kRpt];
+    C he[2][2], ho[2][2];
+    static_assert(kFgSlices * kFgK == 2 * kFgThreads, "two per thread");
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < kRpt; ++q) {
+            const int i = threadIdx.x + q * kFgThreads, k = i / (8 * kRpt), b = i % (8 * kRpt);
             const bool in = k0 + k < kend && b0 + b < f.Ht;
-            t.T[0][k][b] = in ? cx[(size_t)(k0 + k) * f.Ht + b0 + b] : (R)0;
-            t.T[1][k][b] = in ? sx[(size_t)(k0 + k) * f.Ht + b0 + b] : (R)0;
+            tc[q] = in ? cx[(size_t)(k0 + k) * f.Ht + b0 + b] : (R)0;
+            ts[q] = in ? sx[(size_t)(k0 + k) * f.Ht + b0 + b] : (R)0;
         }
-        for (int i = threadIdx.x; i < kFgSlices * kFgK; i += kFgThreads) {
-            const int jl = i / kFgK, k = i % kFgK, j = j0 + jl;
-            C e[2], o[2];                               // at +x, -x
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int i = threadIdx.x + q * kFgThreads, jl = i / kFgK, k = i % kFgK, j = j0 + jl;
 #pragma unroll
             for (int m = 0; m < 2; ++m) {
                 const int x = m == 0 ? fg_plus(k0 + k, f.nx) : fg_minus(k0 + k, f.nx);
                 bool live = k0 + k < kend && x >= s_lo[jl] && x < s_hi[jl];
-                if (kPm && live) {
-                    // the tensor-core sum writes the occupied 8-column chunks only
-                    const int c = j * kGeomChunks + (x >> 3);
-                    live = chunk_y[c] < chunk_y[kGeomChunks * f.nz + c];
-                }
+                // the tensor-core sum writes the occupied 8-column chunks only
+                if (kPm && live) live = (s_live[jl] >> (x >> 3)) & 1u;
                 if (m == 1 && x == fg_plus(k0 + k, f.nx)) live = false;        // the middle of an odd side counts once
-                e[m].x = e[m].y = o[m].x = o[m].y = (R)0;
+                he[q][m].x = he[q][m].y = ho[q][m].x = ho[q][m].y = (R)0;
                 if (live) {
-                    if (kPm) {
-                        const C p = H[((size_t)a * f.nz + j) * Nxp + x], n = H[((size_t)(f.Hs + a) * f.nz + j) * Nxp + x];
-                        e[m].x = (R)0.5 * (p.x + n.x);
-                        e[m].y = (R)0.5 * (p.y + n.y);
-                        o[m].x = (R)0.5 * (p.x - n.x);
-                        o[m].y = (R)0.5 * (p.y - n.y);
-                    } else {
-                        e[m] = H[(((size_t)a * 2) * f.nz + j) * f.nx + x];
-                        o[m] = H[(((size_t)a * 2 + 1) * f.nz + j) * f.nx + x];
-                    }
+                    he[q][m] = kPm ? H[((size_t)a * f.nz + j) * Nxp + x] : H[(((size_t)a * 2) * f.nz + j) * f.nx + x];
+                    ho[q][m] = kPm ? H[((size_t)(f.Hs + a) * f.nz + j) * Nxp + x]
+                                   : H[(((size_t)a * 2 + 1) * f.nz + j) * f.nx + x];
+                }
+            }
+        }
+    };
+    auto store = [&]() {
+#pragma unroll
+        for (int q = 0; q < kRpt; ++q) {
+            const int i = threadIdx.x + q * kFgThreads, k = i / (8 * kRpt), b = i % (8 * kRpt);
+            t.T[0][k][b] = tc[q];
+            t.T[1][k][b] = ts[q];
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int i = threadIdx.x + q * kFgThreads, jl = i / kFgK, k = i % kFgK;
+            C e[2], o[2];                               // at +x, -x
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                e[m] = he[q][m];
+                o[m] = ho[q][m];
+                if (kPm) {
+                    e[m].x = (R)0.5 * (he[q][m].x + ho[q][m].x);
+                    e[m].y = (R)0.5 * (he[q][m].y + ho[q][m].y);
+                    o[m].x = (R)0.5 * (he[q][m].x - ho[q][m].x);
+                    o[m].y = (R)0.5 * (he[q][m].y - ho[q][m].y);
                 }
             }
             V4 v;
@@ -536,6 +603,11 @@ __global__ void __launch_bounds__(kFgThreads) fg_xz_kernel(FieldGrid f, int Nxp,
             v.w = o[0].y - o[1].y;
             *reinterpret_cast<V4 *>(&t.S[1][k][4 * jl]) = v;
         }
+    };
+    for (int k0 = 0; k0 < kend; k0 += kFgK) {
+        load(k0);
+        __syncthreads();
+        store();
         __syncthreads();
         fg_multiply<R, kRpt>(t, grp, bg, cg, min(kFgK, kend - k0), acc);
     }
@@ -571,91 +643,121 @@ __global__ void __launch_bounds__(kFgThreads) fg_xz_kernel(FieldGrid f, int Nxp,
     }
 }
 
+// Place of value c (see fg_columns_kernel) of column (row) i at point p2 in B: the
+// pixel kernel's shared-memory tile, in one piece per tile: 32 columns [point][8][32],
+// on the uniform-q detector 4 rows [point][4][8].
+__device__ __forceinline__ size_t fg_B_at(const FieldGrid &f, int p2, int c, int i) {
+    return f.uniform ? ((size_t)(i >> 2) * f.H2 + p2) * 32 + (i & 3) * 8 + c
+                     : ((size_t)(i >> 5) * f.H2 + p2) * 256 + c * 32 + (i & 31);
+}
+
 // Interpolation along the per-column (per-row) direction, after adding the
-// slice chunks: B[point 2][parity 1 x parity 2][i], with the constants of the
+// slice chunks: B of 32 columns at one point of the per-pixel direction, values
+// [2 parity 1 + parity 2] x (re, im), with the constants of the
 // per-pixel direction's points folded in (c_a x_a on even parts, c_a on odd).
+// The points are split over eight warps: the sums are short and wait for their
+// loads, so the launch is as long as the longest chain of them.
 template <typename R>
-__global__ void __launch_bounds__(128) fg_columns_kernel(FieldGrid f) {
+__global__ void __launch_bounds__(256) fg_columns_kernel(FieldGrid f) {
     using V4 = typename Fg<R>::V4;
     extern __shared__ __align__(32) unsigned char smem[];
     R *q = reinterpret_cast<R *>(smem);                 // [point 1][8]
-    const int p2 = blockIdx.y;
+    __shared__ R part[8][8][32];
+    const int p2 = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
     const size_t chunk = (size_t)f.Hs * f.Ht * 8;
-    for (int i = threadIdx.x; i < f.H1 * 8; i += blockDim.x) {
-        const int p1 = i >> 3, c = i & 7;
+    pdl_wait();
+    for (int k = threadIdx.x; k < f.H1 * 8; k += blockDim.x) {
+        const int p1 = k >> 3, c = k & 7;
         const int a = f.uniform ? p1 : p2, b = f.uniform ? p2 : p1;
         const R *src = (const R *)f.Q + ((size_t)a * f.Ht + b) * 8 + c;
         R v = (R)0;
+#pragma unroll 8
         for (int j = 0; j < f.jc; ++j) v += src[j * chunk];
         // first parity = that of direction 1: t on the flat detector, s on the uniform-q one
         const int pq = c >> 1, d = f.uniform ? pq : ((pq & 1) << 1) | (pq >> 1);
         q[p1 * 8 + 2 * d + (c & 1)] = v;
     }
     __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= f.n1) return;
     const R *we = (const R *)f.w1, *wo = we + (size_t)f.H1 * f.n1;
     R acc[8] = {};
-#pragma unroll 4
-    for (int p = 0; p < f.H1; ++p) {
-        const R e = we[(size_t)p * f.n1 + i], o = wo[(size_t)p * f.n1 + i];
-        const V4 a = *reinterpret_cast<const V4 *>(q + p * 8), b = *reinterpret_cast<const V4 *>(q + p * 8 + 4);
-        acc[0] = fma(e, a.x, acc[0]);
-        acc[1] = fma(e, a.y, acc[1]);
-        acc[2] = fma(e, a.z, acc[2]);
-        acc[3] = fma(e, a.w, acc[3]);
-        acc[4] = fma(o, b.x, acc[4]);
-        acc[5] = fma(o, b.y, acc[5]);
-        acc[6] = fma(o, b.z, acc[6]);
-        acc[7] = fma(o, b.w, acc[7]);
-    }
-    const V4 n = ((const V4 *)f.node2)[p2];
-    // after direction 1 the parities of direction 1 only tell the two mirrored
-    // columns apart: [2 d1 + d2], d2 the per-pixel direction's parity
+    if (sizeof(R) == 4 && f.dot2) {
+        R low[8] = {};
+        for (int p = warp; i < f.n1 && p < f.H1; p += 8) {
+            const R e = we[(size_t)p * f.n1 + i], o = wo[(size_t)p * f.n1 + i];
 #pragma unroll
-    for (int c = 0; c < 8; ++c)
-        ((R *)f.B)[((size_t)p2 * 8 + c) * f.n1 + i] = acc[c] * (((c >> 1) & 1) ? n.w : n.z);
+            for (int c = 0; c < 8; ++c) fg_dot2(c < 4 ? e : o, q[p * 8 + c], acc[c], low[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[c] += low[c];
+    } else if (i < f.n1) {
+#pragma unroll 4
+        for (int p = warp; p < f.H1; p += 8) {
+            const R e = we[(size_t)p * f.n1 + i], o = wo[(size_t)p * f.n1 + i];
+            const V4 a = *reinterpret_cast<const V4 *>(q + p * 8), b = *reinterpret_cast<const V4 *>(q + p * 8 + 4);
+            acc[0] = fma(e, a.x, acc[0]);
+            acc[1] = fma(e, a.y, acc[1]);
+            acc[2] = fma(e, a.z, acc[2]);
+            acc[3] = fma(e, a.w, acc[3]);
+            acc[4] = fma(o, b.x, acc[4]);
+            acc[5] = fma(o, b.y, acc[5]);
+            acc[6] = fma(o, b.z, acc[6]);
+            acc[7] = fma(o, b.w, acc[7]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) part[warp][c][lane] = acc[c];
+    __syncthreads();
+    const int c = warp;                                 // this thread's value
+    R v = part[0][c][lane];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) v += part[w][c][lane];
+    const V4 n = ((const V4 *)f.node2)[p2];
+    // (columns past the last one are zero: the tiles are whole)
+    ((R *)f.B)[fg_B_at(f, p2, c, i)] = v * (((c >> 1) & 1) ? n.w : n.z);
 }
 
 // Field and intensity of the pixels: a thread interpolates kPts quadruples of
 // mirrored pixels, sharing the loads of B (flat: kPts rows of one column; uniform:
-// kPts columns of one row).
-template <typename R, int kPts, bool kUniform>
-__global__ void __launch_bounds__(128) fg_pixels_out_kernel(FieldGrid f, R str_re, R str_im,
+// kPts columns of one row).  A block's part of B (43 KB for 42 points) is one
+// piece of memory, copied with all its loads in flight.
+// kSplit (small detectors in FP64, of which a warp runs an operation in 64 cycles): the
+// four warps share one row, each takes a quarter of the points, a quarter of the
+// sums and one of the four mirrored pixels (32^3 on 64^2: 16 us with a warp per row).
+template <typename R, int kPts, bool kUniform, int kWarps, bool kDot2, bool kSplit>
+__global__ void __launch_bounds__(32 * kWarps) fg_pixels_out_kernel(FieldGrid f, double str_re, double str_im,
                                                             typename Fg<R>::C *__restrict__ A, R *__restrict__ I) {
     using C = typename Fg<R>::C;
     using V4 = typename Fg<R>::V4;
+    static_assert(!kUniform || kWarps == 4, "a warp per row");
+    using S = typename std::conditional<kDot2, double, R>::type;      // of the last few operations per pixel
     extern __shared__ __align__(32) unsigned char smem[];
     R *sB = reinterpret_cast<R *>(smem);
     V4 *sN = reinterpret_cast<V4 *>(sB + (size_t)f.H2 * 8 * (kUniform ? 4 : 32));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // flat: 32 columns x 4 warps x kPts rows; uniform: 4 rows (one per warp) x 32 kPts columns
-    const int first = kUniform ? blockIdx.y * 4 : blockIdx.x * 32;
-    const int width = kUniform ? 4 : 32;
-    for (int k = threadIdx.x; k < f.H2 * 8 * width; k += 128) {
-        const int i = k % width, r = k / width;
-        const R v = first + i < f.n1 ? ((const R *)f.B)[(size_t)r * f.n1 + first + i] : (R)0;
-        if (kUniform)
-            sB[((r >> 3) * 4 + i) * 8 + (r & 7)] = v;   // [point][row][8]
-        else
-            sB[k] = v;                                  // [point][8][column]
-    }
-    for (int k = threadIdx.x; k < f.H2; k += 128) sN[k] = ((const V4 *)f.node2)[k];
+    // flat: 32 columns x kWarps warps x kPts rows; uniform: 4 rows (one per warp) x 32 kPts columns
+    const int tile = kUniform ? blockIdx.y : blockIdx.x;
+    const int count = f.H2 * 8 * (kUniform ? 4 : 32);
+    for (int k = threadIdx.x; k < f.H2; k += 32 * kWarps) sN[k] = ((const V4 *)f.node2)[k];
+    pdl_wait();
+    const R *src = (const R *)f.B + (size_t)tile * count;
+    for (int k = threadIdx.x * (16 / sizeof(R)); k < count; k += 32 * kWarps * (16 / sizeof(R)))
+        cp_async16(sB + k, src + k);
+    cp_async_wait_all();
     __syncthreads();
     int u[kPts], v[kPts];
     V4 px[kPts];
-    R acc[kPts][8];
+    R acc[kPts][8], low[kPts][8];
 #pragma unroll
     for (int p = 0; p < kPts; ++p) {
         u[p] = kUniform ? (blockIdx.x * kPts + p) * 32 + lane : blockIdx.x * 32 + lane;
-        v[p] = kUniform ? blockIdx.y * 4 + warp : (blockIdx.y * 4 + warp) * kPts + p;
+        v[p] = kSplit ? blockIdx.y : kUniform ? blockIdx.y * 4 + warp : (blockIdx.y * kWarps + warp) * kPts + p;
         px[p].x = px[p].y = px[p].z = px[p].w = (R)0;
         if (u[p] < f.U && v[p] < f.V) px[p] = ((const V4 *)f.pix)[(size_t)v[p] * f.U + u[p]];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) acc[p][c] = (R)0;
+        for (int c = 0; c < 8; ++c) acc[p][c] = low[p][c] = (R)0;
     }
 #pragma unroll 2
-    for (int a = 0; a < f.H2; ++a) {
+    for (int a = kSplit ? warp : 0; a < f.H2; a += kSplit ? kWarps : 1) {
         const V4 n = sN[a];
         R b[8];
         if (kUniform) {
@@ -677,21 +779,42 @@ __global__ void __launch_bounds__(128) fg_pixels_out_kernel(FieldGrid f, R str_r
         for (int p = 0; p < kPts; ++p) {
             const R r = fg_recip(px[p].x, px[p].y, n.x, n.y);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) acc[p][c] = fma(r, b[c], acc[p][c]);
+            for (int c = 0; c < 8; ++c) {
+                if (kDot2)
+                    fg_dot2(r, b[c], acc[p][c], low[p][c]);
+                else
+                    acc[p][c] = fma(r, b[c], acc[p][c]);
+            }
         }
+    }
+    if constexpr (kSplit) {
+        static_assert(kPts == 1 && kWarps == 4 && !kUniform && !kDot2, "a quarter each");
+        __shared__ R part[4][8][32];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) part[warp][c][lane] = acc[0][c];
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            R *q = &part[0][2 * warp + c][lane];
+            q[0] = (q[0] + q[8 * 32]) + (q[2 * 8 * 32] + q[3 * 8 * 32]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[0][c] = part[0][c][lane];
     }
 #pragma unroll
     for (int p = 0; p < kPts; ++p) {
         if (u[p] >= f.U || v[p] >= f.V) continue;
         const bool off = !(px[p].z == px[p].z);          // no scattering direction: A = 0
-        const R we = px[p].w, wo = px[p].w * px[p].z;
+        const S we = px[p].w, wo = (S)px[p].w * px[p].z;
         // [2 d1 + d2]: combine the per-pixel direction's parities, then the other's
-        R g[2][4];                                       // [sign of direction 2][parity 1][re, im]
+        S g[2][4];                                       // [sign of direction 2][parity 1][re, im]
 #pragma unroll
         for (int d1 = 0; d1 < 2; ++d1)
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
-                const R e = we * acc[p][4 * d1 + c], o = wo * acc[p][4 * d1 + 2 + c];
+                const int k = 4 * d1 + c;
+                const S e = we * ((S)acc[p][k] + low[p][k]), o = wo * ((S)acc[p][k + 2] + low[p][k + 2]);
                 g[0][2 * d1 + c] = e + o;
                 g[1][2 * d1 + c] = e - o;
             }
@@ -699,17 +822,20 @@ __global__ void __launch_bounds__(128) fg_pixels_out_kernel(FieldGrid f, R str_r
         for (int m2 = 0; m2 < 2; ++m2)
 #pragma unroll
             for (int m1 = 0; m1 < 2; ++m1) {
+                if (kSplit && warp != 2 * m2 + m1) continue;
                 const int mu = kUniform ? m2 : m1, mv = kUniform ? m1 : m2;
                 const int iu = mu ? fg_minus(u[p], f.det_nx) : fg_plus(u[p], f.det_nx);
                 const int iv = mv ? fg_minus(v[p], f.det_ny) : fg_plus(v[p], f.det_ny);
-                const R re = m1 ? g[m2][0] - g[m2][2] : g[m2][0] + g[m2][2];
-                const R im = m1 ? g[m2][1] - g[m2][3] : g[m2][1] + g[m2][3];
-                C o;
-                o.x = off ? (R)0 : str_re * re - str_im * im;
-                o.y = off ? (R)0 : str_re * im + str_im * re;
+                const S re = m1 ? g[m2][0] - g[m2][2] : g[m2][0] + g[m2][2];
+                const S im = m1 ? g[m2][1] - g[m2][3] : g[m2][1] + g[m2][3];
+                const S ox = off ? (S)0 : (S)str_re * re - (S)str_im * im;
+                const S oy = off ? (S)0 : (S)str_re * im + (S)str_im * re;
                 const size_t at = (size_t)iv * f.det_nx + iu;
+                C o;
+                o.x = (R)ox;
+                o.y = (R)oy;
                 A[at] = o;
-                I[at] = o.x * o.x + o.y * o.y;
+                I[at] = (R)(ox * ox + oy * oy);
             }
     }
 }
@@ -724,8 +850,7 @@ static cudaError_t fg_run_y(const FieldGrid &f, const void *s, const int *bounds
     cudaError_t e = fg_smem(fg_y_kernel<R, kRpt>, smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((f.nx + 31) / 32, f.nz, (f.Hs + 8 * kRpt - 1) / (8 * kRpt));
-    fg_y_kernel<R, kRpt><<<grid, kFgThreads, smem, st>>>(f, (const typename Fg<R>::C *)s, bounds);
-    return cudaGetLastError();
+    return launch_pdl(fg_y_kernel<R, kRpt>, grid, dim3(kFgThreads), smem, st, f, (const typename Fg<R>::C *)s, bounds);
 }
 
 template <typename R, int kRpt, bool kPm>
@@ -734,73 +859,88 @@ static cudaError_t fg_run_xz(const FieldGrid &f, int Nxp, const int *bounds, con
     cudaError_t e = fg_smem(fg_xz_kernel<R, kRpt, kPm>, smem);
     if (e != cudaSuccess) return e;
     const dim3 grid(f.Hs, f.jc, (f.Ht + 8 * kRpt - 1) / (8 * kRpt));
-    fg_xz_kernel<R, kRpt, kPm><<<grid, kFgThreads, smem, st>>>(f, Nxp, bounds, chunk_y);
-    return cudaGetLastError();
+    return launch_pdl(fg_xz_kernel<R, kRpt, kPm>, grid, dim3(kFgThreads), smem, st, f, Nxp, bounds, chunk_y);
 }
 
-template <typename R, int kPts, bool kUniform>
+template <typename R, int kPts, bool kUniform, int kWarps, bool kDot2 = false, bool kSplit = false>
 static cudaError_t fg_run_pixels(const FieldGrid &f, double str_re, double str_im, void *A, void *I, cudaStream_t st) {
     using V4 = typename Fg<R>::V4;
     const size_t smem = (size_t)f.H2 * 8 * (kUniform ? 4 : 32) * sizeof(R) + (size_t)f.H2 * sizeof(V4);
     // the largest size any plan uses, so concurrent launches of other handles stay valid
     const size_t most = (size_t)fg_max_half(sizeof(R) == 8) * (8 * (kUniform ? 4 : 32) * sizeof(R) + sizeof(V4));
-    const auto k = fg_pixels_out_kernel<R, kPts, kUniform>;
+    const auto k = fg_pixels_out_kernel<R, kPts, kUniform, kWarps, kDot2, kSplit>;
     cudaError_t e = fg_smem(k, most);
     if (e != cudaSuccess) return e;
     const dim3 grid = kUniform ? dim3((f.U + 32 * kPts - 1) / (32 * kPts), (f.V + 3) / 4)
-                               : dim3((f.U + 31) / 32, (f.V + 4 * kPts - 1) / (4 * kPts));
-    k<<<grid, 128, smem, st>>>(f, (R)str_re, (R)str_im, (typename Fg<R>::C *)A, (R *)I);
-    return cudaGetLastError();
+                 : kSplit ? dim3((f.U + 31) / 32, f.V)
+                          : dim3((f.U + 31) / 32, (f.V + kWarps * kPts - 1) / (kWarps * kPts));
+    return launch_pdl(k, grid, dim3(32 * kWarps), smem, st, f, str_re, str_im, (typename Fg<R>::C *)A, (R *)I);
 }
 
 template <typename R>
 static cudaError_t fg_finish(const FieldGrid &f, double str_re, double str_im, void *A, void *I, int sm_count,
                              cudaStream_t st) {
-    fg_columns_kernel<R><<<dim3((f.n1 + 127) / 128, f.H2), 128, (size_t)f.H1 * 8 * sizeof(R), st>>>(f);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(fg_columns_kernel<R>, dim3((f.n1 + 31) / 32, f.H2), dim3(256),
+                               (size_t)f.H1 * 8 * sizeof(R), st, f);
     if (e != cudaSuccess) return e;
-    // more pixels per thread share the loads of B; fewer fill the SMs on small detectors
+    // more pixels per thread share the loads of B on large detectors; on small
+    // ones fewer rows per block fill the SMs
     const long long blocks = (long long)f.U * f.V / 128;
-    if (blocks >= 8ll * sm_count)
-        return f.uniform ? fg_run_pixels<R, 4, true>(f, str_re, str_im, A, I, st)
-                         : fg_run_pixels<R, 4, false>(f, str_re, str_im, A, I, st);
-    if (blocks >= 2ll * sm_count)
-        return f.uniform ? fg_run_pixels<R, 2, true>(f, str_re, str_im, A, I, st)
-                         : fg_run_pixels<R, 2, false>(f, str_re, str_im, A, I, st);
-    return f.uniform ? fg_run_pixels<R, 1, true>(f, str_re, str_im, A, I, st)
-                     : fg_run_pixels<R, 1, false>(f, str_re, str_im, A, I, st);
+    if (sizeof(R) == 4 && f.dot2)
+        return f.uniform                  ? fg_run_pixels<R, 1, true, 4, true>(f, str_re, str_im, A, I, st)
+               : blocks >= 2ll * sm_count ? fg_run_pixels<R, 1, false, 8, true>(f, str_re, str_im, A, I, st)
+                                          : fg_run_pixels<R, 1, false, 4, true>(f, str_re, str_im, A, I, st);
+    if (f.uniform)
+        return blocks >= 8ll * sm_count   ? fg_run_pixels<R, 4, true, 4>(f, str_re, str_im, A, I, st)
+               : blocks >= 2ll * sm_count ? fg_run_pixels<R, 2, true, 4>(f, str_re, str_im, A, I, st)
+                                          : fg_run_pixels<R, 1, true, 4>(f, str_re, str_im, A, I, st);
+    return blocks >= 8ll * sm_count   ? fg_run_pixels<R, 4, false, 4>(f, str_re, str_im, A, I, st)
+           : blocks >= 2ll * sm_count ? fg_run_pixels<R, 1, false, 8>(f, str_re, str_im, A, I, st)
+           : 2 * blocks >= sm_count   ? fg_run_pixels<R, 1, false, 4>(f, str_re, str_im, A, I, st)
+           : sizeof(R) == 8           ? fg_run_pixels<R, 1, false, 4, false, true>(f, str_re, str_im, A, I, st)
+                                      : fg_run_pixels<R, 1, false, 1>(f, str_re, str_im, A, I, st);
+}
+
+template <typename R>
+static cudaError_t fg_sum_y(const FieldGrid &f, const void *s, const int *bounds, int sm_count, cudaStream_t st) {
+    switch (fg_rows_per_thread(f.Hs, (long long)((f.nx + 31) / 32) * f.nz, sizeof(R) == 8, sm_count)) {
+        case 1: return fg_run_y<R, 1>(f, s, bounds, st);
+        case 2: return fg_run_y<R, 2>(f, s, bounds, st);
+        case 3: return fg_run_y<R, 3>(f, s, bounds, st);
+        case 5: return fg_run_y<R, 5>(f, s, bounds, st);
+        default: return fg_run_y<R, 6>(f, s, bounds, st);
+    }
+}
+
+template <typename R, bool kPm>
+static cudaError_t fg_sum_xz(const FieldGrid &f, int Nxp, const int *bounds, const int *chunk_y, int sm_count,
+                             cudaStream_t st) {
+    switch (fg_rows_per_thread(f.Ht, (long long)f.Hs * f.jc, sizeof(R) == 8, sm_count)) {
+        case 1: return fg_run_xz<R, 1, kPm>(f, Nxp, bounds, chunk_y, st);
+        case 2: return fg_run_xz<R, 2, kPm>(f, Nxp, bounds, chunk_y, st);
+        case 3: return fg_run_xz<R, 3, kPm>(f, Nxp, bounds, chunk_y, st);
+        case 5: return fg_run_xz<R, 5, kPm>(f, Nxp, bounds, chunk_y, st);
+        default: return fg_run_xz<R, 6, kPm>(f, Nxp, bounds, chunk_y, st);
+    }
+}
+
+template <typename R>
+static cudaError_t fg_forward(const FieldGrid &f, const void *s, const int *bounds, double str_re, double str_im,
+                              void *A, void *I, int sm_count, cudaStream_t st) {
+    cudaError_t e = fg_sum_y<R>(f, s, bounds, sm_count, st);
+    if (e == cudaSuccess) e = fg_sum_xz<R, false>(f, f.nx, bounds, nullptr, sm_count, st);
+    return e == cudaSuccess ? fg_finish<R>(f, str_re, str_im, A, I, sm_count, st) : e;
 }
 
 cudaError_t launch_field_grid(const FieldGrid &f, const void *s, const int *bounds, double str_re, double str_im,
                               void *A, void *I, int sm_count, cudaStream_t st) {
-    const int ry = fg_rows_per_thread(f.Hs), rx = fg_rows_per_thread(f.Ht);
-    cudaError_t e;
-    if (f.elem == 8) {
-        e = ry == 3   ? fg_run_y<double, 3>(f, s, bounds, st)
-            : ry == 5 ? fg_run_y<double, 5>(f, s, bounds, st)
-                      : fg_run_y<double, 6>(f, s, bounds, st);
-        if (e == cudaSuccess)
-            e = rx == 3   ? fg_run_xz<double, 3, false>(f, f.nx, bounds, nullptr, st)
-                : rx == 5 ? fg_run_xz<double, 5, false>(f, f.nx, bounds, nullptr, st)
-                          : fg_run_xz<double, 6, false>(f, f.nx, bounds, nullptr, st);
-        return e == cudaSuccess ? fg_finish<double>(f, str_re, str_im, A, I, sm_count, st) : e;
-    }
-    e = ry == 3   ? fg_run_y<float, 3>(f, s, bounds, st)
-        : ry == 5 ? fg_run_y<float, 5>(f, s, bounds, st)
-                  : fg_run_y<float, 6>(f, s, bounds, st);
-    if (e == cudaSuccess)
-        e = rx == 3   ? fg_run_xz<float, 3, false>(f, f.nx, bounds, nullptr, st)
-            : rx == 5 ? fg_run_xz<float, 5, false>(f, f.nx, bounds, nullptr, st)
-                      : fg_run_xz<float, 6, false>(f, f.nx, bounds, nullptr, st);
-    return e == cudaSuccess ? fg_finish<float>(f, str_re, str_im, A, I, sm_count, st) : e;
+    return f.elem == 8 ? fg_forward<double>(f, s, bounds, str_re, str_im, A, I, sm_count, st)
+                       : fg_forward<float>(f, s, bounds, str_re, str_im, A, I, sm_count, st);
 }
 
 cudaError_t launch_field_grid_tc(const FieldGrid &f, int Nxp, const int *bounds, const int *chunk_y, double str_re,
                                  double str_im, float2 *A, float *I, int sm_count, cudaStream_t st) {
-    const int rx = fg_rows_per_thread(f.Ht);
-    const cudaError_t e = rx == 3   ? fg_run_xz<float, 3, true>(f, Nxp, bounds, chunk_y, st)
-                          : rx == 5 ? fg_run_xz<float, 5, true>(f, Nxp, bounds, chunk_y, st)
-                                    : fg_run_xz<float, 6, true>(f, Nxp, bounds, chunk_y, st);
+    const cudaError_t e = fg_sum_xz<float, true>(f, Nxp, bounds, chunk_y, sm_count, st);
     return e == cudaSuccess ? fg_finish<float>(f, str_re, str_im, A, I, sm_count, st) : e;
 }
 

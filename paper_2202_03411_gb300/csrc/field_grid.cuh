@@ -23,11 +23,27 @@ __device__ __forceinline__ float fg_recip(float xh, float xl, float nh, float nl
     d = fabsf(d) < 1e-12f ? 1e-12f : d;
     return __fdividef(1.0f, d);
 }
+// FP64: two Newton-Raphson steps r <- r + r (1 - d r) from the hardware's 2^-20
+// approximation (2^-40, then within 2 ulp): four FP64 operations, which this part
+// runs at 1/64 of its FP32 rate, and none of a division's special cases.
 __device__ __forceinline__ double fg_recip(double xh, double, double nh, double) {
-    double d = xh - nh;
+    double d = xh - nh, r;
     d = fabs(d) < 1e-30 ? 1e-30 : d;
-    return 1.0 / d;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    r = fma(r, fma(-d, r, 1.0), r);
+    return fma(r, fma(-d, r, 1.0), r);
 }
+
+// acc + low gains a b with twice the working precision (Ogita, Rump and Oishi's
+// Dot2: the product's and the sum's rounding errors are collected in low).
+__device__ __forceinline__ void fg_dot2(float a, float b, float &acc, float &low) {
+    const float p = __fmul_rn(a, b), e = fmaf(a, b, -p);
+    const float t = __fadd_rn(acc, p), z = __fsub_rn(t, acc);
+    low += __fadd_rn(__fsub_rn(acc, __fsub_rn(t, z)), __fsub_rn(p, z)) + e;
+    acc = t;
+}
+__device__ __forceinline__ void fg_dot2(double a, double b, double &acc, double &) { acc = fma(a, b, acc); }
+
 // ---------------------------------------------------------------------------
 // The folded sums.  A block of 256 threads computes two real products
 //   out[row][col] = sum_k T[k][row] S[k][col]

@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(kFaThreads) fa_pixels_kernel(FieldGrid f, Fiel
     __shared__ R sx[kFaPix][2][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i0 = blockIdx.x * 32, n2 = kUniform ? f.U : f.V;
+    if (ad.gmax && threadIdx.x == 0 && blockIdx.x + blockIdx.y + blockIdx.z == 0) *ad.gmax = 0u;
     const int per = (n2 + ad.chunks - 1) / ad.chunks, lo = blockIdx.y * per, hi = min(n2, lo + per);
     const int a0 = blockIdx.z * kFaWarps * kFaPts + warp;
     R nh[kFaPts], nl[kFaPts], acc[kFaPts][8];
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(kFaThreads) fa_pixels_kernel(FieldGrid f, Fiel
 // chunks of kFaCols columns in shared memory, then a warp sums kFaColPts points
 // over them, its lanes along the columns.
 constexpr int kFaCols = 256;
-constexpr int kFaColPts = 2;
+constexpr int kFaColPts = 1;
 
 template <typename R>
 __global__ void __launch_bounds__(kFaThreads) fa_columns_kernel(FieldGrid f, FieldGridAdjoint ad) {
@@ -204,6 +205,7 @@ __global__ void __launch_bounds__(kFaThreads) fa_columns_kernel(FieldGrid f, Fie
             R v = (R)0;
             if (i < n) {
                 const R *src = (const R *)ad.B + ((size_t)p2 * 8 + c) * f.n1 + i0 + i;
+#pragma unroll 8
                 for (int k = 0; k < ad.chunks; ++k) v += src[k * chunk];
                 v *= ((c >> 1) & 1) ? nd.w : nd.z;      // the per-pixel direction's constants: c_a x_a even, c_a odd
             }
@@ -256,6 +258,14 @@ __global__ void __launch_bounds__(kFaThreads) fa_columns_kernel(FieldGrid f, Fie
                     out[2 * plane + c] = (R)0.25 * (se - so);
                     out[3 * plane + c] = (R)0.25 * (de - dd);
                 }
+                // the largest magnitude (non-negative floats order like their bits)
+                float most = 0.f;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const float x = (float)out[m * plane], y = (float)out[m * plane + 1];
+                    most = fmaxf(most, sqrtf(x * x + y * y));
+                }
+                atomicMax(ad.gmax, __float_as_uint(most));
             } else {
                 R *out = (R *)ad.G + ((size_t)a * f.Ht + b) * 8;
 #pragma unroll

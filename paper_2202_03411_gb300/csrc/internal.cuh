@@ -210,6 +210,7 @@ struct FieldGrid {
     int H1 = 0, H2 = 0, n1 = 0;     // per-column (per-row) direction: its half points and half pixels; per-pixel direction
     int Kx = 0, Ky = 0, U = 0, V = 0;   // half sides of the grid and the detector, rounded up
     int jc = 0;                     // slice chunks of the x/z sum
+    int dot2 = 0;                   // FP32 interpolation sums with their rounding errors collected
     double sm = 0, tm = 0;          // largest |s|, |t|
     double k0 = 0, voxel = 0, top = 0;  // top: tan or sin of theta_max
     void *ty = nullptr, *tx = nullptr, *tz = nullptr;   // phases of the sums
@@ -225,6 +226,7 @@ struct FieldGridAdjoint {
     bool points = false;            // G holds every direction's weight, for the tensor-core sum over the directions
     void *B = nullptr, *G = nullptr, *T = nullptr;      // pixels gathered along it; onto the grid; x/z sums
     double *q = nullptr;            // the directions' q (points only)
+    unsigned *gmax = nullptr;       // receives max |G| as float bits (points only)
 };
 
 }  // namespace scm
@@ -291,7 +293,6 @@ struct scatman_handle {
     size_t vmap_cap = 0;
     double *d_mdelta = nullptr, *d_mbeta = nullptr;
     size_t mindex_cap = 0;
-    double str_re = 0, str_im = 0;  // global strength factor of s: n^2 - 1, or the map's index scale
     // pinned staging of the last two map uploads, each free again once its event has passed
     struct MapStage {
         unsigned char *p = nullptr;
@@ -301,6 +302,7 @@ struct scatman_handle {
     int map_turn = 0;
     bool map_captured = false;      // the upload under way is being captured
     std::list<std::vector<double>> captured_maps;
+    double str_re = 0, str_im = 0;  // global strength factor of s: n^2 - 1, or the map's index scale
     double map_index_max = 0;       // max |delta|, |beta| over a volume map's cells
     bool on_grid = false;           // the field goes through its sample grid
     bool peak_direct = false;       // (fits in the tensor-core modes) except the pattern's peak
@@ -438,10 +440,10 @@ int grad_voxel_blocks(bool fp64, const ShapeParams &sp, const GridParams &gp, in
 cudaError_t launch_grad_pixels(bool fp64, const void *A, const void *dLdI, long long n_pix,
                                double *partials, int n_blocks, cudaStream_t st);
 int grad_pixel_blocks(long long n_pix);
-// Tensor-core adjoint field (adjoint_tc.cu).
 // out: nv voxel sums over nvb blocks, the pixel sum over npb, the error word (nv + 2 doubles).
 cudaError_t launch_grad_totals(const double *part, int nvb, int nv, int npb, const int *err, double *out,
                                cudaStream_t st);
+// Tensor-core adjoint field (adjoint_tc.cu).
 bool adjoint_tc_supported(int nx, int ny);
 // nz: slices, or in order mode (orders != 0) the number N of Jacobi-Anger orders;
 // S receives the slices' (or orders') fields [nz][nx][ny].
@@ -471,6 +473,39 @@ cudaError_t launch_l2_residual(bool fp64, const void *I, const float *target, lo
 // ---- device helpers ---------------------------------------------------------
 #ifdef __CUDACC__
 namespace scm {
+
+// Programmatic dependent launch: the kernels of a pass are short, and each one's
+// launch and prologue can run under the end of the one before.  A kernel launched
+// so calls pdl_wait before it touches memory that other kernels use (reads or
+// writes: everything before it in the stream is then behind it).  Forward passes in
+// us, ordinary launches / this: 108 / 78 at 128^3 on 512^2 (BF16), 53 / 30 at 70 x 52 x
+// 41 on 301 x 257, 50 / 31 at 30^3 on 512^2 (uniform-q, FP32).  No kernel lets the next
+// one's blocks in early (launch_dependents): they would settle on the first SMs to
+// have room and leave the grid lopsided (88 us for the first of these, and in FP64
+// 275 instead of 190 at 96^3 on 256^2).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... Q>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Q &&...args) {
+    cudaLaunchAttribute a{};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &a;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
+// 16-byte copies to shared memory, all of a thread's in flight until it waits.
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));

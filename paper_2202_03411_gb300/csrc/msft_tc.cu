@@ -184,6 +184,7 @@ __global__ void __launch_bounds__(256) pack_units_kernel(const int *cy, int nz, 
     __shared__ int s_base;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (threadIdx.x == 0) s_base = 0;
+    pdl_wait();
     __syncthreads();
     for (int t0 = 0; t0 < nz; t0 += 256) {
         const int t = t0 + (int)threadIdx.x;
@@ -329,6 +330,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
 
     uint32_t prod_it = 0, oldest = 0, mma_it = 0, acc_it = 0, epi_it = 0;
 
@@ -828,13 +830,16 @@ static cudaError_t launch_tc(const TcMaps &maps, const double *q, long long n_pi
     if (e != cudaSuccess) return e;
     // units of the uniform-q y-sum keep their K steps on the 16-y grid (its
     // epilogue stores G itself, with no room for a per-unit phase)
-    pack_units_kernel<<<1, 256, 0, st>>>(geom_chunk_y(geom, nz), nz, Nxp / 8, max_chunks, store ? 0 : 1, list);
+    e = launch_pdl(pack_units_kernel, dim3(1), dim3(256), 0, st, geom_chunk_y(geom, nz), nz, Nxp / 8, max_chunks,
+                   store ? 0 : 1, list);
+    if (e != cudaSuccess) return e;
     int grid = P.num_units < sm_count ? P.num_units : sm_count;
     if (grid < 1) grid = 1;
     if (store) {
-        msft_tc_kernel<true><<<grid, kTcThreads, smem, st>>>(maps, P);
+        return launch_pdl(msft_tc_kernel<true>, dim3(grid), dim3(kTcThreads), smem, st, maps, P);
     } else {
-        msft_tc_kernel<false><<<grid, kTcThreads, smem, st>>>(maps, P);
+        e = launch_pdl(msft_tc_kernel<false>, dim3(grid), dim3(kTcThreads), smem, st, maps, P);
+        if (e != cudaSuccess) return e;
         if (P.whole < P.num_m_tiles) {
             const long long tail = (long long)(P.num_m_tiles - P.whole) * kBM;
             tc_tail_sum_kernel<<<(unsigned)((tail + 255) / 256), 256, 0, st>>>(

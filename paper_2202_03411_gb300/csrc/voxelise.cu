@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(kVoxThreads, 3) voxelise_scan_kernel(ShapePara
     using Re = typename std::conditional<kFp64, double, float>::type;
     Cx *s_tile = reinterpret_cast<Cx *>(smem);                                // [32][zs]
     float *chi_tile = reinterpret_cast<float *>(smem + sizeof(Cx) * zs * kLinesPerCta);
+    pdl_wait();
 
     const int ix = blockIdx.x;
     const int y0 = blockIdx.y * kLinesPerCta;
@@ -368,6 +369,7 @@ __global__ void __launch_bounds__(kVoxThreads, 3) voxelise_binary_kernel(ShapePa
     __shared__ int s_nn, s_qn;
     __shared__ ShTerms s_sh;
     if (threadIdx.x == 0) s_nn = s_qn = 0;
+    pdl_wait();
     if (!kMaps && sp.kind == SCATMAN_SPHHARM) {
         if (out.stage)
             block_copy(&s_sh, out.stage, sizeof(ShTerms));
@@ -615,6 +617,7 @@ __global__ void __launch_bounds__(kVoxThreads, 3) voxelise_binary_kernel(ShapePa
 template <typename ScanT, typename Cx>
 __global__ void voxelise_init_kernel(ShapeParams sp, int *b, int nz, int *cy, Cx *table, VoxConst vc, int first,
                                      void *stage, float *rtab) {
+    pdl_wait();
     if ((int)blockIdx.x == first) {
         sh_stage_terms(sp, *reinterpret_cast<ShTerms *>(stage));
         sh_stage_tables(sp, reinterpret_cast<double *>(reinterpret_cast<unsigned char *>(stage) + sizeof(ShTerms)));
@@ -648,9 +651,9 @@ static cudaError_t run_voxelise(const ShapeParams &sp, const GridParams &gp, con
         const int first = (2 * kGeomChunks * gp.nz + 255) / 256;
         const int cells = binary ? 6 * sp.rtab_n * sp.rtab_n : 0;
         const int more = binary && sp.kind == SCATMAN_SPHHARM ? 1 + (cells + 255) / 256 : 0;
-        voxelise_init_kernel<ScanT, Cx><<<first + more, 256, 0, st>>>(
-            sp, out.bounds, gp.nz, out.chunk_y, binary ? (Cx *)out.table : nullptr, vc, first, out.stage, out.rtab);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_pdl(voxelise_init_kernel<ScanT, Cx>, dim3(first + more), dim3(256), 0, st, sp,
+                                         out.bounds, gp.nz, out.chunk_y, binary ? (Cx *)out.table : nullptr, vc, first,
+                                         out.stage, out.rtab);
         if (e != cudaSuccess) return e;
     }
     if (binary) {
@@ -662,8 +665,7 @@ static cudaError_t run_voxelise(const ShapeParams &sp, const GridParams &gp, con
         auto k = small ? (maps ? voxelise_binary_kernel<kFp64, ScanT, true, 8> : voxelise_binary_kernel<kFp64, ScanT, false, 8>)
                        : (maps ? voxelise_binary_kernel<kFp64, ScanT, true, 16>
                                : voxelise_binary_kernel<kFp64, ScanT, false, 16>);
-        k<<<grid, kVoxThreads, smem, st>>>(sp, gp, out, vc);
-        return cudaGetLastError();
+        return launch_pdl(k, grid, dim3(kVoxThreads), smem, st, sp, gp, out, vc);
     }
     const dim3 grid(gp.nx, (gp.ny + kLinesPerCta - 1) / kLinesPerCta);
     const size_t smem = (sizeof(Cx) + sizeof(float)) * (size_t)(gp.nz + 1) * kLinesPerCta;
@@ -673,8 +675,7 @@ static cudaError_t run_voxelise(const ShapeParams &sp, const GridParams &gp, con
     auto k = maps ? voxelise_scan_kernel<kFp64, ScanT, true> : voxelise_scan_kernel<kFp64, ScanT, false>;
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
     if (e != cudaSuccess) return e;
-    k<<<grid, kVoxThreads, smem, st>>>(sp, gp, out, vc);
-    return cudaGetLastError();
+    return launch_pdl(k, grid, dim3(kVoxThreads), smem, st, sp, gp, out, vc);
 }
 
 cudaError_t launch_voxelise(const ShapeParams &sp, const GridParams &gp, const SliceOut &out, bool scan_fp64,
