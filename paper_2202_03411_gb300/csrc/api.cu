@@ -173,7 +173,6 @@ void scatman_destroy(scatman_handle *h) {
         if (h->ev_copy[b]) cudaEventDestroy(h->ev_copy[b]);
     }
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
-    cudaFree(h->d_err);
     cudaFree(h->d_part);
     cudaFree(h->d_S);
     cudaFree(h->d_partial);
@@ -382,8 +381,10 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
     if ((rc = alloc_dev(h, (void **)&h->d_chi, nvox * sizeof(float), "occupancy buffer"))) return fail(rc);
     // per-slice occupied boxes (every mode skips the empty parts of each
     // slice), then the tensor-core kernel's occupied-slice list
-    if ((rc = alloc_dev(h, (void **)&h->d_bounds, slice_geom_ints(c.nz) * sizeof(int), "slice geometry")))
-        return fail(rc);
+    // (and at its end the status block)
+    const size_t geom_bytes = (slice_geom_ints(c.nz) * sizeof(int) + 15) / 16 * 16;
+    if ((rc = alloc_dev(h, (void **)&h->d_bounds, geom_bytes + kStatusBytes, "slice geometry"))) return fail(rc);
+    h->d_err = (int *)((unsigned char *)h->d_bounds + geom_bytes);
     if (h->tensor_core) {
         h->s_bytes = h->b_rows * (size_t)h->Kp * 2;
     } else {
@@ -393,7 +394,6 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
     const size_t cx = f64 ? sizeof(double2) : sizeof(float2);
     if ((rc = alloc_dev(h, &h->d_A, npix * cx, "field buffer"))) return fail(rc);
     if ((rc = alloc_dev(h, &h->d_I, npix * (f64 ? 8 : 4), "intensity buffer"))) return fail(rc);
-    if ((rc = alloc_dev(h, (void **)&h->d_err, kStatusBytes, "status block"))) return fail(rc);
     if (h->on_grid && (rc = need_field_grid(h))) return fail(rc);
     if (h->uniform_q && !h->on_grid && (rc = alloc_dev(h, (void **)&h->d_uq_qz, npix * sizeof(float2), "q_z table")))
         return fail(rc);
@@ -618,7 +618,7 @@ static MapScan scan_map_index(const scatman_shape *s, size_t n, double *dl, doub
     const double *md = s->map_delta, *mb = s->map_beta;
     const double d0[kL] = {s->delta, s->delta, s->delta, s->delta, s->delta, s->delta, s->delta, s->delta};
     const double b0[kL] = {s->beta, s->beta, s->beta, s->beta, s->beta, s->beta, s->beta, s->beta};
-    auto lanes = [&](const double *vd, const double *vb, size_t k, size_t m) {
+    auto lanes = [&](const double *vd, const double *vb, size_t k, size_t m) __attribute__((always_inline)) {
         for (size_t i = 0; i < m; ++i) {
             const double d = vd[i], b = vb[i];
             dl[k + i] = d;
