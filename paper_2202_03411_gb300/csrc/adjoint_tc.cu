@@ -38,9 +38,9 @@
 // scattering directions (field_grid_adjoint.cu), q runs over its few thousand
 // points.  Fewer terms average the FP16 roundings less, so both operands are
 // held as FP16 pairs there and every chunk of 32 points is taken three times,
-// L_hi R_hi + L_lo R_hi + L_hi R_lo, into the same accumulators.  Measured (fit
-// step, 96^3 on 256^2 to 45 degrees, 19 orders): 104.6 us over the 65536 pixels;
-// over the 2704 points see adjoint_tc_kernel's caller in api.cu.
+// L_hi R_hi + L_lo R_hi + L_hi R_lo, into the same accumulators.  Measured (96^3 on
+// 256^2 to 45 degrees, FP16 fit): 104.6 us over the 65536 pixels with a gradient
+// error of 1.9e-6 against 64 bits, 35 us and 6e-7 over the grid's points.
 #include "internal.cuh"
 #include "tc_ptx.cuh"
 

@@ -869,7 +869,7 @@ static cudaError_t fg_run_pixels(const FieldGrid &f, double str_re, double str_i
     // the largest size any plan uses, so concurrent launches of other handles stay valid
     const size_t most = (size_t)fg_max_half(sizeof(R) == 8) * (8 * (kUniform ? 4 : 32) * sizeof(R) + sizeof(V4));
     const auto k = fg_pixels_out_kernel<R, kPts, kUniform, kWarps, kDot2, kSplit>;
-    cudaError_t e = fg_smem(k, most);
+    cudaError_t e = smem <= (size_t)40 << 10 ? cudaSuccess : fg_smem(k, most);
     if (e != cudaSuccess) return e;
     const dim3 grid = kUniform ? dim3((f.U + 32 * kPts - 1) / (32 * kPts), (f.V + 3) / 4)
                  : kSplit ? dim3((f.U + 31) / 32, f.V)

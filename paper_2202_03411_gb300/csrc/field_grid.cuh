@@ -86,8 +86,12 @@ __device__ __forceinline__ void fg_multiply(const FgTile<R, kRpt, kPad> &t, int 
 __device__ __forceinline__ int fg_plus(int k, int n) { return n / 2 + k; }
 __device__ __forceinline__ int fg_minus(int k, int n) { return (n - 1) / 2 - k; }
 
+// Opts a kernel in to `bytes` of dynamic shared memory where that needs it (beside at
+// most 8 KB of static); always the same bytes per kernel or its plans' largest, so
+// that launches of other threads stay valid.
 template <typename K>
 static cudaError_t fg_smem(K kernel, size_t bytes) {
+    if (bytes <= (size_t)40 << 10) return cudaSuccess;
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 

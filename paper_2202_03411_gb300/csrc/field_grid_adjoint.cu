@@ -14,6 +14,10 @@
 // FP32 and FP64 modes run all of it here; the tensor-core modes gather onto the
 // grid here and sum over its directions on the tensor cores (adjoint_tc.cu).
 //
+// Short kernels, bound by their launches and the latency of their loads: 48^3 on
+// 128^2, FP32: pixels 6.2 us, columns 8.9, x/z 5.2, y 6.4 (the direct sums over pixels
+// and voxels: 12.4 ms).
+//
 // All sums have a fixed order (chunks of pixels are added in order), so the
 // gradient is the same bit for bit on every call.
 #include "internal.cuh"
