@@ -618,14 +618,16 @@ def run_reference(args):
 
 
 def launches_per_pattern(precision: str, n_pix: int, sm_count: int) -> int:
-    """Kernels one voxelise + forward launches: tensor-core modes reset the
-    slice boxes, voxelise with the scan, pack the occupied-slice list and run
-    the contraction, plus the sum of the cut tiles' partial fields when the
-    last wave of 128-pixel tiles is cut into slice ranges; the CUDA-core modes
-    voxelise and run the contraction with its fixed-order partial-sum
-    reduction."""
+    """Kernels one voxelise + forward launches.  Every mode resets the slice boxes
+    and voxelises; the split phases list the work units, sum over y on the tensor
+    cores, then over x and z, and interpolate in two steps (FP32 and FP64: the
+    same without the list); the single-product modes list the units and run the
+    direct contraction, plus the sum of the cut tiles' partial fields when the
+    last wave of 128-pixel tiles is cut into slice ranges."""
     if not precision.startswith("tc_"):
-        return 3
+        return 6
+    if "split" in precision:
+        return 7
     tiles = (n_pix + 127) // 128
     rem = tiles % sm_count if tiles > sm_count else tiles
     parts = min(4, max(1, (sm_count + rem // 2) // rem)) if rem else 1
@@ -775,31 +777,29 @@ def main():
     clocks = sampler.stop()
     single_stream = world * B * args.steps / (max_over_ranks(sum(step1_ms), dist, "cuda") / 1e3)
 
-    # roofline of the contraction kernel (the dominant launch)
+    # the forward pass: its tensor-core work (the sums over y at the grid's
+    # directions) over its whole duration, beside the direct sums' work that it
+    # stands for (8 flop per pixel, occupied voxel and phase product)
     peaks, peak_kind = measured_peaks()
     n_vox = g.nx * g.ny * g.nz
     products = 2 if "split" in args.precision else 1
-    executed = statistics.mean(issued)                 # real flops the contraction executes per pattern
-    method = 8.0 * g.n_pix * statistics.mean(occupied) * products    # the method's own work per pattern
+    executed = statistics.mean(issued)                 # real flops the tensor cores execute per pattern
+    direct = 8.0 * g.n_pix * statistics.mean(occupied) * products
     fwd_avg_s = statistics.mean(fwd_ms) / 1e3
-    achieved = method / fwd_avg_s / 1e12
     peak = float(peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops")))
-    roofline = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": achieved / peak,
+    roofline = {"bound": "latency", "achieved": executed / fwd_avg_s / 1e12, "peak": peak, "unit": "TFLOP/s",
+                "frac": executed / fwd_avg_s / 1e12 / peak,
                 "traffic": recorded_traffic("msft_tc_kernel", "paper_2202_03411_gb300/csrc/msft_tc.cu"),
-                "kernel": "msft_tc_kernel",
+                "kernel": "forward pass (msft_tc_kernel in store mode, fg_xz_kernel, fg_columns_kernel, "
+                          "fg_pixels_out_kernel)",
                 "peak_source": f"{peak_kind} bf16_tflops_sustained (cuBLAS bf16; f16 has the same nominal rate)",
-                "flops_per_launch": method,
-                "flops_basis": "the method's work: 8 flop x pixels x occupied voxels x phase products "
-                               f"({statistics.mean(occupied):.0f} occupied voxels of {n_vox} on average)",
-                "executed_flops_per_launch": executed,
-                "executed_tflops": executed / fwd_avg_s / 1e12,
-                "executed_frac": executed / fwd_avg_s / 1e12 / peak,
-                "executed_over_method": executed / method,
-                "dense_flops_per_launch": statistics.mean(dense),
-                "dense_equivalent_tflops": statistics.mean(dense) / fwd_avg_s / 1e12,
-                "frac_of_burst_peak": achieved / float(peaks.get("bf16_tflops", peak)),
-                "useful_single_product_tflops": achieved / products}
+                "flops_per_launch": executed,
+                "flops_basis": "tensor-core flops of the sums over y; the x/z sums and the interpolation run on the "
+                               "CUDA cores",
+                "direct_sum_flops": direct,
+                "direct_sum_basis": "8 flop x pixels x occupied voxels x phase products "
+                                    f"({statistics.mean(occupied):.0f} occupied voxels of {n_vox} on average)",
+                "dense_direct_sum_flops": statistics.mean(dense)}
 
     # the voxeliser + scan: ALU-bound (the harmonic radius per voxel); its HBM
     # writes are the slice operand and the occupancy
@@ -811,7 +811,8 @@ def main():
     voxelise = {"bound": "alu", "bytes_written_per_launch": vox_bytes, "achieved_gbs": vox_bytes / vox_s / 1e9,
                 "hbm_peak_gbs": float(peaks.get("hbm_gbs", 0.0)),
                 "frac_of_hbm": vox_bytes / vox_s / 1e9 / float(peaks.get("hbm_gbs", 1.0)),
-                "note": "one spherical-harmonics radius (l <= 8) per voxel; the writes are far below HBM speed"}
+                "note": "band and radius-table tests per voxel, one spherical-harmonics radius (l <= 8) near the "
+                        "surface; the writes are far below HBM speed"}
 
     # end to end through the C ABI with host memory: voxelise + forward + D2H per pattern
     # (the pipelined batch call: pattern i computes while pattern i - 1 downloads),
