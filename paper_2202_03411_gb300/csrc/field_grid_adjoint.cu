@@ -183,11 +183,11 @@ __global__ void __launch_bounds__(kFaThreads) fa_pixels_kernel(FieldGrid f, Fiel
 // [sign of s][sign of t][a][b]: the columns (rows) gathered onto the other
 // direction's points.  Block: one point of the per-pixel direction; it adds the
 // chunks of kFaCols columns in shared memory, then a warp sums kFaColPts points
-// over them, its lanes along the columns.  Adding the chunks takes the time, so a
-// block serves all points of up to 40 (with two points per warp, and the chunks
-// added again by each block, 13 us at 256^2 pixels and 21 us at 512^2).
+// over them, its lanes along the columns.  (Five points per warp, so that one block
+// adds the chunks for all, took 18 us instead of 13 at 96^3 on 256^2 pixels: the
+// points' sums are as long a chain as the chunks'.)
 constexpr int kFaCols = 256;
-constexpr int kFaColPts = 5;
+constexpr int kFaColPts = 2;
 
 template <typename R>
 __global__ void __launch_bounds__(kFaThreads) fa_columns_kernel(FieldGrid f, FieldGridAdjoint ad) {
@@ -211,8 +211,13 @@ __global__ void __launch_bounds__(kFaThreads) fa_columns_kernel(FieldGrid f, Fie
             R v = (R)0;
             if (i < n) {
                 const R *src = (const R *)ad.B + ((size_t)p2 * 8 + c) * f.n1 + i0 + i;
-#pragma unroll 16
-                for (int k = 0; k < ad.chunks; ++k) v += src[k * chunk];
+                for (int k = 0; k < ad.chunks; k += 8) {
+                    R part[8];                          // eight chunks' loads in flight, added in order
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) part[q] = k + q < ad.chunks ? src[(k + q) * chunk] : (R)0;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) v += part[q];
+                }
                 v *= ((c >> 1) & 1) ? nd.w : nd.z;      // the per-pixel direction's constants: c_a x_a even, c_a odd
             }
             sb[c][i] = v;
