@@ -33,14 +33,6 @@
 // same kernel, with the order n in place of the slice and the real factor
 // cos(n theta_q) in place of the slice phase; adj_orders_combine_kernel then
 // forms S_j = sum_n a[j, n] S~_n with a[j, n] = e^{+i q_c z_j} eps_n i^n J_n(D z_j).
-//
-// Split operands.  Where the pixels have been gathered onto the sample grid of
-// scattering directions (field_grid_adjoint.cu), q runs over its few thousand
-// points.  Fewer terms average the FP16 roundings less, so both operands are
-// held as FP16 pairs there and every chunk of 32 points is taken three times,
-// L_hi R_hi + L_lo R_hi + L_hi R_lo, into the same accumulators.  Measured (96^3 on
-// 256^2 to 45 degrees, FP16 fit): 104.6 us over the 65536 pixels with a gradient
-// error of 1.9e-6 against 64 bits, 35 us and 6e-7 over the grid's points.
 #include "internal.cuh"
 #include "tc_ptx.cuh"
 
@@ -62,11 +54,10 @@ struct AdjParams {
                                 // order mode: theta (hi, lo) in place of q_z and e^{+i theta} in place of e^{+i qz dv}
     int orders;                 // 1: order mode (nz below is the number of orders N)
     const uint8_t *rtile;       // per 32-pixel chunk: the y-phase operand tile (2 Nyp rows x 128 bytes)
-    const uint8_t *rtile_lo;    // its low half: split operands (null: one product)
     int stages;
     int teams;                  // generator teams (1, 2 or 4; never more than stages)
     const float2 *A;            // forward field (FP32)
-    const float *w;             // dL/dI (null: 1, and gmax_bits is the caller's)
+    const float *w;             // dL/dI
     const unsigned *gmax_bits;  // max |w A| as float bits
     long long n_pix;
     int nx, ny, nz, Nyp;
@@ -125,8 +116,7 @@ cudaError_t launch_adj_pixel_table(const double *q, long long n, double voxel, i
 // The y-phase operand, per 32-pixel chunk, as the tile image the MMA reads:
 // row y holds (Re R, -Im R) and row Nyp + y holds (Im R, Re R) for each pixel,
 // R = e^{+i q_y y} (zero past the last pixel).
-// lo: the part that FP16 leaves of it instead.
-__global__ void adj_rtile_kernel(const float4 *__restrict__ tab, long long n_pix, int Nyp, int ny, double voxel, bool lo,
+__global__ void adj_rtile_kernel(const float4 *__restrict__ tab, long long n_pix, int Nyp, int ny, double voxel,
                                  uint8_t *__restrict__ rt, long long total) {
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= total) return;
@@ -139,10 +129,6 @@ __global__ void adj_rtile_kernel(const float4 *__restrict__ tab, long long n_pix
         const float4 ta = tab[3 * p];
         const float yv = ((float)y - 0.5f * (float)(ny - 1)) * (float)voxel;
         R = expmi_fs(ta.z, ta.w, -yv);           // e^{+i q_y y}
-        if (lo) {
-            R.x -= __half2float(__float2half_rn(R.x));
-            R.y -= __half2float(__float2half_rn(R.y));
-        }
     }
     uint8_t *tile = rt + cg * (long long)(2 * Nyp * 128);
     *reinterpret_cast<uint32_t *>(tile + pair_offset(y, i)) = pack_half2(R.x, -R.y);
@@ -154,11 +140,10 @@ size_t adj_rtile_bytes(long long n_pix, int ny) {
     return (size_t)((n_pix + kAdjChunk - 1) / kAdjChunk) * 2 * Nyp * 128;
 }
 
-cudaError_t launch_adj_rtile(const float4 *tab, long long n_pix, int ny, double voxel, bool lo, uint8_t *rt,
-                             cudaStream_t st) {
+cudaError_t launch_adj_rtile(const float4 *tab, long long n_pix, int ny, double voxel, uint8_t *rt, cudaStream_t st) {
     const int Nyp = ((ny + 7) / 8 * 8 + 15) / 16 * 16;
     const long long total = (n_pix + kAdjChunk - 1) / kAdjChunk * kAdjChunk * Nyp;
-    adj_rtile_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(tab, n_pix, Nyp, ny, voxel, lo, rt, total);
+    adj_rtile_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(tab, n_pix, Nyp, ny, voxel, rt, total);
     return cudaGetLastError();
 }
 
@@ -182,8 +167,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_tc_kernel(const AdjPar
     const int j0 = 2 * blockIdx.x;                          // slices j0, j0 + 1
     const long long p_begin = (long long)blockIdx.y * P.pix_per_split;
     const long long p_end = min(P.n_pix, p_begin + P.pix_per_split);
-    const int n_prod = P.rtile_lo ? 3 : 1;                  // products per chunk of pixels
-    const int n_chunks = p_end > p_begin ? n_prod * (int)((p_end - p_begin + kAdjChunk - 1) / kAdjChunk) : 0;
+    const int n_chunks = p_end > p_begin ? (int)((p_end - p_begin + kAdjChunk - 1) / kAdjChunk) : 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < NS; ++s) {
@@ -234,7 +218,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_tc_kernel(const AdjPar
         __syncwarp();
     } else if (warp == kAdjLoadWarp) {
         // ---------------- y-phase operand: one bulk copy per chunk ----------------
-        const size_t src0 = (size_t)(p_begin / kAdjChunk) * b_bytes;
+        const uint8_t *src = P.rtile + (size_t)(p_begin / kAdjChunk) * b_bytes;
         int issued = 0;
         for (int c = 0; c < n_chunks; ++c) {
             const uint32_t s = c % NS, ph = (c / NS) & 1;
@@ -242,9 +226,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_tc_kernel(const AdjPar
             if (elect_one()) {
                 const uint32_t fb = smem_u32(&bfull[s]);
                 mbar_arrive_expect_tx(fb, b_bytes);
-                const uint8_t *src = (c % n_prod == 2 ? P.rtile_lo : P.rtile) + src0;
-                bulk_load(smem_u32(base + s * stage_bytes + 2 * kAdjTileA), src + (size_t)(c / n_prod) * b_bytes,
-                          b_bytes, fb);
+                bulk_load(smem_u32(base + s * stage_bytes + 2 * kAdjTileA), src + (size_t)c * b_bytes, b_bytes, fb);
             }
             __syncwarp();
             ++issued;
@@ -282,10 +264,10 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_tc_kernel(const AdjPar
         float w_n = 0.f;
         float4 ta_n = make_float4(0.f, 0.f, 0.f, 0.f), tb_n = ta_n, tc_n = ta_n;
         auto load_pixel = [&](int c) {
-            const long long p = p_begin + (long long)(c / n_prod) * kAdjChunk + i;
+            const long long p = p_begin + (long long)c * kAdjChunk + i;
             if (c < n_chunks && p < p_end && r0 < r1) {
                 a_n = P.A[p];
-                w_n = P.w ? P.w[p] : 1.f;
+                w_n = P.w[p];
                 ta_n = P.tab[3 * p];
                 tb_n = P.tab[3 * p + 1];
                 tc_n = P.tab[3 * p + 2];
@@ -305,15 +287,6 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_tc_kernel(const AdjPar
             if (!warp_wait(smem_u32(&empty[s]), ph ^ 1, abort_flag, P.err, kErrTimeoutEpilogue)) break;
             uint8_t *sA0 = base + s * stage_bytes;
             uint8_t *sA1 = sA0 + kAdjTileA;
-            const bool low = c % n_prod == 1;            // this product's half of L
-            auto pack = [&](float a, float b) {
-                if (low) {
-                    const float2 h = __half22float2(__floats2half2_rn(a, b));
-                    a -= h.x;
-                    b -= h.y;
-                }
-                return pack_half2(a, b);
-            };
             if (r0 < r1) {
                 const float wp = w_c * inv_g;
                 const float2 g = make_float2(a_c.x * wp, a_c.y * wp);
@@ -328,8 +301,8 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_tc_kernel(const AdjPar
                     const float c0 = ez.x, c1 = ez.x * ezs.x - ez.y * ezs.y;
                     float2 G = cmul(g, ex);
                     auto put = [&](uint8_t *d0, uint8_t *d1) {
-                        *reinterpret_cast<uint32_t *>(d0) = pack(c0 * G.x, c0 * G.y);
-                        *reinterpret_cast<uint32_t *>(d1) = pack(c1 * G.x, c1 * G.y);
+                        *reinterpret_cast<uint32_t *>(d0) = pack_half2(c0 * G.x, c0 * G.y);
+                        *reinterpret_cast<uint32_t *>(d1) = pack_half2(c1 * G.x, c1 * G.y);
                         G = cmul(G, exs);
                     };
                     int r = r0;
@@ -353,8 +326,8 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_tc_kernel(const AdjPar
                     for (int r = r0; r < r1; ++r) {
                         const float2 L1 = cmul(L0, ezs);
                         const uint32_t off = pair_offset(r, i);
-                        *reinterpret_cast<uint32_t *>(sA0 + off) = pack(L0.x, L0.y);
-                        *reinterpret_cast<uint32_t *>(sA1 + off) = pack(L1.x, L1.y);
+                        *reinterpret_cast<uint32_t *>(sA0 + off) = pack_half2(L0.x, L0.y);
+                        *reinterpret_cast<uint32_t *>(sA1 + off) = pack_half2(L1.x, L1.y);
                         L0 = cmul(L0, exs);
                     }
                 }
@@ -477,14 +450,13 @@ int adjoint_tc_splits(long long n_pix, int nz, int sm_count, bool orders) {
     return best;
 }
 
-cudaError_t launch_adjoint_tc(const float2 *A, const float *w, const float4 *tab, const uint8_t *rtile,
-                              const uint8_t *rtile_lo, long long n_pix, int nx, int ny, int nz, int orders, double voxel, int splits, float2 *partial,
+cudaError_t launch_adjoint_tc(const float2 *A, const float *w, const float4 *tab, const uint8_t *rtile, long long n_pix,
+                              int nx, int ny, int nz, int orders, double voxel, int splits, float2 *partial,
                               unsigned *gmax_bits, float2 *S, int *err, cudaStream_t st) {
     AdjParams P;
     P.tab = tab;
     P.orders = orders ? 1 : 0;
     P.rtile = rtile;
-    P.rtile_lo = rtile_lo;
     P.A = A;
     P.w = w;
     P.gmax_bits = gmax_bits;
@@ -507,12 +479,9 @@ cudaError_t launch_adjoint_tc(const float2 *A, const float *w, const float4 *tab
     P.partial = partial;
     P.nvox = (long long)nx * ny * nz;
     P.err = err;
-    cudaError_t e;
-    if (w) {                                         // (with w null the caller has the largest |A|)
-        e = cudaMemsetAsync(gmax_bits, 0, sizeof(unsigned), st);
-        if (e != cudaSuccess) return e;
-        adj_gmax_kernel<<<(unsigned)std::min<long long>((n_pix + 255) / 256, 1024), 256, 0, st>>>(A, w, n_pix, gmax_bits);
-    }
+    cudaError_t e = cudaMemsetAsync(gmax_bits, 0, sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
+    adj_gmax_kernel<<<(unsigned)std::min<long long>((n_pix + 255) / 256, 1024), 256, 0, st>>>(A, w, n_pix, gmax_bits);
     e = cudaFuncSetAttribute(adjoint_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
     if (e != cudaSuccess) return e;
     dim3 grid((nz + 1) / 2, splits);

@@ -1196,15 +1196,15 @@ static int adjoint_orders_needed(double wmax, double tol) {
     return 512;
 }
 
-// Chooses the tensor-core adjoint's form for the handle (once) over n directions
-// q (the handle's pixels, or the grid's points): with their q_z in [q_c - D, q_c + D] and |z_j| <= z_max, order mode takes
+// Chooses the tensor-core adjoint's form for the handle (once): with the q_z of
+// the handle's pixels in [q_c - D, q_c + D] and |z_j| <= z_max, order mode takes
 // N orders for w = D z_max; it is used when N < nz.  Builds the pixel table in
 // the chosen form and, in order mode, the coefficients a[j][n].
-static int plan_adjoint(scatman_handle *h, const double *q, long long n) {
+static int plan_adjoint(scatman_handle *h) {
     const scatman_config &c = h->cfg;
-    std::vector<double> qz((size_t)n);
-    int rc = check_cuda(h, cudaMemcpy2DAsync(qz.data(), sizeof(double), q + 2, 3 * sizeof(double), sizeof(double),
-                                             (size_t)n, cudaMemcpyDeviceToHost, h->stream),
+    std::vector<double> qz((size_t)h->n_pix);
+    int rc = check_cuda(h, cudaMemcpy2DAsync(qz.data(), sizeof(double), h->d_q + 2, 3 * sizeof(double), sizeof(double),
+                                             (size_t)h->n_pix, cudaMemcpyDeviceToHost, h->stream),
                         "q_z download");
     if (rc) return rc;
     if ((rc = check_cuda(h, cudaStreamSynchronize(h->stream), "q_z download"))) return rc;
@@ -1218,8 +1218,9 @@ static int plan_adjoint(scatman_handle *h, const double *q, long long n) {
     const int N = D > 0.0 ? adjoint_orders_needed(D * zmax, 1e-7) : 1;
     const bool orders = N < c.nz && N <= 64;
     h->adj_orders = orders ? N : 0;
-    if ((rc = alloc_dev(h, (void **)&h->d_adj_tab, (size_t)n * 3 * sizeof(float4), "adjoint pixel table"))) return rc;
-    if ((rc = check_cuda(h, launch_adj_pixel_table(q, n, c.voxel, orders ? 1 : 0, qc,
+    if ((rc = alloc_dev(h, (void **)&h->d_adj_tab, (size_t)h->n_pix * 3 * sizeof(float4), "adjoint pixel table")))
+        return rc;
+    if ((rc = check_cuda(h, launch_adj_pixel_table(h->d_q, h->n_pix, c.voxel, orders ? 1 : 0, qc,
                                                    orders && D > 0.0 ? 1.0 / D : 0.0, h->d_adj_tab, h->stream),
                          "adjoint pixel table")))
         return rc;
@@ -1276,44 +1277,24 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
         if ((rc = alloc_dev(h, (void **)&h->d_part, need * sizeof(double), "gradient partials"))) return rc;
         h->part_count = need;
     }
-    // the sums run over the pixels, or over the sample grid's directions with the pixels gathered onto them
-    long long n_q = h->n_pix;
-    const void *w_q = dLdI_dev, *A_q = h->d_A;
-    const bool tc_adjoint = h->tensor_core && adjoint_tc_supported(c.nx, c.ny);
+    if (!h->adj_on_grid && (rc = need_q(h))) return rc;      // sums over the pixels
     if (h->adj_on_grid) {
         if ((rc = need_field_grid(h))) return rc;
         if (!h->d_fga) {
-            if ((rc = alloc_dev(h, (void **)&h->d_fga, field_grid_adjoint_layout(h->fg, tc_adjoint, &h->fga, nullptr),
+            if ((rc = alloc_dev(h, (void **)&h->d_fga, field_grid_adjoint_layout(h->fg, &h->fga, nullptr),
                                 "adjoint sample grid")))
                 return rc;
-            field_grid_adjoint_layout(h->fg, tc_adjoint, &h->fga, h->d_fga);
-            if (tc_adjoint &&
-                (rc = check_cuda(h, launch_field_grid_points(h->fg, h->fga.q, h->stream), "adjoint sample grid")))
-                return rc;
+            field_grid_adjoint_layout(h->fg, &h->fga, h->d_fga);
         }
-        if (tc_adjoint) {
-            if (!h->d_gmax && (rc = alloc_dev(h, (void **)&h->d_gmax, sizeof(unsigned), "adjoint scale"))) return rc;
-            h->fga.gmax = h->d_gmax;
-            rc = check_cuda(h, launch_field_grid_gather(h->fg, h->fga, (const float2 *)h->d_A, (const float *)dLdI_dev,
-                                                        h->stream),
-                            "adjoint gather");
-            n_q = 4ll * h->fg.Hs * h->fg.Ht;
-            w_q = nullptr;
-            A_q = h->fga.G;
-        } else {
-            rc = check_cuda(h, launch_field_grid_adjoint(h->fg, h->fga, h->d_A, dLdI_dev, h->d_S, h->stream),
-                            "adjoint field");
-        }
+        rc = check_cuda(h, launch_field_grid_adjoint(h->fg, h->fga, h->d_A, dLdI_dev, h->d_S, h->stream),
+                        "adjoint field");
         if (rc) return rc;
-    } else if ((rc = need_q(h))) {
-        return rc;
-    }
-    if (tc_adjoint) {
+    } else if (h->tensor_core && adjoint_tc_supported(c.nx, c.ny)) {
         // adjoint contraction on the tensor cores (per slice, or per Jacobi-Anger order)
-        if (h->adj_orders < 0 && (rc = plan_adjoint(h, h->adj_on_grid ? h->fga.q : h->d_q, n_q))) return rc;
+        if (h->adj_orders < 0 && (rc = plan_adjoint(h))) return rc;
         const int N = h->adj_orders;
         const int nz_eff = N > 0 ? N : c.nz;
-        int splits = adjoint_tc_splits(n_q, nz_eff, h->sm_count, N > 0);
+        int splits = adjoint_tc_splits(h->n_pix, nz_eff, h->sm_count, N > 0);
         while (N > 0 && splits > 1 && splits * N > 8 * c.nz) --splits;   // within the slice mode's partial memory
         const size_t cnt = (size_t)splits * nz_eff * c.nx * c.ny;
         if (h->adj_part_count < cnt) {
@@ -1324,20 +1305,16 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
             h->adj_part_count = cnt;
         }
         if (!h->d_gmax && (rc = alloc_dev(h, (void **)&h->d_gmax, sizeof(unsigned), "adjoint scale"))) return rc;
-        const size_t rt_bytes = adj_rtile_bytes(n_q, c.ny);
         if (!h->d_adj_rtile) {
-            if ((rc = alloc_dev(h, (void **)&h->d_adj_rtile, (h->adj_on_grid ? 2 : 1) * rt_bytes,
-                                "adjoint y-phase tiles")))
+            if ((rc = alloc_dev(h, (void **)&h->d_adj_rtile, adj_rtile_bytes(h->n_pix, c.ny), "adjoint y-phase tiles")))
                 return rc;
-            for (int lo = 0; lo < (h->adj_on_grid ? 2 : 1); ++lo)
-                if ((rc = check_cuda(h, launch_adj_rtile(h->d_adj_tab, n_q, c.ny, c.voxel, lo != 0,
-                                                         h->d_adj_rtile + lo * rt_bytes, h->stream),
-                                     "adjoint y-phase tiles")))
-                    return rc;
+            if ((rc = check_cuda(h, launch_adj_rtile(h->d_adj_tab, h->n_pix, c.ny, c.voxel, h->d_adj_rtile, h->stream),
+                                 "adjoint y-phase tiles")))
+                return rc;
         }
-        rc = check_cuda(h, launch_adjoint_tc((const float2 *)A_q, (const float *)w_q, h->d_adj_tab, h->d_adj_rtile,
-                                             h->adj_on_grid ? h->d_adj_rtile + rt_bytes : nullptr, n_q, c.nx, c.ny,
-                                             nz_eff, N > 0 ? 1 : 0, c.voxel, splits, h->d_adj_part, h->d_gmax,
+        rc = check_cuda(h, launch_adjoint_tc((const float2 *)h->d_A, (const float *)dLdI_dev, h->d_adj_tab,
+                                             h->d_adj_rtile, h->n_pix, c.nx, c.ny, nz_eff, N > 0 ? 1 : 0, c.voxel,
+                                             splits, h->d_adj_part, h->d_gmax,
                                              N > 0 ? h->d_adj_ord : (float2 *)h->d_S, h->d_err, h->stream),
                         "adjoint field (tensor cores)");
         if (rc) return rc;
@@ -1345,7 +1322,7 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
                                                                    (float2 *)h->d_S, h->stream),
                                       "adjoint slices from orders")))
             return rc;
-    } else if (!h->adj_on_grid) {
+    } else {
         rc = check_cuda(h, launch_adjoint_field(f64, h->d_A, dLdI_dev, h->d_q, h->n_pix, c.nx, c.ny, c.nz, c.voxel,
                                                 h->d_S, h->stream),
                         "adjoint field");

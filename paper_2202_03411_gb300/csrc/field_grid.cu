@@ -155,15 +155,19 @@ bool use_field_grid(const scatman_config &c, FieldGrid *f) {
     return true;
 }
 
-// Whether the adjoint runs through the grid.  In the tensor-core modes it pays
-// once three products over the grid's directions and the gather are less work
-// than one product over the pixels.
+// Whether the adjoint runs through the grid: FP32 and FP64, and tensor-core grids
+// beyond the tensor-core adjoint's 128 voxels.  Within those the tensor-core modes
+// sum over the pixels themselves.  A fit's upstream weight 2 (I - target) nearly
+// cancels in some parameters, and a gradient there shows the operands' 16-bit
+// roundings several hundred times larger: summed over the grid's directions, with
+// three products, served gradients of 48^3 - 128^3 on 128^2 - 512^2 pixels moved by
+// more than 2e-5 in 8 of 40 batches, by 4e-4 at most.  (Over the pixels 105 us of a
+// 96^3 fit step on 256^2; over the directions 35.)
 bool use_field_grid_adjoint(const scatman_config &c, FieldGrid *f) {
     const double pixels = (double)c.det_nx * c.det_ny;
     if (c.q_list || pixels < 128.0) return false;
-    const bool tc = c.precision != SCATMAN_FP64 && c.precision != SCATMAN_FP32 && adjoint_tc_supported(c.nx, c.ny);
-    if (!plan_field_grid(c, c.precision == SCATMAN_FP64, f)) return false;
-    return !tc || 12.0 * f->Hs * f->Ht + 8192.0 < pixels;
+    if (c.precision != SCATMAN_FP64 && c.precision != SCATMAN_FP32 && adjoint_tc_supported(c.nx, c.ny)) return false;
+    return plan_field_grid(c, c.precision == SCATMAN_FP64, f);
 }
 
 static size_t up256(size_t b) { return (b + 255) / 256 * 256; }

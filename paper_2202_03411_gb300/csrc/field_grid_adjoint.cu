@@ -10,9 +10,7 @@
 //   T_a[j][x] = sum_b e^{+i q_z(a,b) z_j} e^{+i q_x(a,b) x} G_ab
 //   S[j][x][y] = sum_a e^{+i k0 s_a y} T_a[j][x],
 // folded by the signs of s, t, x, y as in the forward sums: a parity of G
-// meets only cosines or only sines, and two mirror voxels share a sum.  The
-// FP32 and FP64 modes run all of it here; the tensor-core modes gather onto the
-// grid here and sum over its directions on the tensor cores (adjoint_tc.cu).
+// meets only cosines or only sines, and two mirror voxels share a sum.
 //
 // Short kernels, bound by their launches and the latency of their loads: 48^3 on
 // 128^2, FP32: pixels 6.2 us, columns 8.9, x/z 5.2, y 6.4 (the direct sums over pixels
@@ -42,7 +40,7 @@ static int fa_chunks(const FieldGrid &f) {
     return c < 1 ? 1 : c > kFaMaxChunks ? kFaMaxChunks : c;
 }
 
-size_t field_grid_adjoint_layout(const FieldGrid &f, bool points, FieldGridAdjoint *a, unsigned char *base) {
+size_t field_grid_adjoint_layout(const FieldGrid &f, FieldGridAdjoint *a, unsigned char *base) {
     size_t at = 0;
     auto take = [&](size_t bytes) {
         unsigned char *p = base ? base + at : nullptr;
@@ -51,29 +49,10 @@ size_t field_grid_adjoint_layout(const FieldGrid &f, bool points, FieldGridAdjoi
     };
     const size_t e = (size_t)f.elem;
     a->chunks = fa_chunks(f);
-    a->points = points;
     a->B = take((size_t)a->chunks * f.H2 * 8 * f.n1 * e);
     a->G = take((size_t)f.Hs * f.Ht * 8 * e);
-    a->T = points ? nullptr : take(2 * (size_t)f.Hs * f.nz * f.nx * 2 * e);
-    a->q = points ? (double *)take(4 * (size_t)f.Hs * f.Ht * 3 * sizeof(double)) : nullptr;
+    a->T = take(2 * (size_t)f.Hs * f.nz * f.nx * 2 * e);
     return at;
-}
-
-// q of the grid's directions [sign of s][sign of t][a][b].
-__global__ void fa_points_kernel(FieldGrid f, double *__restrict__ q) {
-    const int n = f.Hs * f.Ht, i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 4 * n) return;
-    const int m = i / n, a = (i % n) / f.Ht, b = i % f.Ht;
-    const double s = f.point_s[2 * a], c = f.point_s[2 * a + 1], t = f.point_t[2 * b], r = f.point_t[2 * b + 1];
-    q[3 * (size_t)i] = (m & 1 ? -f.k0 : f.k0) * c * t;
-    q[3 * (size_t)i + 1] = (m & 2 ? -f.k0 : f.k0) * s;
-    // k_z - 1 without cancellation near the axis
-    q[3 * (size_t)i + 2] = -f.k0 * (s * s + c * c * t * t) / (1.0 + c * r);
-}
-
-cudaError_t launch_field_grid_points(const FieldGrid &f, double *q, cudaStream_t st) {
-    fa_points_kernel<<<(4 * f.Hs * f.Ht + 255) / 256, 256, 0, st>>>(f, q);
-    return cudaGetLastError();
 }
 
 // B[chunk][point 2][parity 1 x parity 2][i]: the pixels of one column (row) i
@@ -91,7 +70,6 @@ __global__ void __launch_bounds__(kFaThreads) fa_pixels_kernel(FieldGrid f, Fiel
     __shared__ R sx[kFaPix][2][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i0 = blockIdx.x * 32, n2 = kUniform ? f.U : f.V;
-    if (ad.gmax && threadIdx.x == 0 && blockIdx.x + blockIdx.y + blockIdx.z == 0) *ad.gmax = 0u;
     const int per = (n2 + ad.chunks - 1) / ad.chunks, lo = blockIdx.y * per, hi = min(n2, lo + per);
     const int a0 = blockIdx.z * kFaWarps * kFaPts + warp;
     R nh[kFaPts], nl[kFaPts], acc[kFaPts][8];
@@ -179,8 +157,7 @@ __global__ void __launch_bounds__(kFaThreads) fa_pixels_kernel(FieldGrid f, Fiel
     }
 }
 
-// G[a][b][parity s x parity t], or for a sum over the directions themselves
-// [sign of s][sign of t][a][b]: the columns (rows) gathered onto the other
+// G[a][b][parity s x parity t]: the columns (rows) gathered onto the other
 // direction's points.  Block: one point of the per-pixel direction; it adds the
 // chunks of kFaCols columns in shared memory, then a warp sums kFaColPts points
 // over them, its lanes along the columns.  (Five points per warp, so that one block
@@ -257,31 +234,9 @@ __global__ void __launch_bounds__(kFaThreads) fa_columns_kernel(FieldGrid f, Fie
                 g[2 * d] = f.uniform ? acc[k][2 * d] : acc[k][2 * e];
                 g[2 * d + 1] = f.uniform ? acc[k][2 * d + 1] : acc[k][2 * e + 1];
             }
-            if (ad.points) {
-                // the weights of the four mirrored directions
-                R *out = (R *)ad.G + ((size_t)a * f.Ht + b) * 2;
-                const size_t plane = 2 * (size_t)f.Hs * f.Ht;
+            R *out = (R *)ad.G + ((size_t)a * f.Ht + b) * 8;
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const R se = g[c] + g[2 + c], de = g[c] - g[2 + c], so = g[4 + c] + g[6 + c], dd = g[4 + c] - g[6 + c];
-                    out[c] = (R)0.25 * (se + so);
-                    out[plane + c] = (R)0.25 * (de + dd);
-                    out[2 * plane + c] = (R)0.25 * (se - so);
-                    out[3 * plane + c] = (R)0.25 * (de - dd);
-                }
-                // the largest magnitude (non-negative floats order like their bits)
-                float most = 0.f;
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    const float x = (float)out[m * plane], y = (float)out[m * plane + 1];
-                    most = fmaxf(most, sqrtf(x * x + y * y));
-                }
-                atomicMax(ad.gmax, __float_as_uint(most));
-            } else {
-                R *out = (R *)ad.G + ((size_t)a * f.Ht + b) * 8;
-#pragma unroll
-                for (int c = 0; c < 8; ++c) out[c] = g[c];
-            }
+            for (int c = 0; c < 8; ++c) out[c] = g[c];
         }
     }
 }
@@ -492,11 +447,6 @@ static cudaError_t fa_run(const FieldGrid &f, const FieldGridAdjoint &ad, const 
     return ry == 3   ? fa_run_y<R, 3>(f, ad, S, st)
            : ry == 4 ? fa_run_y<R, 4>(f, ad, S, st)
                      : fa_run_y<R, 6>(f, ad, S, st);
-}
-
-cudaError_t launch_field_grid_gather(const FieldGrid &f, const FieldGridAdjoint &ad, const float2 *A, const float *w,
-                                     cudaStream_t st) {
-    return fa_gather<float>(f, ad, A, w, st);
 }
 
 cudaError_t launch_field_grid_adjoint(const FieldGrid &f, const FieldGridAdjoint &ad, const void *A, const void *w,

@@ -223,10 +223,7 @@ struct FieldGrid {
 // Buffers of the adjoint through the grid (field_grid_adjoint.cu), one allocation.
 struct FieldGridAdjoint {
     int chunks = 0;                 // of the per-pixel direction
-    bool points = false;            // G holds every direction's weight, for the tensor-core sum over the directions
     void *B = nullptr, *G = nullptr, *T = nullptr;      // pixels gathered along it; onto the grid; x/z sums
-    double *q = nullptr;            // the directions' q (points only)
-    unsigned *gmax = nullptr;       // receives max |G| as float bits (points only)
 };
 
 }  // namespace scm
@@ -283,8 +280,7 @@ struct scatman_handle {
     float2 *d_adj_coef = nullptr;   // order mode: a[j][n] = e^{+i q_c z_j} eps_n i^n J_n(D z_j), [nz][N]
     float2 *d_adj_ord = nullptr;    // order mode: the orders' fields S~ [N][nx][ny]
     float4 *d_adj_tab = nullptr;    // tensor-core adjoint: per-pixel constants (built at the first backward)
-    uint8_t *d_adj_rtile = nullptr; // tensor-core adjoint: y-phase operand tiles (built at the first backward),
-                                    // then their low halves where it runs over the grid's directions
+    uint8_t *d_adj_rtile = nullptr; // tensor-core adjoint: y-phase operand tiles (built at the first backward)
     // map shapes: device copies of the last voxelised map (grown as needed)
     double *d_rmap = nullptr;
     float *d_rmapf = nullptr;
@@ -410,11 +406,7 @@ cudaError_t launch_field_grid_tc(const FieldGrid &f, int Nxp, const int *bounds,
 // Whether a handle of this configuration runs its adjoint through the grid.
 bool use_field_grid_adjoint(const scatman_config &c, FieldGrid *f);
 // The adjoint field (field_grid_adjoint.cu); layout: buffer offsets from base, returns the bytes.
-size_t field_grid_adjoint_layout(const FieldGrid &f, bool points, FieldGridAdjoint *a, unsigned char *base);
-cudaError_t launch_field_grid_points(const FieldGrid &f, double *q, cudaStream_t st);
-// The pixels' weights gathered onto the grid's directions only (ad.points).
-cudaError_t launch_field_grid_gather(const FieldGrid &f, const FieldGridAdjoint &ad, const float2 *A, const float *w,
-                                     cudaStream_t st);
+size_t field_grid_adjoint_layout(const FieldGrid &f, FieldGridAdjoint *a, unsigned char *base);
 cudaError_t launch_field_grid_adjoint(const FieldGrid &f, const FieldGridAdjoint &ad, const void *A, const void *w,
                                       void *S, cudaStream_t st);
 // Real flops one contraction launch issues for the recorded slice geometry
@@ -448,17 +440,15 @@ bool adjoint_tc_supported(int nx, int ny);
 // nz: slices, or in order mode (orders != 0) the number N of Jacobi-Anger orders;
 // S receives the slices' (or orders') fields [nz][nx][ny].
 int adjoint_tc_splits(long long n_pix, int nz, int sm_count, bool orders);
-// rtile_lo: the low halves of the y-phase tiles, for split operands (null: one product); w null: 1.
-cudaError_t launch_adjoint_tc(const float2 *A, const float *w, const float4 *tab, const uint8_t *rtile,
-                              const uint8_t *rtile_lo, long long n_pix, int nx, int ny, int nz, int orders, double voxel, int splits, float2 *partial,
+cudaError_t launch_adjoint_tc(const float2 *A, const float *w, const float4 *tab, const uint8_t *rtile, long long n_pix,
+                              int nx, int ny, int nz, int orders, double voxel, int splits, float2 *partial,
                               unsigned *gmax_bits, float2 *S, int *err, cudaStream_t st);
 // Order mode: the slices' fields from the orders' (coef: [nz][N] complex).
 cudaError_t launch_adj_orders_combine(const float2 *Sord, const float2 *coef, int N, int nz, int nx, int ny, float2 *S,
                                       cudaStream_t st);
 // The adjoint's y-phase operand tiles (once per handle).
 size_t adj_rtile_bytes(long long n_pix, int ny);
-cudaError_t launch_adj_rtile(const float4 *tab, long long n_pix, int ny, double voxel, bool lo, uint8_t *rt,
-                             cudaStream_t st);
+cudaError_t launch_adj_rtile(const float4 *tab, long long n_pix, int ny, double voxel, uint8_t *rt, cudaStream_t st);
 // Per-pixel constants of the tensor-core adjoint (3 float4 per pixel), once per handle.
 // orders != 0: order mode with theta = acos((q_z - qc) inv_d) in place of q_z.
 cudaError_t launch_adj_pixel_table(const double *q, long long n, double voxel, int orders, double qc, double inv_d,

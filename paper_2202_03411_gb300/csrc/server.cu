@@ -356,7 +356,7 @@ long long scatman_footprint_bytes(const scatman_config *c) {
     FieldGrid fg;
     FieldGridAdjoint fga;
     const bool adj_on_grid = use_field_grid_adjoint(*c, &fg);
-    if (adj_on_grid) b += round_2mib((long long)field_grid_adjoint_layout(fg, tc && adjoint_tc_supported(c->nx, c->ny), &fga, nullptr));
+    if (adj_on_grid) b += round_2mib((long long)field_grid_adjoint_layout(fg, &fga, nullptr));
     if (use_field_grid(*c, &fg) || adj_on_grid) // the field's sample grid: phases, sums, weights
         b += round_2mib((long long)field_grid_layout(&fg, tc, (c->nx + 15) / 16 * 16, nullptr));
     b += round_2mib(nvox * cx);                 // adjoint field (backward)

@@ -138,3 +138,41 @@ def test_fit_handles_keep_the_peak_direct(shape, peak):
     d = np.linalg.norm(out[0][at] - out[1][at]) / np.linalg.norm(out[1][at])
     assert d < 5e-7, d
     assert np.linalg.norm(out[0] - out[1]) / np.linalg.norm(out[1]) < 1e-4
+
+
+def _fit_gradient(g, s, target_shape, prec, q_list=None):
+    """I and the gradient of sum (I - t)^2, with t the pattern of `target_shape` in FP32."""
+    import torch
+    import paper_2202_03411_gb300 as sm
+    h = sm.scatman_create(g, "fp32")
+    t = torch.empty(g.n_pix, device="cuda")
+    sm.scatman_voxelise(h, target_shape)
+    sm.scatman_forward(h, t)
+    sm.scatman_sync(h)
+    q = sm.scatman_get_q(h)
+    h.close()
+    h = sm.scatman_create(g, prec, soft=True, soft_width=0.5, q_list=q if q_list else None)
+    I = torch.empty(g.n_pix, device="cuda")
+    sm.scatman_voxelise(h, s)
+    sm.scatman_forward(h, I)
+    sm.scatman_sync(h)
+    grad = sm.scatman_backward(h, 2 * (I - t))
+    h.close()
+    return I.cpu().numpy(), grad
+
+
+@pytest.mark.parametrize("prec", ["tc_f16_split", "tc_bf16_split", "tc_bf16"])
+def test_tensor_core_fit_gradient_is_the_pixel_sum(prec):
+    """A served fit (48^3 on 128^2 pixels) near its target: the upstream weight cancels,
+    so the gradient shows the adjoint's operand roundings (1e-4 of it between the sum
+    over the pixels and one over the grid's directions).  The detector's pixels
+    and the same pixels as a list of q take the same sums: bit for bit equal."""
+    g = Geometry(48, 48, 48, 1.0, 10.0, 45.0, 128, 128)
+    rng = np.random.default_rng(5)
+    s = Shape(SPHHARM, R0=14.4, lmax=6, alm=random_alm(rng, 6), delta=0.012, beta=0.0012, latitude=25, longitude=-130,
+              rotation=70)
+    near = Shape(SPHERE, r=14.6, delta=0.012, beta=0.0012)
+    I, grad = _fit_gradient(g, s, near, prec)
+    I_q, grad_q = _fit_gradient(g, s, near, prec, q_list=True)
+    assert np.array_equal(I, I_q)
+    assert np.any(grad != 0) and np.array_equal(grad, grad_q)
