@@ -375,9 +375,7 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
     int rc;
     h->adj_on_grid = use_field_grid_adjoint(*cfg, &h->fg);      // (the same plan)
     h->on_grid = use_field_grid(*cfg, &h->fg);
-    h->peak_direct = h->on_grid && h->tensor_core && c.soft;
-    const bool direct = !h->on_grid || h->peak_direct;          // some pixels' sums run over their own q
-    if (direct && (rc = alloc_dev(h, (void **)&h->d_q, npix * 3 * sizeof(double), "q buffer"))) return fail(rc);
+    if (!h->on_grid && (rc = alloc_dev(h, (void **)&h->d_q, npix * 3 * sizeof(double), "q buffer"))) return fail(rc);
     if ((rc = alloc_dev(h, (void **)&h->d_chi, nvox * sizeof(float), "occupancy buffer"))) return fail(rc);
     // per-slice occupied boxes (every mode skips the empty parts of each
     // slice), then the tensor-core kernel's occupied-slice list
@@ -400,11 +398,7 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
     if (h->uniform_tc &&
         (rc = alloc_dev(h, (void **)&h->d_uq_qrow, (size_t)c.det_ny * 3 * sizeof(double), "detector row q")))
         return fail(rc);
-    if (h->peak_direct) {
-        if ((rc = alloc_dev(h, (void **)&h->d_tail, tc_tail_part_bytes_any(h->n_pix, h->sm_count),
-                            "tail partial fields")))
-            return fail(rc);
-    } else if (h->on_grid) {
+    if (h->on_grid) {
         // (its sums live in the grid's own buffers)
     } else if (h->uniform_tc) {
         const size_t hb = uq_tc_h_bytes(c.nx, c.nz, c.det_ny);
@@ -428,7 +422,7 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
                         "q upload");
         if (rc) return fail(rc);
         if ((rc = check_cuda(h, cudaStreamSynchronize(h->stream), "q upload"))) return fail(rc);
-    } else if (direct) {
+    } else if (!h->on_grid) {
         if ((rc = fill_detector_q(h))) return fail(rc);
     }
     if (h->tensor_core) {
@@ -856,35 +850,6 @@ int scatman_voxelise(scatman_handle *h, const scatman_shape *s) {
     return SCATMAN_OK;
 }
 
-// The pixels around the forward direction that hold a parametric shape's central
-// peak, |q| r < 4.5 with r its smallest half-width (up to a sphere's first zero;
-// beyond it its intensity is below 0.8 % of the peak's); none for a map.  A fit's
-// loss is the difference between the pattern and a measured one that nearly equals
-// it, twenty times smaller and more, and its value and gradient are set in the
-// peak: there the 16-bit phase pairs' rounding, 1e-6 of the intensity and another
-// for the grid's directions than for the pixel's own, would move the loss by 4e-5
-// (measured, 96^3 on 256^2; with the peak's sums direct 1e-6), and a nearly
-// cancelling gradient by as much already from a rim at 3.3 (7 % of the peak).
-static PixelRect peak_pixels(const scatman_handle *h) {
-    const scatman_config &c = h->cfg;
-    const scatman_shape &s = h->shape;
-    double r = 0.0;
-    if (s.kind == SCATMAN_SPHERE) r = s.r;
-    if (s.kind == SCATMAN_ELLIPSOID) r = std::fmin(s.a, std::fmin(s.b, s.c));
-    if (s.kind == SCATMAN_SPHHARM) r = s.R0;
-    PixelRect p;
-    if (!(r > 0.0)) return p;
-    const double sn = 4.5 / (r * 2.0 * h->k0);                   // sin(theta / 2) at the rim
-    const double X = sn < 0.7 ? std::tan(2.0 * std::asin(sn)) / std::tan(c.theta_max_deg * kPi / 180.0) : 1.0;
-    auto margin = [&](int n) { return X < 1.0 ? (int)std::floor(0.5 * ((n - 1) - X * n)) : 0; };
-    p.u0 = std::max(0, margin(c.det_nx));
-    p.v0 = std::max(0, margin(c.det_ny));
-    p.w = c.det_nx - 2 * p.u0;
-    p.h = c.det_ny - 2 * p.v0;
-    p.det_nx = c.det_nx;
-    return p;
-}
-
 int scatman_forward(scatman_handle *h, void *I_dev, void *A_dev) {
     const StageRange nvtx_range("scatman_forward");
     if (!h || !I_dev) return set_error(h, SCATMAN_ERR_ARG, "I_dev is NULL");
@@ -892,20 +857,13 @@ int scatman_forward(scatman_handle *h, void *I_dev, void *A_dev) {
     const scatman_config &c = h->cfg;
     const double str_re = h->str_re, str_im = h->str_im;     // set by voxelise
     cudaError_t e;
-    const PixelRect peak = h->peak_direct ? peak_pixels(h) : PixelRect();
-    // (a peak over more than half of the detector: every pixel's sums are direct)
-    const bool on_grid = h->on_grid && 2ll * peak.w * peak.h < h->n_pix;
-    if (on_grid && h->tensor_core) {
+    if (h->on_grid && h->tensor_core) {
         e = launch_rows_y_tc(h->tmap_B, h->fg.qrow, 2 * h->fg.Hs, c.nx, c.ny, c.nz, h->Nxp, h->Nyp, c.voxel, h->split,
                              h->s_bf16, h->d_bounds, (float2 *)h->fg.H, h->d_err, h->sm_count, h->stream);
         if (e == cudaSuccess)
             e = launch_field_grid_tc(h->fg, h->Nxp, h->d_bounds, geom_chunk_y(h->d_bounds, c.nz), str_re, str_im,
                                      (float2 *)h->d_A, (float *)I_dev, h->sm_count, h->stream);
-        if (e == cudaSuccess && peak.w > 0)
-            e = launch_msft_tc(h->tmap_B, h->d_q, h->n_pix, c.nx, c.ny, c.nz, h->Nxp, h->Nyp, c.voxel, str_re, str_im,
-                               h->split, h->bf16, h->d_bounds, (float2 *)h->d_A, (float *)I_dev, h->d_err, h->sm_count,
-                               h->stream, h->d_tail, peak);
-    } else if (on_grid) {
+    } else if (h->on_grid) {
         e = launch_field_grid(h->fg, h->d_s, h->d_bounds, str_re, str_im, h->d_A, I_dev, h->sm_count, h->stream);
     } else if (h->uniform_tc) {
         // the y sum writes only occupied slices and x spans: the rest of H is zero

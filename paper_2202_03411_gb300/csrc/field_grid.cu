@@ -138,15 +138,21 @@ bool plan_field_grid(const scatman_config &c, bool fp64, FieldGrid *f) {
 // 128^2; 48 / 47 at 96^3 on 64^2, 46 / 56 on 96^2; and where the grid has more points
 // than the detector has pixels (60 degrees, wavelength 6) 58 / 47 at 96^3 on 64^2,
 // 68 / 84 at 128^3 on 96^2.
-// Fits in the split phases keep their pattern's peak on the direct sums
-// (api.cu), and a small problem's other pixels too: the gradient of a nearly
-// cancelling loss sees their rounding (3e-5 at 64^3 on 128^2).
+// Fits in the split phases sum over the pixels themselves, as their adjoint does:
+// the 16-bit phase pairs round to 1e-6 of the intensity, and to another 1e-6 at the
+// grid's directions.  A loss near its minimum, and more so a gradient that nearly
+// cancels, shows that 25 to 100 times larger: with only the pattern's peak
+// summed directly, served gradients of 96^3 and 128^3 still moved by up to 7e-5
+// (by more than 2e-5 in 4 of 40 batches), and a 96^3 fit's on 256^2 by 1.9e-5.  The
+// price: 8.5 ms instead of 2.8 for the 12 mixed server requests, 842 us instead of
+// 614 for a fit step of 96^3 on 256^2 (forward and adjoint together).
 bool use_field_grid(const scatman_config &c, FieldGrid *f) {
     const bool split = c.precision == SCATMAN_TC_F16_SPLIT || c.precision == SCATMAN_TC_BF16_SPLIT;
     const bool plain = c.precision == SCATMAN_FP64 || c.precision == SCATMAN_FP32;
     if (c.q_list || !(plain || (split && c.detector == SCATMAN_DETECTOR_FLAT))) return false;
+    if (split && c.soft) return false;
     const double pixels = (double)c.det_nx * c.det_ny, terms = pixels * ((double)c.nx * c.ny * c.nz);
-    if (plain ? pixels < 128.0 : terms < (c.soft ? 2e10 : 5e8)) return false;
+    if (plain ? pixels < 128.0 : terms < 5e8) return false;
     if (!plan_field_grid(c, c.precision == SCATMAN_FP64, f)) return false;
     if (split && terms < 8e9 && pixels < 2.4 * f->Hs * f->Ht) return false;
     // FP32 fits: a loss near its minimum shows the pattern's rounding many times

@@ -195,11 +195,6 @@ struct SliceOut {
     float *rtab;                    // their radius table
 };
 
-// A rectangle of the detector's pixels (w = 0: all of them).
-struct PixelRect {
-    int u0 = 0, v0 = 0, w = 0, h = 0, det_nx = 0;
-};
-
 // The field's sample grid on the Ewald sphere (field_grid.cu): sizes, then
 // device buffers in one allocation.  Passed to its kernels by value.
 struct FieldGrid {
@@ -301,7 +296,6 @@ struct scatman_handle {
     double str_re = 0, str_im = 0;  // global strength factor of s: n^2 - 1, or the map's index scale
     double map_index_max = 0;       // max |delta|, |beta| over a volume map's cells
     bool on_grid = false;           // the field goes through its sample grid
-    bool peak_direct = false;       // (fits in the tensor-core modes) except the pattern's peak
     scm::FieldGrid fg;
     unsigned char *d_fg = nullptr;  // its buffers
     bool adj_on_grid = false;       // the adjoint goes through the grid
@@ -367,14 +361,12 @@ double simt_issued_flops(const int *bounds, int nz, int ny, long long n_pix, boo
 bool tc_grid_ok(int Nxp, int Nyp, bool split);
 // geom: the slice-geometry buffer (slice_geom_ints); tail_part: scratch of
 // tc_tail_part_bytes for the partial fields of the last partial wave's tiles
-// (null: every tile whole).  rect: only those pixels of the detector whose q and
-// n_pix are given (tc_tail_part_bytes_any covers every rectangle).
+// (null: every tile whole).
 cudaError_t launch_msft_tc(const TcMaps &maps, const double *q, long long n_pix, int nx, int ny, int nz,
                            int Nxp, int Nyp, double voxel, double str_re, double str_im, bool split,
                            bool bf16, int *geom, float2 *A, float *I, int *err,
-                           int sm_count, cudaStream_t st, float2 *tail_part, const PixelRect &rect = PixelRect());
+                           int sm_count, cudaStream_t st, float2 *tail_part);
 size_t tc_tail_part_bytes(long long n_pix, int sm_count);
-size_t tc_tail_part_bytes_any(long long n_pix, int sm_count);
 // The same kernel in store mode, the uniform-q detector's y-contraction on the
 // tensor cores: rows are detector rows v (q_y(v) = qrow[3 v + 1]) and G is
 // written to the x/z operand H as 16-bit planes.

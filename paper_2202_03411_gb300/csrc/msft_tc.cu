@@ -88,7 +88,6 @@ struct TcParams {
     float2 *A;
     float *I;
     int *err;
-    PixelRect rect;             // the pixels are this part of the detector (w = 0: all, in order)
     // store mode (the uniform-q detector's y-contraction): rows m are detector
     // rows v with q_y(v) = q[3 v + 1]; G is written as 16-bit planes
     // [-Im | Re | Im] of H at rows (3 (v / h_Rg) + plane) h_Jg + (v % h_Rg) h_Jp + j
@@ -210,11 +209,6 @@ __global__ void __launch_bounds__(256) pack_units_kernel(const int *cy, int nz, 
         __syncthreads();
     }
     if (threadIdx.x == 0) list[0] = make_uint2((uint32_t)s_base, 0u);
-}
-
-// The detector's pixel behind pixel p of the launch.
-__host__ __device__ inline long long pixel_at(const PixelRect &r, long long p) {
-    return r.w > 0 ? (r.v0 + p / r.w) * r.det_nx + r.u0 + p % r.w : p;
 }
 
 // Tile, part (-1: whole tile) and unit range [i_lo, i_hi) of work unit u.
@@ -546,10 +540,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         if (blockIdx.x < (unsigned)P.num_units) {
             const long long p0 = (long long)unit_info(P, blockIdx.x, n_list).mt * kBM + m;
             if (p0 < P.n_pix) {
-                const double *q = P.q + 3 * pixel_at(P.rect, p0);
-                nq0 = q[0];
-                nq1 = q[1];
-                nq2 = q[2];
+                nq0 = P.q[3 * p0];
+                nq1 = P.q[3 * p0 + 1];
+                nq2 = P.q[3 * p0 + 2];
             }
         }
         for (int u = blockIdx.x; u < P.num_units; u += gridDim.x) {
@@ -561,10 +554,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if (u + (int)gridDim.x < P.num_units) {
                 const long long pn = (long long)unit_info(P, u + gridDim.x, n_list).mt * kBM + m;
                 if (pn < P.n_pix) {
-                    const double *q = P.q + 3 * pixel_at(P.rect, pn);
-                    nq0 = q[0];
-                    nq1 = q[1];
-                    nq2 = q[2];
+                    nq0 = P.q[3 * pn];
+                    nq1 = P.q[3 * pn + 1];
+                    nq2 = P.q[3 * pn + 2];
                 }
             }
             // The tensor core is done with the previous tile's phase operand:
@@ -666,9 +658,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 float2 a = make_float2(acc.x + o.x, acc.y + o.y);
                 a = cmul(make_float2(P.str_re, P.str_im), a);
                 if (un.part < 0) {
-                    const long long at = pixel_at(P.rect, p);
-                    P.A[at] = a;
-                    P.I[at] = a.x * a.x + a.y * a.y;
+                    P.A[p] = a;
+                    P.I[p] = a.x * a.x + a.y * a.y;
                 } else {
                     const long long tail = (long long)(P.num_m_tiles - P.whole) * kBM;
                     P.Apart[un.part * tail + (long long)(mt - P.whole) * kBM + m] = a;
@@ -704,7 +695,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // Fields of the tiles whose unit lists were cut into parts: A = the parts'
 // sum in part order, I = |A|^2.
 __global__ void tc_tail_sum_kernel(const float2 *__restrict__ Apart, int parts, long long tail, long long p0,
-                                   long long n_pix, PixelRect rect, float2 *__restrict__ A, float *__restrict__ I) {
+                                   long long n_pix, float2 *__restrict__ A, float *__restrict__ I) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= tail || p0 + t >= n_pix) return;
     float2 a = Apart[t];
@@ -713,9 +704,8 @@ __global__ void tc_tail_sum_kernel(const float2 *__restrict__ Apart, int parts, 
         a.x += b.x;
         a.y += b.y;
     }
-    const long long at = pixel_at(rect, p0 + t);
-    A[at] = a;
-    I[at] = a.x * a.x + a.y * a.y;
+    A[p0 + t] = a;
+    I[p0 + t] = a.x * a.x + a.y * a.y;
 }
 
 // ---- host side ------------------------------------------------------------------
@@ -757,7 +747,7 @@ bool encode_tmap_B(TcMaps *maps, void *base, int Kp, int Nxp, int nz, bool bf16,
 static cudaError_t launch_tc(const TcMaps &maps, const double *q, long long n_pix, int nx, int ny, int nz, int Nxp,
                              int Nyp, double voxel, double str_re, double str_im, bool split, bool bf16, int *geom,
                              float2 *A, float *I, int *err, int sm_count, cudaStream_t st, const UqStore *store,
-                             float2 *tail_part, const PixelRect &rect) {
+                             float2 *tail_part) {
     if (!tc_grid_ok(Nxp, Nyp, split) || nz < 1 || nz > 512 || nx > Nxp || ny > Nyp) return cudaErrorInvalidValue;
     const size_t ring = tc_ring_bytes(Nxp, Nyp, split);
     if (ring == 0) return cudaErrorInvalidValue;
@@ -767,7 +757,6 @@ static cudaError_t launch_tc(const TcMaps &maps, const double *q, long long n_pi
     P.q = q;
     P.list = list;
     P.n_pix = n_pix;
-    P.rect = rect;
     P.nx = nx;
     P.ny = ny;
     P.nz = nz;
@@ -843,7 +832,7 @@ static cudaError_t launch_tc(const TcMaps &maps, const double *q, long long n_pi
         if (P.whole < P.num_m_tiles) {
             const long long tail = (long long)(P.num_m_tiles - P.whole) * kBM;
             tc_tail_sum_kernel<<<(unsigned)((tail + 255) / 256), 256, 0, st>>>(
-                P.Apart, P.parts, tail, (long long)P.whole * kBM, n_pix, P.rect, A, I);
+                P.Apart, P.parts, tail, (long long)P.whole * kBM, n_pix, A, I);
         }
     }
     return cudaGetLastError();
@@ -856,24 +845,19 @@ size_t tc_tail_part_bytes(long long n_pix, int sm_count) {
     return (size_t)(rem * kBM * kTcMaxTailParts) * sizeof(float2);
 }
 
-size_t tc_tail_part_bytes_any(long long n_pix, int sm_count) {
-    const long long tiles = (n_pix + kBM - 1) / kBM, most = tiles < sm_count ? tiles : sm_count;
-    return (size_t)(most * kBM * kTcMaxTailParts) * sizeof(float2);
-}
-
 cudaError_t launch_msft_tc(const TcMaps &maps, const double *q, long long n_pix, int nx, int ny, int nz,
                            int Nxp, int Nyp, double voxel, double str_re, double str_im, bool split,
                            bool bf16, int *geom, float2 *A, float *I, int *err,
-                           int sm_count, cudaStream_t st, float2 *tail_part, const PixelRect &rect) {
-    return launch_tc(maps, q, rect.w > 0 ? (long long)rect.w * rect.h : n_pix, nx, ny, nz, Nxp, Nyp, voxel, str_re,
-                     str_im, split, bf16, geom, A, I, err, sm_count, st, nullptr, tail_part, rect);
+                           int sm_count, cudaStream_t st, float2 *tail_part) {
+    return launch_tc(maps, q, n_pix, nx, ny, nz, Nxp, Nyp, voxel, str_re, str_im, split, bf16, geom, A, I, err,
+                     sm_count, st, nullptr, tail_part);
 }
 
 cudaError_t launch_uq_y_tc_mma(const TcMaps &maps, const double *qrow, int det_ny, int nx, int ny, int nz, int Nxp,
                                int Nyp, double voxel, bool split, bool bf16, int *geom, const UqStore &store,
                                int *err, int sm_count, cudaStream_t st) {
     return launch_tc(maps, qrow, det_ny, nx, ny, nz, Nxp, Nyp, voxel, 1.0, 0.0, split, bf16, geom, nullptr,
-                     nullptr, err, sm_count, st, &store, nullptr, PixelRect());
+                     nullptr, err, sm_count, st, &store, nullptr);
 }
 
 cudaError_t launch_rows_y_tc(const TcMaps &maps, const double *qrow, int rows, int nx, int ny, int nz, int Nxp,
@@ -883,7 +867,7 @@ cudaError_t launch_rows_y_tc(const TcMaps &maps, const double *qrow, int rows, i
     store.H32 = H;
     store.Rg = 1;
     return launch_tc(maps, qrow, rows, nx, ny, nz, Nxp, Nyp, voxel, 1.0, 0.0, split, bf16, geom, nullptr, nullptr,
-                     err, sm_count, st, &store, nullptr, PixelRect());
+                     err, sm_count, st, &store, nullptr);
 }
 
 }  // namespace scm

@@ -176,3 +176,21 @@ def test_tensor_core_fit_gradient_is_the_pixel_sum(prec):
     I_q, grad_q = _fit_gradient(g, s, near, prec, q_list=True)
     assert np.array_equal(I, I_q)
     assert np.any(grad != 0) and np.array_equal(grad, grad_q)
+
+
+@pytest.mark.parametrize("shape", [
+    Shape(SPHERE, r=30.0, delta=0.01, beta=0.001),
+    Shape(SPHHARM, R0=30.0, lmax=2, alm=np.array([0, 0, 0, 0, 0, 0, -0.35, 0, 0.25]), delta=0.01, beta=0.001,
+          latitude=35, longitude=20, rotation=10),              # 0.75 R0 across its thinnest axis
+])
+@pytest.mark.parametrize("prec", ["tc_f16_split", "tc_bf16_split"])
+def test_split_phase_fit_is_the_pixel_sum(shape, prec):
+    """The pattern of a fit of 96^3 on 256^2, where a forward pass without soft occupancy
+    goes through the grid: the phase pairs' roundings of every pixel are its
+    own, and so are loss and gradient near the target (bit for bit)."""
+    g = Geometry(96, 96, 96, 1.0, 10.0, 45.0, 256, 256)
+    near = Shape(SPHERE, r=30.3, delta=0.01, beta=0.001)
+    I, grad = _fit_gradient(g, shape, near, prec)
+    I_q, grad_q = _fit_gradient(g, shape, near, prec, q_list=True)
+    assert I.max() > 0 and np.array_equal(I, I_q)
+    assert np.any(grad != 0) and np.array_equal(grad, grad_q)
