@@ -288,13 +288,27 @@ static int need_q(scatman_handle *h) {
 }
 
 // The sample grid's buffers and tables.
-static int need_field_grid(scatman_handle *h) {
-    if (h->d_fg) return SCATMAN_OK;
-    int rc = alloc_dev(h, (void **)&h->d_fg, field_grid_layout(&h->fg, h->tensor_core, h->Nxp, nullptr),
-                       "field sample grid");
+static int make_field_grid(scatman_handle *h) {
+    int rc = alloc_dev(h, (void **)&h->d_fg, field_grid_layout(&h->fg, true, h->Nxp, nullptr), "field sample grid");
     if (rc) return rc;
-    field_grid_layout(&h->fg, h->tensor_core, h->Nxp, h->d_fg);
+    field_grid_layout(&h->fg, true, h->Nxp, h->d_fg);
     return check_cuda(h, launch_field_grid_tables(h->fg, h->stream), "field sample grid");
+}
+
+// The adjoint's (once).
+static int need_adjoint_grid(scatman_handle *h) {
+    if (h->d_fga) return SCATMAN_OK;
+    const FieldGrid *fwd = h->on_grid ? &h->fg : nullptr;
+    unsigned char *d = nullptr;
+    int rc = alloc_dev(h, (void **)&d, field_grid_adjoint_layout(&h->fg_adj, fwd, &h->fga, nullptr), "adjoint sample grid");
+    if (rc) return rc;
+    field_grid_adjoint_layout(&h->fg_adj, fwd, &h->fga, d);
+    if (h->fga.own && (rc = check_cuda(h, launch_field_grid_tables(h->fg_adj, h->stream), "adjoint sample grid"))) {
+        cudaFree(d);
+        return rc;
+    }
+    h->d_fga = d;
+    return SCATMAN_OK;
 }
 
 int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle **out) {
@@ -373,7 +387,7 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
     const size_t npix = (size_t)h->n_pix;
     const bool f64 = (h->precision == SCATMAN_FP64);
     int rc;
-    h->adj_on_grid = use_field_grid_adjoint(*cfg, &h->fg);      // (the same plan)
+    h->adj_on_grid = use_field_grid_adjoint(*cfg, &h->fg_adj);
     h->on_grid = use_field_grid(*cfg, &h->fg);
     if (!h->on_grid && (rc = alloc_dev(h, (void **)&h->d_q, npix * 3 * sizeof(double), "q buffer"))) return fail(rc);
     if ((rc = alloc_dev(h, (void **)&h->d_chi, nvox * sizeof(float), "occupancy buffer"))) return fail(rc);
@@ -392,7 +406,7 @@ int scatman_create(const scatman_config *cfg, void *cuda_stream, scatman_handle 
     const size_t cx = f64 ? sizeof(double2) : sizeof(float2);
     if ((rc = alloc_dev(h, &h->d_A, npix * cx, "field buffer"))) return fail(rc);
     if ((rc = alloc_dev(h, &h->d_I, npix * (f64 ? 8 : 4), "intensity buffer"))) return fail(rc);
-    if (h->on_grid && (rc = need_field_grid(h))) return fail(rc);
+    if (h->on_grid && (rc = make_field_grid(h))) return fail(rc);
     if (h->uniform_q && !h->on_grid && (rc = alloc_dev(h, (void **)&h->d_uq_qz, npix * sizeof(float2), "q_z table")))
         return fail(rc);
     if (h->uniform_tc &&
@@ -1237,14 +1251,8 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
     }
     if (!h->adj_on_grid && (rc = need_q(h))) return rc;      // sums over the pixels
     if (h->adj_on_grid) {
-        if ((rc = need_field_grid(h))) return rc;
-        if (!h->d_fga) {
-            if ((rc = alloc_dev(h, (void **)&h->d_fga, field_grid_adjoint_layout(h->fg, &h->fga, nullptr),
-                                "adjoint sample grid")))
-                return rc;
-            field_grid_adjoint_layout(h->fg, &h->fga, h->d_fga);
-        }
-        rc = check_cuda(h, launch_field_grid_adjoint(h->fg, h->fga, h->d_A, dLdI_dev, h->d_S, h->stream),
+        if ((rc = need_adjoint_grid(h))) return rc;
+        rc = check_cuda(h, launch_field_grid_adjoint(h->fg_adj, h->fga, h->d_A, dLdI_dev, h->d_S, h->stream),
                         "adjoint field");
         if (rc) return rc;
     } else if (h->tensor_core && adjoint_tc_supported(c.nx, c.ny)) {

@@ -71,10 +71,11 @@ static int plan_points(double k0, double top, double along, double across, doubl
 
 // Half the points of a direction at most (the per-pixel interpolation holds all
 // points of 32 columns in shared memory: 131 KB in FP32, 200 KB in FP64).
-static int fg_max_half(bool fp64) { return fp64 ? 96 : 128; }
+static int fg_max_half(int elem) { return elem == 8 ? 96 : 128; }
 constexpr int kFgMaxSide = 512;          // grid side in x and y
 
-bool plan_field_grid(const scatman_config &c, bool fp64, FieldGrid *f) {
+// elem: bytes of a real number in the sums.
+bool plan_field_grid(const scatman_config &c, int elem, FieldGrid *f) {
     *f = FieldGrid();
     if (c.q_list || c.nx > kFgMaxSide || c.ny > kFgMaxSide) return false;
     const bool uniform = c.detector == SCATMAN_DETECTOR_UNIFORM_Q;
@@ -100,9 +101,10 @@ bool plan_field_grid(const scatman_config &c, bool fp64, FieldGrid *f) {
     const double hyp = std::hypot(Lx, Lz);
     // max over |t| <= tm of |t| Lx + sqrt(1 - t^2) Lz
     const double across = hyp > 0.0 && Lx / hyp <= tm ? hyp : tm * Lx + std::sqrt(1.0 - tm * tm) * Lz;
+    const bool fp64 = c.precision == SCATMAN_FP64;
     const double tol = fp64 ? 1e-12 : 1e-5;
     const int Ns = plan_points(k0, sm, Ly, across, tol), Nt = plan_points(k0, tm, Lx, Lz, tol);
-    if (Ns > 2 * fg_max_half(fp64) || Nt > 2 * fg_max_half(fp64)) return false;
+    if (Ns > 2 * fg_max_half(elem) || Nt > 2 * fg_max_half(elem)) return false;
     f->uniform = uniform;
     f->Hs = Ns / 2;
     f->Ht = Nt / 2;
@@ -124,7 +126,8 @@ bool plan_field_grid(const scatman_config &c, bool fp64, FieldGrid *f) {
     f->H2 = uniform ? f->Ht : f->Hs;
     f->n1 = uniform ? f->V : f->U;
     f->jc = (c.nz + kFgSlices - 1) / kFgSlices;
-    f->elem = fp64 ? 8 : 4;
+    f->elem = elem;
+    f->io = fp64 ? 8 : 4;
     return true;
 }
 
@@ -138,6 +141,16 @@ bool plan_field_grid(const scatman_config &c, bool fp64, FieldGrid *f) {
 // 128^2; 48 / 47 at 96^3 on 64^2, 46 / 56 on 96^2; and where the grid has more points
 // than the detector has pixels (60 degrees, wavelength 6) 58 / 47 at 96^3 on 64^2,
 // 68 / 84 at 128^3 on 96^2.
+// FP32 fits sum over the voxels and interpolate in FP64 (slices, field and pattern stay
+// FP32).  A loss near its minimum shows the pattern's rounding many times larger: over
+// 63 fits of 20^3 - 64^3 voxels the FP32 sums left the loss 7.0e-7 off (the direct
+// FP32 sums 5.4e-7), these 3.4e-7, most of it the slices' own FP32; the pattern 2.1e-7
+// (3.1e-7) and 6e-8.  A fit step of 48^3 on 128^2 takes 530 us instead of 515.  Where the
+// points exceed the FP64 plan's limit the sums stay FP32.
+// Patterns in FP32 keep FP32 sums: 2.1e-7 of the intensity off on the flat detector (the
+// direct sums 2.9e-7), 2.0e-7 on the uniform-q one (its separable sums 1.3e-7: the
+// alternating weights of the interpolation; 1.5e-7 at 67 us instead of 31 with only the
+// pixels' own sums in FP32, 3e-8 at 153 us all in FP64, 30^3 on 512^2).
 // Fits in the split phases sum over the pixels themselves, as their adjoint does:
 // the 16-bit phase pairs round to 1e-6 of the intensity, and to another 1e-6 at the
 // grid's directions.  A loss near its minimum, and more so a gradient that nearly
@@ -153,12 +166,9 @@ bool use_field_grid(const scatman_config &c, FieldGrid *f) {
     if (split && c.soft) return false;
     const double pixels = (double)c.det_nx * c.det_ny, terms = pixels * ((double)c.nx * c.ny * c.nz);
     if (plain ? pixels < 128.0 : terms < 5e8) return false;
-    if (!plan_field_grid(c, c.precision == SCATMAN_FP64, f)) return false;
-    if (split && terms < 8e9 && pixels < 2.4 * f->Hs * f->Ht) return false;
-    // FP32 fits: a loss near its minimum shows the pattern's rounding many times
-    // larger.  Dot2 sums halve it, at ten FP32 operations a term instead of one.
-    f->dot2 = c.precision == SCATMAN_FP32 && c.soft;
-    return true;
+    const bool fit = c.precision == SCATMAN_FP32 && c.soft;
+    if (!(fit && plan_field_grid(c, 8, f)) && !plan_field_grid(c, c.precision == SCATMAN_FP64 ? 8 : 4, f)) return false;
+    return !(split && terms < 8e9 && pixels < 2.4 * f->Hs * f->Ht);
 }
 
 // Whether the adjoint runs through the grid: FP32 and FP64, and tensor-core grids
@@ -173,13 +183,14 @@ bool use_field_grid_adjoint(const scatman_config &c, FieldGrid *f) {
     const double pixels = (double)c.det_nx * c.det_ny;
     if (c.q_list || pixels < 128.0) return false;
     if (c.precision != SCATMAN_FP64 && c.precision != SCATMAN_FP32 && adjoint_tc_supported(c.nx, c.ny)) return false;
-    return plan_field_grid(c, c.precision == SCATMAN_FP64, f);
+    return plan_field_grid(c, c.precision == SCATMAN_FP64 ? 8 : 4, f);
 }
 
 static size_t up256(size_t b) { return (b + 255) / 256 * 256; }
 
-// Lays the grid's buffers out from `base` (null: sizes only); returns the bytes.
-size_t field_grid_layout(FieldGrid *f, bool tensor_core, int Nxp, unsigned char *base) {
+// Lays the grid's tables and, for the forward pass, its sums out from `base` (null:
+// sizes only); returns the bytes.  Nxp: row of the tensor-core y-sums (0: none).
+size_t field_grid_layout(FieldGrid *f, bool forward, int Nxp, unsigned char *base) {
     size_t at = 0;
     auto take = [&](size_t bytes) {
         unsigned char *p = base ? base + at : nullptr;
@@ -196,11 +207,11 @@ size_t field_grid_layout(FieldGrid *f, bool tensor_core, int Nxp, unsigned char 
     f->qrow = (double *)take(2 * (size_t)f->Hs * 3 * sizeof(double));
     f->point_s = (double *)take(2 * (size_t)f->Hs * sizeof(double));
     f->point_t = (double *)take(2 * (size_t)f->Ht * sizeof(double));
-    const size_t row = (size_t)(tensor_core && Nxp > f->nx ? Nxp : f->nx);
+    if (!forward) return at;
+    const size_t row = (size_t)(Nxp > f->nx ? Nxp : f->nx);
     f->H = take(2 * (size_t)f->Hs * f->nz * row * 2 * e);
     f->Q = take((size_t)f->jc * f->Hs * f->Ht * 8 * e);
     f->B = take((size_t)f->H2 * 8 * ((f->n1 + 31) / 32 * 32) * e);
-    f->bytes = at;
     return at;
 }
 
@@ -420,8 +431,8 @@ static int fg_rows_per_thread(int n, long long others, bool fp64, int sm_count) 
 // H[a][even, odd][j][x] = sum over y' of cos (q_a y') even s, -i sin (q_a y') odd s.
 // Block: 32 columns x of one slice.  Slices and columns outside the occupied
 // box are not written (and not read later), y' beyond the box is skipped.
-template <typename R, int kRpt>
-__global__ void __launch_bounds__(kFgThreads) fg_y_kernel(FieldGrid f, const typename Fg<R>::C *__restrict__ s,
+template <typename R, typename IO, int kRpt>
+__global__ void __launch_bounds__(kFgThreads) fg_y_kernel(FieldGrid f, const typename Fg<IO>::C *__restrict__ s,
                                                           const int *__restrict__ bounds) {
     using C = typename Fg<R>::C;
     extern __shared__ __align__(32) unsigned char smem[];
@@ -453,10 +464,14 @@ __global__ void __launch_bounds__(kFgThreads) fg_y_kernel(FieldGrid f, const typ
             const int x = x0 + warp * 4 + c, k = k0 + lane;
             sp[c].x = sp[c].y = sm[c].x = sm[c].y = (R)0;
             if (x < f.nx && k < kend) {
-                const C *line = s + ((size_t)j * f.nx + x) * f.ny;
+                const auto *line = s + ((size_t)j * f.nx + x) * f.ny;
                 const int ip = fg_plus(k, f.ny), im = fg_minus(k, f.ny);
-                sp[c] = line[ip];
-                if (im != ip) sm[c] = line[im];
+                sp[c].x = line[ip].x;
+                sp[c].y = line[ip].y;
+                if (im != ip) {
+                    sm[c].x = line[im].x;
+                    sm[c].y = line[im].y;
+                }
             }
         }
     };
@@ -690,16 +705,7 @@ __global__ void __launch_bounds__(256) fg_columns_kernel(FieldGrid f) {
     __syncthreads();
     const R *we = (const R *)f.w1, *wo = we + (size_t)f.H1 * f.n1;
     R acc[8] = {};
-    if (sizeof(R) == 4 && f.dot2) {
-        R low[8] = {};
-        for (int p = warp; i < f.n1 && p < f.H1; p += 8) {
-            const R e = we[(size_t)p * f.n1 + i], o = wo[(size_t)p * f.n1 + i];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) fg_dot2(c < 4 ? e : o, q[p * 8 + c], acc[c], low[c]);
-        }
-#pragma unroll
-        for (int c = 0; c < 8; ++c) acc[c] += low[c];
-    } else if (i < f.n1) {
+    if (i < f.n1) {
 #pragma unroll 4
         for (int p = warp; p < f.H1; p += 8) {
             const R e = we[(size_t)p * f.n1 + i], o = wo[(size_t)p * f.n1 + i];
@@ -733,13 +739,12 @@ __global__ void __launch_bounds__(256) fg_columns_kernel(FieldGrid f) {
 // kSplit (small detectors in FP64, of which a warp runs an operation in 64 cycles): the
 // four warps share one row, each takes a quarter of the points, a quarter of the
 // sums and one of the four mirrored pixels (32^3 on 64^2: 16 us with a warp per row).
-template <typename R, int kPts, bool kUniform, int kWarps, bool kDot2, bool kSplit>
+template <typename R, typename IO, int kPts, bool kUniform, int kWarps, bool kSplit>
 __global__ void __launch_bounds__(32 * kWarps) fg_pixels_out_kernel(FieldGrid f, double str_re, double str_im,
-                                                            typename Fg<R>::C *__restrict__ A, R *__restrict__ I) {
-    using C = typename Fg<R>::C;
+                                                            typename Fg<IO>::C *__restrict__ A, IO *__restrict__ I) {
+    using C = typename Fg<IO>::C;
     using V4 = typename Fg<R>::V4;
     static_assert(!kUniform || kWarps == 4, "a warp per row");
-    using S = typename std::conditional<kDot2, double, R>::type;      // of the last few operations per pixel
     extern __shared__ __align__(32) unsigned char smem[];
     R *sB = reinterpret_cast<R *>(smem);
     V4 *sN = reinterpret_cast<V4 *>(sB + (size_t)f.H2 * 8 * (kUniform ? 4 : 32));
@@ -756,7 +761,7 @@ __global__ void __launch_bounds__(32 * kWarps) fg_pixels_out_kernel(FieldGrid f,
     __syncthreads();
     int u[kPts], v[kPts];
     V4 px[kPts];
-    R acc[kPts][8], low[kPts][8];
+    R acc[kPts][8];
 #pragma unroll
     for (int p = 0; p < kPts; ++p) {
         u[p] = kUniform ? (blockIdx.x * kPts + p) * 32 + lane : blockIdx.x * 32 + lane;
@@ -764,7 +769,7 @@ __global__ void __launch_bounds__(32 * kWarps) fg_pixels_out_kernel(FieldGrid f,
         px[p].x = px[p].y = px[p].z = px[p].w = (R)0;
         if (u[p] < f.U && v[p] < f.V) px[p] = ((const V4 *)f.pix)[(size_t)v[p] * f.U + u[p]];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) acc[p][c] = low[p][c] = (R)0;
+        for (int c = 0; c < 8; ++c) acc[p][c] = (R)0;
     }
 #pragma unroll 2
     for (int a = kSplit ? warp : 0; a < f.H2; a += kSplit ? kWarps : 1) {
@@ -789,16 +794,11 @@ __global__ void __launch_bounds__(32 * kWarps) fg_pixels_out_kernel(FieldGrid f,
         for (int p = 0; p < kPts; ++p) {
             const R r = fg_recip(px[p].x, px[p].y, n.x, n.y);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                if (kDot2)
-                    fg_dot2(r, b[c], acc[p][c], low[p][c]);
-                else
-                    acc[p][c] = fma(r, b[c], acc[p][c]);
-            }
+            for (int c = 0; c < 8; ++c) acc[p][c] = fma(r, b[c], acc[p][c]);
         }
     }
     if constexpr (kSplit) {
-        static_assert(kPts == 1 && kWarps == 4 && !kUniform && !kDot2, "a quarter each");
+        static_assert(kPts == 1 && kWarps == 4 && !kUniform, "a quarter each");
         __shared__ R part[4][8][32];
 #pragma unroll
         for (int c = 0; c < 8; ++c) part[warp][c][lane] = acc[0][c];
@@ -816,15 +816,15 @@ __global__ void __launch_bounds__(32 * kWarps) fg_pixels_out_kernel(FieldGrid f,
     for (int p = 0; p < kPts; ++p) {
         if (u[p] >= f.U || v[p] >= f.V) continue;
         const bool off = !(px[p].z == px[p].z);          // no scattering direction: A = 0
-        const S we = px[p].w, wo = (S)px[p].w * px[p].z;
+        const R we = px[p].w, wo = px[p].w * px[p].z;
         // [2 d1 + d2]: combine the per-pixel direction's parities, then the other's
-        S g[2][4];                                       // [sign of direction 2][parity 1][re, im]
+        R g[2][4];                                       // [sign of direction 2][parity 1][re, im]
 #pragma unroll
         for (int d1 = 0; d1 < 2; ++d1)
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int k = 4 * d1 + c;
-                const S e = we * ((S)acc[p][k] + low[p][k]), o = wo * ((S)acc[p][k + 2] + low[p][k + 2]);
+                const R e = we * acc[p][k], o = wo * acc[p][k + 2];
                 g[0][2 * d1 + c] = e + o;
                 g[1][2 * d1 + c] = e - o;
             }
@@ -836,16 +836,16 @@ __global__ void __launch_bounds__(32 * kWarps) fg_pixels_out_kernel(FieldGrid f,
                 const int mu = kUniform ? m2 : m1, mv = kUniform ? m1 : m2;
                 const int iu = mu ? fg_minus(u[p], f.det_nx) : fg_plus(u[p], f.det_nx);
                 const int iv = mv ? fg_minus(v[p], f.det_ny) : fg_plus(v[p], f.det_ny);
-                const S re = m1 ? g[m2][0] - g[m2][2] : g[m2][0] + g[m2][2];
-                const S im = m1 ? g[m2][1] - g[m2][3] : g[m2][1] + g[m2][3];
-                const S ox = off ? (S)0 : (S)str_re * re - (S)str_im * im;
-                const S oy = off ? (S)0 : (S)str_re * im + (S)str_im * re;
+                const R re = m1 ? g[m2][0] - g[m2][2] : g[m2][0] + g[m2][2];
+                const R im = m1 ? g[m2][1] - g[m2][3] : g[m2][1] + g[m2][3];
+                const R ox = off ? (R)0 : (R)str_re * re - (R)str_im * im;
+                const R oy = off ? (R)0 : (R)str_re * im + (R)str_im * re;
                 const size_t at = (size_t)iv * f.det_nx + iu;
                 C o;
-                o.x = (R)ox;
-                o.y = (R)oy;
+                o.x = (IO)ox;
+                o.y = (IO)oy;
                 A[at] = o;
-                I[at] = (R)(ox * ox + oy * oy);
+                I[at] = (IO)(ox * ox + oy * oy);
             }
     }
 }
@@ -854,13 +854,13 @@ __global__ void __launch_bounds__(32 * kWarps) fg_pixels_out_kernel(FieldGrid f,
 // Forward launches
 // ---------------------------------------------------------------------------
 
-template <typename R, int kRpt>
+template <typename R, typename IO, int kRpt>
 static cudaError_t fg_run_y(const FieldGrid &f, const void *s, const int *bounds, cudaStream_t st) {
     const size_t smem = sizeof(FgTile<R, kRpt>);
-    cudaError_t e = fg_smem(fg_y_kernel<R, kRpt>, smem);
+    cudaError_t e = fg_smem(fg_y_kernel<R, IO, kRpt>, smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((f.nx + 31) / 32, f.nz, (f.Hs + 8 * kRpt - 1) / (8 * kRpt));
-    return launch_pdl(fg_y_kernel<R, kRpt>, grid, dim3(kFgThreads), smem, st, f, (const typename Fg<R>::C *)s, bounds);
+    return launch_pdl(fg_y_kernel<R, IO, kRpt>, grid, dim3(kFgThreads), smem, st, f, (const typename Fg<IO>::C *)s, bounds);
 }
 
 template <typename R, int kRpt, bool kPm>
@@ -872,22 +872,22 @@ static cudaError_t fg_run_xz(const FieldGrid &f, int Nxp, const int *bounds, con
     return launch_pdl(fg_xz_kernel<R, kRpt, kPm>, grid, dim3(kFgThreads), smem, st, f, Nxp, bounds, chunk_y);
 }
 
-template <typename R, int kPts, bool kUniform, int kWarps, bool kDot2 = false, bool kSplit = false>
+template <typename R, typename IO, int kPts, bool kUniform, int kWarps, bool kSplit = false>
 static cudaError_t fg_run_pixels(const FieldGrid &f, double str_re, double str_im, void *A, void *I, cudaStream_t st) {
     using V4 = typename Fg<R>::V4;
     const size_t smem = (size_t)f.H2 * 8 * (kUniform ? 4 : 32) * sizeof(R) + (size_t)f.H2 * sizeof(V4);
     // the largest size any plan uses, so concurrent launches of other handles stay valid
-    const size_t most = (size_t)fg_max_half(sizeof(R) == 8) * (8 * (kUniform ? 4 : 32) * sizeof(R) + sizeof(V4));
-    const auto k = fg_pixels_out_kernel<R, kPts, kUniform, kWarps, kDot2, kSplit>;
+    const size_t most = (size_t)fg_max_half((int)sizeof(R)) * (8 * (kUniform ? 4 : 32) * sizeof(R) + sizeof(V4));
+    const auto k = fg_pixels_out_kernel<R, IO, kPts, kUniform, kWarps, kSplit>;
     cudaError_t e = smem <= (size_t)40 << 10 ? cudaSuccess : fg_smem(k, most);
     if (e != cudaSuccess) return e;
     const dim3 grid = kUniform ? dim3((f.U + 32 * kPts - 1) / (32 * kPts), (f.V + 3) / 4)
                  : kSplit ? dim3((f.U + 31) / 32, f.V)
                           : dim3((f.U + 31) / 32, (f.V + kWarps * kPts - 1) / (kWarps * kPts));
-    return launch_pdl(k, grid, dim3(32 * kWarps), smem, st, f, str_re, str_im, (typename Fg<R>::C *)A, (R *)I);
+    return launch_pdl(k, grid, dim3(32 * kWarps), smem, st, f, str_re, str_im, (typename Fg<IO>::C *)A, (IO *)I);
 }
 
-template <typename R>
+template <typename R, typename IO>
 static cudaError_t fg_finish(const FieldGrid &f, double str_re, double str_im, void *A, void *I, int sm_count,
                              cudaStream_t st) {
     cudaError_t e = launch_pdl(fg_columns_kernel<R>, dim3((f.n1 + 31) / 32, f.H2), dim3(256),
@@ -896,29 +896,25 @@ static cudaError_t fg_finish(const FieldGrid &f, double str_re, double str_im, v
     // more pixels per thread share the loads of B on large detectors; on small
     // ones fewer rows per block fill the SMs
     const long long blocks = (long long)f.U * f.V / 128;
-    if (sizeof(R) == 4 && f.dot2)
-        return f.uniform                  ? fg_run_pixels<R, 1, true, 4, true>(f, str_re, str_im, A, I, st)
-               : blocks >= 2ll * sm_count ? fg_run_pixels<R, 1, false, 8, true>(f, str_re, str_im, A, I, st)
-                                          : fg_run_pixels<R, 1, false, 4, true>(f, str_re, str_im, A, I, st);
     if (f.uniform)
-        return blocks >= 8ll * sm_count   ? fg_run_pixels<R, 4, true, 4>(f, str_re, str_im, A, I, st)
-               : blocks >= 2ll * sm_count ? fg_run_pixels<R, 2, true, 4>(f, str_re, str_im, A, I, st)
-                                          : fg_run_pixels<R, 1, true, 4>(f, str_re, str_im, A, I, st);
-    return blocks >= 8ll * sm_count   ? fg_run_pixels<R, 4, false, 4>(f, str_re, str_im, A, I, st)
-           : blocks >= 2ll * sm_count ? fg_run_pixels<R, 1, false, 8>(f, str_re, str_im, A, I, st)
-           : 2 * blocks >= sm_count   ? fg_run_pixels<R, 1, false, 4>(f, str_re, str_im, A, I, st)
-           : sizeof(R) == 8           ? fg_run_pixels<R, 1, false, 4, false, true>(f, str_re, str_im, A, I, st)
-                                      : fg_run_pixels<R, 1, false, 1>(f, str_re, str_im, A, I, st);
+        return blocks >= 8ll * sm_count   ? fg_run_pixels<R, IO, 4, true, 4>(f, str_re, str_im, A, I, st)
+               : blocks >= 2ll * sm_count ? fg_run_pixels<R, IO, 2, true, 4>(f, str_re, str_im, A, I, st)
+                                          : fg_run_pixels<R, IO, 1, true, 4>(f, str_re, str_im, A, I, st);
+    return blocks >= 8ll * sm_count   ? fg_run_pixels<R, IO, 4, false, 4>(f, str_re, str_im, A, I, st)
+           : blocks >= 2ll * sm_count ? fg_run_pixels<R, IO, 1, false, 8>(f, str_re, str_im, A, I, st)
+           : 2 * blocks >= sm_count   ? fg_run_pixels<R, IO, 1, false, 4>(f, str_re, str_im, A, I, st)
+           : sizeof(R) == 8           ? fg_run_pixels<R, IO, 1, false, 4, true>(f, str_re, str_im, A, I, st)
+                                      : fg_run_pixels<R, IO, 1, false, 1>(f, str_re, str_im, A, I, st);
 }
 
-template <typename R>
+template <typename R, typename IO>
 static cudaError_t fg_sum_y(const FieldGrid &f, const void *s, const int *bounds, int sm_count, cudaStream_t st) {
     switch (fg_rows_per_thread(f.Hs, (long long)((f.nx + 31) / 32) * f.nz, sizeof(R) == 8, sm_count)) {
-        case 1: return fg_run_y<R, 1>(f, s, bounds, st);
-        case 2: return fg_run_y<R, 2>(f, s, bounds, st);
-        case 3: return fg_run_y<R, 3>(f, s, bounds, st);
-        case 5: return fg_run_y<R, 5>(f, s, bounds, st);
-        default: return fg_run_y<R, 6>(f, s, bounds, st);
+        case 1: return fg_run_y<R, IO, 1>(f, s, bounds, st);
+        case 2: return fg_run_y<R, IO, 2>(f, s, bounds, st);
+        case 3: return fg_run_y<R, IO, 3>(f, s, bounds, st);
+        case 5: return fg_run_y<R, IO, 5>(f, s, bounds, st);
+        default: return fg_run_y<R, IO, 6>(f, s, bounds, st);
     }
 }
 
@@ -934,24 +930,25 @@ static cudaError_t fg_sum_xz(const FieldGrid &f, int Nxp, const int *bounds, con
     }
 }
 
-template <typename R>
+template <typename R, typename IO>
 static cudaError_t fg_forward(const FieldGrid &f, const void *s, const int *bounds, double str_re, double str_im,
                               void *A, void *I, int sm_count, cudaStream_t st) {
-    cudaError_t e = fg_sum_y<R>(f, s, bounds, sm_count, st);
+    cudaError_t e = fg_sum_y<R, IO>(f, s, bounds, sm_count, st);
     if (e == cudaSuccess) e = fg_sum_xz<R, false>(f, f.nx, bounds, nullptr, sm_count, st);
-    return e == cudaSuccess ? fg_finish<R>(f, str_re, str_im, A, I, sm_count, st) : e;
+    return e == cudaSuccess ? fg_finish<R, IO>(f, str_re, str_im, A, I, sm_count, st) : e;
 }
 
 cudaError_t launch_field_grid(const FieldGrid &f, const void *s, const int *bounds, double str_re, double str_im,
                               void *A, void *I, int sm_count, cudaStream_t st) {
-    return f.elem == 8 ? fg_forward<double>(f, s, bounds, str_re, str_im, A, I, sm_count, st)
-                       : fg_forward<float>(f, s, bounds, str_re, str_im, A, I, sm_count, st);
+    return f.io == 8     ? fg_forward<double, double>(f, s, bounds, str_re, str_im, A, I, sm_count, st)
+           : f.elem == 8 ? fg_forward<double, float>(f, s, bounds, str_re, str_im, A, I, sm_count, st)
+                         : fg_forward<float, float>(f, s, bounds, str_re, str_im, A, I, sm_count, st);
 }
 
 cudaError_t launch_field_grid_tc(const FieldGrid &f, int Nxp, const int *bounds, const int *chunk_y, double str_re,
                                  double str_im, float2 *A, float *I, int sm_count, cudaStream_t st) {
     const cudaError_t e = fg_sum_xz<float, true>(f, Nxp, bounds, chunk_y, sm_count, st);
-    return e == cudaSuccess ? fg_finish<float>(f, str_re, str_im, A, I, sm_count, st) : e;
+    return e == cudaSuccess ? fg_finish<float, float>(f, str_re, str_im, A, I, sm_count, st) : e;
 }
 
 }  // namespace scm

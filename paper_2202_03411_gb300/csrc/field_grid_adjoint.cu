@@ -40,8 +40,14 @@ static int fa_chunks(const FieldGrid &f) {
     return c < 1 ? 1 : c > kFaMaxChunks ? kFaMaxChunks : c;
 }
 
-size_t field_grid_adjoint_layout(const FieldGrid &f, FieldGridAdjoint *a, unsigned char *base) {
+size_t field_grid_adjoint_layout(FieldGrid *grid, const FieldGrid *fwd, FieldGridAdjoint *a, unsigned char *base) {
+    FieldGrid &f = *grid;
+    a->own = !(fwd && fwd->elem == f.elem);
     size_t at = 0;
+    if (a->own)
+        at = field_grid_layout(grid, false, 0, base);
+    else
+        f = *fwd;
     auto take = [&](size_t bytes) {
         unsigned char *p = base ? base + at : nullptr;
         at += (bytes + 255) / 256 * 256;
@@ -51,7 +57,7 @@ size_t field_grid_adjoint_layout(const FieldGrid &f, FieldGridAdjoint *a, unsign
     a->chunks = fa_chunks(f);
     a->B = take((size_t)a->chunks * f.H2 * 8 * f.n1 * e);
     a->G = take((size_t)f.Hs * f.Ht * 8 * e);
-    a->T = take(2 * (size_t)f.Hs * f.nz * f.nx * 2 * e);
+    a->T = a->own ? take(2 * (size_t)f.Hs * f.nz * f.nx * 2 * e) : f.H;      // (the forward pass is done with H)
     return at;
 }
 

@@ -199,25 +199,25 @@ struct SliceOut {
 // device buffers in one allocation.  Passed to its kernels by value.
 struct FieldGrid {
     int uniform = 0;                // uniform-q detector (rows fix s) instead of the flat one (columns fix t)
-    int elem = 4;                   // bytes of a real number
+    int elem = 4;                   // bytes of a real number in the sums and tables,
+    int io = 4;                     // and in the slices, the field and the pattern
     int nx = 0, ny = 0, nz = 0, det_nx = 0, det_ny = 0;
     int Hs = 0, Ht = 0;             // half the points in s and t
     int H1 = 0, H2 = 0, n1 = 0;     // per-column (per-row) direction: its half points and half pixels; per-pixel direction
     int Kx = 0, Ky = 0, U = 0, V = 0;   // half sides of the grid and the detector, rounded up
     int jc = 0;                     // slice chunks of the x/z sum
-    int dot2 = 0;                   // FP32 interpolation sums with their rounding errors collected
     double sm = 0, tm = 0;          // largest |s|, |t|
     double k0 = 0, voxel = 0, top = 0;  // top: tan or sin of theta_max
     void *ty = nullptr, *tx = nullptr, *tz = nullptr;   // phases of the sums
     void *node2 = nullptr, *w1 = nullptr, *pix = nullptr;   // interpolation: points, weights, pixels
     double *qrow = nullptr, *point_s = nullptr, *point_t = nullptr;
     void *H = nullptr, *Q = nullptr, *B = nullptr;      // y-sums, samples, per-column interpolants
-    size_t bytes = 0;
 };
 
 // Buffers of the adjoint through the grid (field_grid_adjoint.cu), one allocation.
 struct FieldGridAdjoint {
     int chunks = 0;                 // of the per-pixel direction
+    bool own = false;               // the grid's tables are its own (the forward pass has none of this type)
     void *B = nullptr, *G = nullptr, *T = nullptr;      // pixels gathered along it; onto the grid; x/z sums
 };
 
@@ -299,6 +299,7 @@ struct scatman_handle {
     scm::FieldGrid fg;
     unsigned char *d_fg = nullptr;  // its buffers
     bool adj_on_grid = false;       // the adjoint goes through the grid
+    scm::FieldGrid fg_adj;
     scm::FieldGridAdjoint fga;
     unsigned char *d_fga = nullptr; // its buffers (from the first backward on)
     int splits = 1;
@@ -386,9 +387,9 @@ cudaError_t launch_rows_y_tc(const TcMaps &maps, const double *qrow, int rows, i
                              int sm_count, cudaStream_t st);
 // The field through its sample grid (field_grid.cu).  plan: whether the
 // detector and box allow it, and its sizes; layout: buffer offsets from base.
-bool plan_field_grid(const scatman_config &c, bool fp64, FieldGrid *f);
+bool plan_field_grid(const scatman_config &c, int elem, FieldGrid *f);
 bool use_field_grid(const scatman_config &c, FieldGrid *f);
-size_t field_grid_layout(FieldGrid *f, bool tensor_core, int Nxp, unsigned char *base);
+size_t field_grid_layout(FieldGrid *f, bool forward, int Nxp, unsigned char *base);
 cudaError_t launch_field_grid_tables(const FieldGrid &f, cudaStream_t st);
 // Forward from the slices (FP32 or FP64), or from the tensor-core y-sums in f.H.
 cudaError_t launch_field_grid(const FieldGrid &f, const void *s, const int *bounds, double str_re, double str_im,
@@ -397,8 +398,10 @@ cudaError_t launch_field_grid_tc(const FieldGrid &f, int Nxp, const int *bounds,
                                  double str_im, float2 *A, float *I, int sm_count, cudaStream_t st);
 // Whether a handle of this configuration runs its adjoint through the grid.
 bool use_field_grid_adjoint(const scatman_config &c, FieldGrid *f);
-// The adjoint field (field_grid_adjoint.cu); layout: buffer offsets from base, returns the bytes.
-size_t field_grid_adjoint_layout(const FieldGrid &f, FieldGridAdjoint *a, unsigned char *base);
+// The adjoint field (field_grid_adjoint.cu).  layout: buffer offsets from base of the
+// planned grid f, with the tables and sums of the forward pass's grid fwd (null: it has
+// none) where that holds the same type; returns the bytes.
+size_t field_grid_adjoint_layout(FieldGrid *f, const FieldGrid *fwd, FieldGridAdjoint *a, unsigned char *base);
 cudaError_t launch_field_grid_adjoint(const FieldGrid &f, const FieldGridAdjoint &ad, const void *A, const void *w,
                                       void *S, cudaStream_t st);
 // Real flops one contraction launch issues for the recorded slice geometry

@@ -353,12 +353,13 @@ long long scatman_footprint_bytes(const scatman_config *c) {
     } else {
         b += round_2mib(256LL * 128 * 4 * 8);   // last wave's partial fields (< 256 SMs, <= 4 parts)
     }
-    FieldGrid fg;
+    FieldGrid fg, fg_adj;
     FieldGridAdjoint fga;
-    const bool adj_on_grid = use_field_grid_adjoint(*c, &fg);
-    if (adj_on_grid) b += round_2mib((long long)field_grid_adjoint_layout(fg, &fga, nullptr));
-    if (use_field_grid(*c, &fg) || adj_on_grid) // the field's sample grid: phases, sums, weights
-        b += round_2mib((long long)field_grid_layout(&fg, tc, (c->nx + 15) / 16 * 16, nullptr));
+    const bool on_grid = use_field_grid(*c, &fg);
+    if (on_grid)                                // the field's sample grid: phases, sums, weights
+        b += round_2mib((long long)field_grid_layout(&fg, true, tc ? (c->nx + 15) / 16 * 16 : 0, nullptr));
+    if (use_field_grid_adjoint(*c, &fg_adj))
+        b += round_2mib((long long)field_grid_adjoint_layout(&fg_adj, on_grid ? &fg : nullptr, &fga, nullptr));
     b += round_2mib(nvox * cx);                 // adjoint field (backward)
     if (tc) {
         // adjoint partial fields (<= 8), scale, pixel table, y-phase operand tiles

@@ -121,3 +121,28 @@ def test_empty_and_repeated_shapes(prec):
     h.close()
     assert np.array_equal(out[0], out[2]) and out[0].max() > 0
     assert np.all(out[3] == 0.0)
+
+
+@pytest.mark.parametrize("g", [
+    Geometry(48, 48, 48, 1.0, 10.0, 45.0, 64, 64),
+    Geometry(33, 41, 26, 1.0, 7.0, 55.0, 71, 58),
+    Geometry(24, 27, 30, 1.0, 5.0, 40.0, 70, 65, DETECTOR_UNIFORM_Q),
+])
+def test_fp32_fit_sums_are_exact_to_the_stored_pattern(g):
+    """A fit's loss is the difference of two nearly equal patterns, so an FP32 fit's
+    sums over its (FP32) slices run in FP64.  I is rounded to FP32 once: 2^-24 = 6e-8 of it,
+    and the plan leaves up to 1e-8 of a field; FP32 sums leave 2e-7."""
+    import torch
+    import oracle
+    import paper_2202_03411_gb300 as sm
+    s = Shape(ELLIPSOID, a=0.36 * g.nx, b=0.28 * g.ny, c=0.3 * g.nz, delta=0.012, beta=0.0012, latitude=30,
+              longitude=70, rotation=-20)
+    h = sm.scatman_create(g, "fp32", soft=True, soft_width=0.5)
+    I = torch.empty(g.n_pix, device="cuda")
+    sm.scatman_voxelise(h, s)
+    sm.scatman_forward(h, I)
+    rho = np.asarray(sm.scatman_get_slices(h, (g.nz, g.nx, g.ny)), dtype=np.complex128)
+    q = sm.scatman_get_q(h)
+    h.close()
+    ref = np.abs(oracle.msft(rho * ((1 - s.delta + 1j * s.beta) ** 2 - 1), q, g.voxel)) ** 2
+    assert rel_l2(I.cpu().double().numpy(), ref) < 8e-8
