@@ -73,11 +73,12 @@ static int plan_points(double k0, double top, double along, double across, doubl
 // points of 32 columns in shared memory: 131 KB in FP32, 200 KB in FP64).
 static int fg_max_half(int elem) { return elem == 8 ? 96 : 128; }
 constexpr int kFgMaxSide = 512;          // grid side in x and y
+constexpr int kFgMaxRows = 65535;        // half the detector's rows: they are fg_pixels_kernel's grid.y
 
 // elem: bytes of a real number in the sums.
 bool plan_field_grid(const scatman_config &c, int elem, FieldGrid *f) {
     *f = FieldGrid();
-    if (c.q_list || c.nx > kFgMaxSide || c.ny > kFgMaxSide) return false;
+    if (c.q_list || c.nx > kFgMaxSide || c.ny > kFgMaxSide || c.det_ny > 2 * kFgMaxRows) return false;
     const bool uniform = c.detector == SCATMAN_DETECTOR_UNIFORM_Q;
     const double k0 = 2.0 * kPi / c.wavelength;
     const double Lx = 0.5 * (c.nx - 1) * c.voxel, Ly = 0.5 * (c.ny - 1) * c.voxel, Lz = 0.5 * (c.nz - 1) * c.voxel;

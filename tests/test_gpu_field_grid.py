@@ -146,3 +146,37 @@ def test_fp32_fit_sums_are_exact_to_the_stored_pattern(g):
     h.close()
     ref = np.abs(oracle.msft(rho * ((1 - s.delta + 1j * s.beta) ** 2 - 1), q, g.voxel)) ** 2
     assert rel_l2(I.cpu().double().numpy(), ref) < 8e-8
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("tc_bf16_split", 1e-3)])
+@pytest.mark.parametrize("rows", [131070, 140001])
+def test_strip_detectors(rows, prec, tol):
+    """A line of pixels up to the last row that the grid takes, and past it (direct sums)."""
+    from gpu_helpers import oracle_field
+    g = Geometry(17, 18, 16, 1.0, 7.0, 50.0, 1, rows)
+    s = Shape(ELLIPSOID, a=6.0, b=5.0, c=6.5, delta=0.01, beta=0.001, latitude=20, longitude=50)
+    at = np.concatenate([np.arange(40), rows // 2 + np.arange(-20, 20), rows - 1 - np.arange(40)])
+    I, _ = run_gpu(g, s, prec)
+    ref, _ = oracle_field(g, s, sample=at)
+    assert rel_l2(I[at], ref) < tol
+
+
+@pytest.mark.parametrize("rows", [131070, 140001])
+def test_strip_detector_gradients(rows):
+    """The same in the adjoint of an FP32 fit, against an FP64 fit of the weighted pixels."""
+    import torch
+    import oracle
+    import paper_2202_03411_gb300 as sm
+    g = Geometry(17, 18, 16, 1.0, 7.0, 50.0, 1, rows)
+    s = Shape(ELLIPSOID, a=6.0, b=5.0, c=6.5, delta=0.01, beta=0.001, latitude=20, longitude=50)
+    at = np.concatenate([np.arange(40), rows // 2 + np.arange(-20, 20), rows - 1 - np.arange(40)])
+    w = torch.zeros(rows, device="cuda")
+    w[torch.as_tensor(at, device="cuda")] = 1.0
+    grads = []
+    for prec, q, up in (("fp32", None, w), ("fp64", oracle.detector_q(g)[at], torch.ones(len(at), device="cuda").double())):
+        h = sm.scatman_create(g, prec, soft=True, soft_width=0.5, q_list=q)
+        sm.scatman_voxelise(h, s)
+        sm.scatman_forward(h, torch.empty_like(up))
+        grads.append(sm.scatman_backward(h, up))
+        h.close()
+    assert np.linalg.norm(grads[0] - grads[1]) / np.linalg.norm(grads[1]) < 2e-5
