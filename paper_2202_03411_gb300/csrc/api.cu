@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstring>
 #include <atomic>
+#include <functional>
 #include <new>
 
 #include "internal.cuh"
@@ -280,11 +281,19 @@ static int fill_detector_q(scatman_handle *h) {
                       "detector q");
 }
 
-// The same for a handle whose forward pass does without it (the sample grid).
-static int need_q(scatman_handle *h) {
-    if (h->d_q) return SCATMAN_OK;
-    const int rc = alloc_dev(h, (void **)&h->d_q, (size_t)h->n_pix * 3 * sizeof(double), "q buffer");
-    return rc ? rc : fill_detector_q(h);
+// Runs `use` with the pixels' q in d_q, which a handle whose sums run through the
+// sample grid does not keep.
+static int with_q(scatman_handle *h, const std::function<int()> &use) {
+    if (h->d_q) return use();
+    const size_t bytes = (size_t)h->n_pix * 3 * sizeof(double);
+    int rc = alloc_dev(h, (void **)&h->d_q, bytes, "q buffer");
+    if (rc) return rc;
+    if (!(rc = fill_detector_q(h))) rc = use();
+    const int e = check_cuda(h, cudaStreamSynchronize(h->stream), "stream synchronize");
+    cudaFree(h->d_q);
+    h->d_q = nullptr;
+    h->device_bytes -= (long long)bytes;
+    return rc ? rc : e;
 }
 
 // The sample grid's buffers and tables.
@@ -1102,13 +1111,12 @@ int scatman_contraction_flops(scatman_handle *h, double *issued, double *dense) 
 
 int scatman_get_q(scatman_handle *h, double *q_host) {
     if (!h || !q_host) return SCATMAN_ERR_ARG;
-    int rc = need_q(h);
-    if (rc) return rc;
-    rc = check_cuda(h, cudaMemcpyAsync(q_host, h->d_q, (size_t)h->n_pix * 3 * sizeof(double),
-                                           cudaMemcpyDeviceToHost, h->stream),
-                        "q download");
-    if (rc) return rc;
-    return scatman_sync(h);
+    const int rc = with_q(h, [&] {
+        return check_cuda(h, cudaMemcpyAsync(q_host, h->d_q, (size_t)h->n_pix * 3 * sizeof(double),
+                                             cudaMemcpyDeviceToHost, h->stream),
+                          "q download");
+    });
+    return rc ? rc : scatman_sync(h);
 }
 
 int scatman_photon_counts(scatman_handle *h, double photon_density, unsigned long long seed, const void *I_dev,
@@ -1249,7 +1257,6 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
         if ((rc = alloc_dev(h, (void **)&h->d_part, need * sizeof(double), "gradient partials"))) return rc;
         h->part_count = need;
     }
-    if (!h->adj_on_grid && (rc = need_q(h))) return rc;      // sums over the pixels
     if (h->adj_on_grid) {
         if ((rc = need_adjoint_grid(h))) return rc;
         rc = check_cuda(h, launch_field_grid_adjoint(h->fg_adj, h->fga, h->d_A, dLdI_dev, h->d_S, h->stream),
@@ -1257,7 +1264,7 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
         if (rc) return rc;
     } else if (h->tensor_core && adjoint_tc_supported(c.nx, c.ny)) {
         // adjoint contraction on the tensor cores (per slice, or per Jacobi-Anger order)
-        if (h->adj_orders < 0 && (rc = plan_adjoint(h))) return rc;
+        if (h->adj_orders < 0 && (rc = with_q(h, [&] { return plan_adjoint(h); }))) return rc;
         const int N = h->adj_orders;
         const int nz_eff = N > 0 ? N : c.nz;
         int splits = adjoint_tc_splits(h->n_pix, nz_eff, h->sm_count, N > 0);
@@ -1289,9 +1296,11 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
                                       "adjoint slices from orders")))
             return rc;
     } else {
-        rc = check_cuda(h, launch_adjoint_field(f64, h->d_A, dLdI_dev, h->d_q, h->n_pix, c.nx, c.ny, c.nz, c.voxel,
-                                                h->d_S, h->stream),
-                        "adjoint field");
+        rc = with_q(h, [&] {
+            return check_cuda(h, launch_adjoint_field(f64, h->d_A, dLdI_dev, h->d_q, h->n_pix, c.nx, c.ny, c.nz,
+                                                      c.voxel, h->d_S, h->stream),
+                              "adjoint field");
+        });
         if (rc) return rc;
     }
     rc = check_cuda(h, launch_grad_voxels(f64, h->sp, gp, h->d_S, h->d_part, nvb, h->stream), "voxel gradient");

@@ -335,31 +335,35 @@ long long scatman_footprint_bytes(const scatman_config *c) {
         s_bytes = nvox * cx;
     }
     long long b = 0;
-    b += round_2mib(npix * 24);                 // q
     b += round_2mib(4LL * (long long)scm::slice_geom_ints(c->nz));   // slice geometry and the unit list
     b += round_2mib(nvox * 4);                  // occupancy
     b += round_2mib(s_bytes);                   // slices
     b += round_2mib(npix * cx);                 // field cache
     b += round_2mib(npix * (f64 ? 8 : 4));      // intensity scratch
+    long long direct = round_2mib(npix * 24);   // of the direct sums: q
     if (uniform && c->precision >= SCATMAN_TC_F16_SPLIT) {
-        b += round_2mib((long long)scm::uq_tc_h_bytes(c->nx, c->nz, c->det_ny));   // y-contracted 16-bit planes
-        b += round_2mib(npix * 8);                                                 // q_z table
-        b += round_2mib(24LL * c->det_ny);                                         // detector row q
+        direct += round_2mib((long long)scm::uq_tc_h_bytes(c->nx, c->nz, c->det_ny));   // y-contracted 16-bit planes
+        direct += round_2mib(npix * 8);                                                 // q_z table
+        direct += round_2mib(24LL * c->det_ny);                                         // detector row q
     } else if (uniform) {
-        b += round_2mib((long long)c->det_ny * c->nx * c->nz * cx);   // y-contracted slices
-        b += round_2mib(npix * 8);                                    // q_z table
+        direct += round_2mib((long long)c->det_ny * c->nx * c->nz * cx);   // y-contracted slices
+        direct += round_2mib(npix * 8);                                    // q_z table
     } else if (!tc) {
-        b += round_2mib(64 * npix * cx);        // partial fields (upper bound on splits)
+        direct += round_2mib(64 * npix * cx);        // partial fields (upper bound on splits)
     } else {
-        b += round_2mib(256LL * 128 * 4 * 8);   // last wave's partial fields (< 256 SMs, <= 4 parts)
+        direct += round_2mib(256LL * 128 * 4 * 8);   // last wave's partial fields (< 256 SMs, <= 4 parts)
     }
+    // the field's sample grid (phases, sums, weights) and its adjoint
     FieldGrid fg, fg_adj;
     FieldGridAdjoint fga;
     const bool on_grid = use_field_grid(*c, &fg);
-    if (on_grid)                                // the field's sample grid: phases, sums, weights
-        b += round_2mib((long long)field_grid_layout(&fg, true, tc ? (c->nx + 15) / 16 * 16 : 0, nullptr));
+    long long grid = 0;
+    if (on_grid)
+        grid += round_2mib((long long)field_grid_layout(&fg, true, tc ? (c->nx + 15) / 16 * 16 : 0, nullptr));
     if (use_field_grid_adjoint(*c, &fg_adj))
-        b += round_2mib((long long)field_grid_adjoint_layout(&fg_adj, on_grid ? &fg : nullptr, &fga, nullptr));
+        grid += round_2mib((long long)field_grid_adjoint_layout(&fg_adj, on_grid ? &fg : nullptr, &fga, nullptr));
+    // (a pass through the grid holds neither q nor the direct sums' scratch)
+    b += on_grid ? std::max(direct, grid) : direct + grid;
     b += round_2mib(nvox * cx);                 // adjoint field (backward)
     if (tc) {
         // adjoint partial fields (<= 8), scale, pixel table, y-phase operand tiles

@@ -160,3 +160,19 @@ def test_binding_checks_output_buffers_before_any_kernel():
                 _FakeTensor(n=99)):
         with pytest.raises(ValueError):
             _device_ptr(bad, ["float32"], 100, "I")
+
+
+def test_footprint_of_the_grid_of_directions(lib):
+    """A handle whose sums run through the grid of directions holds none of the direct
+    sums' scratch, which a list of as many q needs: no more is reserved for it."""
+    import numpy as np
+    from paper_2202_03411_gb300 import _lib
+    from paper_2202_03411_gb300.api import make_config
+    for prec in ("fp64", "fp32"):
+        for n, det in ((48, 128), (96, 256), (128, 512)):
+            g = Geometry(n, n, n, 1.0, 10.0, 45.0, det, det)
+            sizes = []
+            for q in (None, np.zeros((det * det, 3))):
+                cfg, keep = make_config(g, prec, soft=True, soft_width=0.5, q_list=q)
+                sizes.append(_lib.load().scatman_footprint_bytes(ctypes.byref(cfg)))
+            assert 0 < sizes[0] <= sizes[1], (prec, n, det, sizes)
