@@ -1179,7 +1179,8 @@ static int adjoint_orders_needed(double wmax, double tol) {
 // Chooses the tensor-core adjoint's form for the handle (once): with the q_z of
 // the handle's pixels in [q_c - D, q_c + D] and |z_j| <= z_max, order mode takes
 // N orders for w = D z_max; it is used when N < nz.  Builds the pixel table in
-// the chosen form and, in order mode, the coefficients a[j][n].
+// the chosen form and, in order mode, the coefficients a[j][n].  The form is set
+// last: after a failure (no memory) the next backward plans again.
 static int plan_adjoint(scatman_handle *h) {
     const scatman_config &c = h->cfg;
     std::vector<double> qz((size_t)h->n_pix);
@@ -1197,14 +1198,17 @@ static int plan_adjoint(scatman_handle *h) {
     const double zmax = 0.5 * (c.nz - 1) * c.voxel;
     const int N = D > 0.0 ? adjoint_orders_needed(D * zmax, 1e-7) : 1;
     const bool orders = N < c.nz && N <= 64;
-    h->adj_orders = orders ? N : 0;
-    if ((rc = alloc_dev(h, (void **)&h->d_adj_tab, (size_t)h->n_pix * 3 * sizeof(float4), "adjoint pixel table")))
+    if (!h->d_adj_tab &&
+        (rc = alloc_dev(h, (void **)&h->d_adj_tab, (size_t)h->n_pix * 3 * sizeof(float4), "adjoint pixel table")))
         return rc;
     if ((rc = check_cuda(h, launch_adj_pixel_table(h->d_q, h->n_pix, c.voxel, orders ? 1 : 0, qc,
                                                    orders && D > 0.0 ? 1.0 / D : 0.0, h->d_adj_tab, h->stream),
                          "adjoint pixel table")))
         return rc;
-    if (!orders) return SCATMAN_OK;
+    if (!orders) {
+        h->adj_orders = 0;
+        return SCATMAN_OK;
+    }
     // a[j][n] = e^{+i q_c z_j} eps_n i^n J_n(D z_j)
     std::vector<float2> coef((size_t)c.nz * N);
     std::vector<double> J((size_t)N);
@@ -1225,12 +1229,17 @@ static int plan_adjoint(scatman_handle *h) {
             coef[(size_t)jz * N + n] = make_float2((float)(pr * ar - pi * ai), (float)(pr * ai + pi * ar));
         }
     }
-    if ((rc = alloc_dev(h, (void **)&h->d_adj_coef, coef.size() * sizeof(float2), "adjoint order coefficients")))
+    if (!h->d_adj_coef &&
+        (rc = alloc_dev(h, (void **)&h->d_adj_coef, coef.size() * sizeof(float2), "adjoint order coefficients")))
         return rc;
     if ((rc = check_cuda(h, cudaMemcpy(h->d_adj_coef, coef.data(), coef.size() * sizeof(float2), cudaMemcpyHostToDevice),
                          "adjoint order coefficients")))
         return rc;
-    return alloc_dev(h, (void **)&h->d_adj_ord, (size_t)N * c.nx * c.ny * sizeof(float2), "adjoint order fields");
+    if (!h->d_adj_ord &&
+        (rc = alloc_dev(h, (void **)&h->d_adj_ord, (size_t)N * c.nx * c.ny * sizeof(float2), "adjoint order fields")))
+        return rc;
+    h->adj_orders = N;
+    return SCATMAN_OK;
 }
 
 int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams) {
@@ -1254,6 +1263,7 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
     if (h->part_count < need) {
         cudaFree(h->d_part);
         h->d_part = nullptr;
+        h->part_count = 0;
         if ((rc = alloc_dev(h, (void **)&h->d_part, need * sizeof(double), "gradient partials"))) return rc;
         h->part_count = need;
     }
@@ -1273,6 +1283,7 @@ int scatman_backward(scatman_handle *h, const void *dLdI_dev, double *dLdparams)
         if (h->adj_part_count < cnt) {
             cudaFree(h->d_adj_part);
             h->d_adj_part = nullptr;
+            h->adj_part_count = 0;
             if ((rc = alloc_dev(h, (void **)&h->d_adj_part, cnt * sizeof(float2), "adjoint partial fields")))
                 return rc;
             h->adj_part_count = cnt;

@@ -198,3 +198,43 @@ def test_server_cancels_a_queued_request():
             srv.cancel(tickets[-1])                 # collected already: unknown ticket
     finally:
         srv.close()
+
+
+@pytest.mark.parametrize("prec", ["tc_bf16_split", "fp32", "fp64"])
+@pytest.mark.parametrize("nz,wavelength,theta", [(8, 3.0, 50.0), (40, 8.0, 20.0)])    # per slice; over Jacobi-Anger orders
+def test_backward_after_a_failed_allocation(prec, nz, wavelength, theta):
+    """The first backward fails for want of memory at each of its allocations in turn
+    (ERR_OOM); the next one on the same handle gives the gradient of a handle that never failed."""
+    import torch
+    import paper_2202_03411_gb300 as sm
+    g = Geometry(30, 26, nz, 1.0, wavelength, theta, 40, 44)
+    s = Shape(SPHHARM, R0=2.0 if nz < 16 else 8.0, lmax=3, alm=random_alm(np.random.default_rng(2), 3), delta=0.02,
+              beta=0.003)
+    dt = torch.float64 if prec == "fp64" else torch.float32
+    w = torch.rand(g.n_pix, device="cuda", dtype=dt)
+    k, want = 0, None
+    while True:
+        h = sm.scatman_create(g, prec, soft=True, soft_width=0.5)
+        sm.scatman_voxelise(h, s)
+        sm.scatman_forward(h, torch.empty_like(w))
+        sm.scatman_sync(h)
+        if want is None:
+            want = sm.scatman_backward(h, w)
+            h.close()
+            continue
+        failed = False
+        sm.scatman_debug_fail_allocation(k)
+        try:
+            sm.scatman_backward(h, w)
+        except sm.ScatmanError as e:
+            assert e.code == -2, e                              # ERR_OOM
+            failed = True
+        finally:
+            sm.scatman_debug_fail_allocation(-1)
+        assert np.array_equal(sm.scatman_backward(h, w), want)
+        h.close()
+        if not failed:
+            break
+        k += 1
+        assert k < 64
+    assert k >= 3                                               # several allocations happened
