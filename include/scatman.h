@@ -320,12 +320,15 @@ SCATMAN_API int scatman_get_slices(scatman_handle *h, double *s_host);
 SCATMAN_API int scatman_get_q(scatman_handle *h, double *q_host);
 
 /*
- * Real floating-point operations of one contraction launch for the current
- * shape: *issued counts what the tensor-core kernel executes (it skips the
- * parts of each slice outside the occupied box, and counts both products of
- * a split-phase mode); *dense is 8 flop per (pixel, voxel) pair times the
- * number of products.  CUDA-core modes report the dense count for both.
- * Synchronises.  Errors: ERR_STATE before voxelise.
+ * Real floating-point operations of a forward pass's sums over voxels for the
+ * current shape.  *issued counts what runs: on the tensor cores the MMAs of the
+ * sums over the pixels, or of the sums over y where the field goes through the
+ * grid of directions (both products of a split-phase mode; the tensor-core
+ * uniform-q detector: its x/z sums); in FP32 and FP64 the folded sums over y and
+ * over x and z on the grid, else the direct sums.  The parts of each slice outside the
+ * occupied box are skipped and not counted (the uniform-q detector's separable
+ * sums: the dense count).  *dense is 8 flop per (pixel, voxel) pair times the number
+ * of products.  Synchronises.  Errors: ERR_STATE before voxelise.
  */
 SCATMAN_API int scatman_contraction_flops(scatman_handle *h, double *issued, double *dense);
 

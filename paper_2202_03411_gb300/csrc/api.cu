@@ -1091,12 +1091,9 @@ int scatman_contraction_flops(scatman_handle *h, double *issued, double *dense) 
     if (rc) return rc;
     if ((rc = scatman_sync(h))) return rc;
     if (h->on_grid) {
-        // the y-sum of the sample grid's rows: on the tensor cores as issued, else
-        // four flops a folded term (dense: the direct sums over the detector's pixels)
-        const FieldGrid &f = h->fg;
         *dense = 8.0 * dense_pairs * (h->split ? 2.0 : 1.0);
-        *issued = h->tensor_core ? tc_issued_flops(b.data(), c.nz, h->Nxp, h->Nyp, 2 * f.Hs, h->split)
-                                 : 8.0 * (double)f.Hs * f.Ky * c.nx * c.nz;
+        *issued = h->tensor_core ? tc_issued_flops(b.data(), c.nz, h->Nxp, h->Nyp, 2 * h->fg.Hs, h->split)
+                                 : field_grid_issued_flops(h->fg, b.data());
         return SCATMAN_OK;
     }
     if (!h->tensor_core) {

@@ -27,6 +27,7 @@
 // 512^2 to 60 degrees, BF16 split phases 74 us (1798); 96^3 on 256^2, FP32
 // 28 us (5195), FP64 164 us (73600, the same ellipsoid); 32^3 on 64^2, FP64 31 us
 // (736); uniform-q 30^3 on 512^2, FP32 29 us (125, the separable sums per pixel row).
+#include <algorithm>
 #include <cmath>
 #include <complex>
 
@@ -429,6 +430,17 @@ static int fg_rows_per_thread(int n, long long others, bool fp64, int sm_count) 
     return best;
 }
 
+// Half-coordinates of a side of n that meet [lo, hi): above the middle up to hi - 1,
+// below it down to lo; from the start of a tile of them.
+struct FgFold {
+    int beg, end;
+};
+__host__ __device__ __forceinline__ FgFold fg_fold(int lo, int hi, int n) {
+    const int up = hi - n / 2, down = (n - 1) / 2 - lo + 1, most = (n + 1) / 2;
+    const int far = up > down ? up : down, a = lo - n / 2, b = (n - 1) / 2 - (hi - 1), near = a > b ? a : b;
+    return {(near > 0 ? near : 0) & ~(kFgK - 1), far < most ? far : most};
+}
+
 // H[a][even, odd][j][x] = sum over y' of cos (q_a y') even s, -i sin (q_a y') odd s.
 // Block: 32 columns x of one slice.  Slices and columns outside the occupied
 // box are not written (and not read later), y' beyond the box is skipped.
@@ -444,9 +456,8 @@ __global__ void __launch_bounds__(kFgThreads) fg_y_kernel(FieldGrid f, const typ
     if (xlo >= xhi || x0 >= xhi || x0 + 32 <= xlo) return;
     const int grp = threadIdx.x >> 7, tt = threadIdx.x & 127, cg = tt & 15, bg = tt >> 4;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // half-coordinates that meet [ylo, yhi): above the middle up to yhi - 1, below it down to ylo
-    const int kend = min(f.Ky, max(yhi - f.ny / 2, (f.ny - 1) / 2 - ylo + 1));
-    const int kbeg = max(0, max(ylo - f.ny / 2, (f.ny - 1) / 2 - (yhi - 1))) & ~(kFgK - 1);
+    const FgFold y = fg_fold(ylo, yhi, f.ny);
+    const int kend = y.end, kbeg = y.beg;
     const R *cy = (const R *)f.ty, *sy = cy + (size_t)f.Ky * f.Hs;
     R acc[kRpt][4] = {};
     // one tile's operands on their way from memory
@@ -558,8 +569,7 @@ __global__ void __launch_bounds__(kFgThreads) fg_xz_kernel(FieldGrid f, int Nxp,
     int kend = 0;
 #pragma unroll
     for (int j = 0; j < kFgSlices; ++j)
-        if (s_lo[j] < s_hi[j]) kend = max(kend, max(s_hi[j] - f.nx / 2, (f.nx - 1) / 2 - s_lo[j] + 1));
-    kend = min(kend, f.Kx);
+        if (s_lo[j] < s_hi[j]) kend = max(kend, fg_fold(s_lo[j], s_hi[j], f.nx).end);
     const R *cx = (const R *)f.tx + (size_t)a * f.Kx * f.Ht, *sx = cx + (size_t)f.Hs * f.Kx * f.Ht;
     const C *H = (const C *)f.H;
     R acc[kRpt][4] = {};
@@ -937,6 +947,24 @@ static cudaError_t fg_forward(const FieldGrid &f, const void *s, const int *boun
     cudaError_t e = fg_sum_y<R, IO>(f, s, bounds, sm_count, st);
     if (e == cudaSuccess) e = fg_sum_xz<R, false>(f, f.nx, bounds, nullptr, sm_count, st);
     return e == cudaSuccess ? fg_finish<R, IO>(f, str_re, str_im, A, I, sm_count, st) : e;
+}
+
+double field_grid_issued_flops(const FieldGrid &f, const int *bounds) {
+    // a folded term of either sum: an FMA each for even and odd parts, 64 columns a block
+    constexpr double kTerm = 2.0 * 2.0 * kFgCols;
+    double flops = 0.0;
+    for (int j0 = 0; j0 < f.nz; j0 += kFgSlices) {
+        int kx = 0;
+        for (int j = j0; j < j0 + kFgSlices && j < f.nz; ++j) {
+            const int xlo = bounds[j], xhi = bounds[f.nz + j], ylo = bounds[2 * f.nz + j], yhi = bounds[3 * f.nz + j];
+            if (xlo >= xhi) continue;
+            const FgFold y = fg_fold(ylo, yhi, f.ny);
+            flops += kTerm * f.Hs * ((xhi + 31) / 32 - xlo / 32) * (y.end - y.beg);
+            kx = std::max(kx, fg_fold(xlo, xhi, f.nx).end);
+        }
+        flops += kTerm * f.Hs * f.Ht * kx;
+    }
+    return flops;
 }
 
 cudaError_t launch_field_grid(const FieldGrid &f, const void *s, const int *bounds, double str_re, double str_im,

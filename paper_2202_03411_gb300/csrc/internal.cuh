@@ -394,6 +394,9 @@ cudaError_t launch_field_grid_tables(const FieldGrid &f, cudaStream_t st);
 // Forward from the slices (FP32 or FP64), or from the tensor-core y-sums in f.H.
 cudaError_t launch_field_grid(const FieldGrid &f, const void *s, const int *bounds, double str_re, double str_im,
                               void *A, void *I, int sm_count, cudaStream_t st);
+// Real flops of its folded sums over y and over x and z for the recorded slice
+// geometry (a host copy of the first 4 nz ints of the buffer).
+double field_grid_issued_flops(const FieldGrid &f, const int *bounds_host);
 cudaError_t launch_field_grid_tc(const FieldGrid &f, int Nxp, const int *bounds, const int *chunk_y, double str_re,
                                  double str_im, float2 *A, float *I, int sm_count, cudaStream_t st);
 // Whether a handle of this configuration runs its adjoint through the grid.

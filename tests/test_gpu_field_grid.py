@@ -180,3 +180,40 @@ def test_strip_detector_gradients(rows):
         grads.append(sm.scatman_backward(h, up))
         h.close()
     assert np.linalg.norm(grads[0] - grads[1]) / np.linalg.norm(grads[1]) < 2e-5
+
+
+def _flops(g, s, prec, soft=False, q_list=None):
+    import paper_2202_03411_gb300 as sm
+    h = sm.scatman_create(g, prec, soft=soft, soft_width=0.5, q_list=q_list)
+    sm.scatman_voxelise(h, s)
+    out = sm.scatman_contraction_flops(h)
+    h.close()
+    return out
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "tc_bf16_split"])
+def test_issued_flops_follow_the_box(prec):
+    """The grid's sums skip what a shape leaves empty: a sphere of a quarter of the
+    side in a corner counts well below the filled box (x/z sums: its half-coordinates reach
+    the rim; y sums: a third of the slices, columns and y), and an empty shape nothing."""
+    g = Geometry(96, 96, 96, 1.0, 10.0, 45.0, 200, 190)
+    box, dense = _flops(g, _solid(g), prec)
+    part, dense_part = _flops(g, Shape(SPHERE, r=12.0, cx=30, cy=-30, cz=20, delta=0.01, beta=0.001), prec)
+    none, _ = _flops(g, Shape(SPHERE, r=0.1, cx=0.25, cy=0.25, cz=0.25, delta=0.01, beta=0.001), prec)
+    assert none == 0 and 0 < part < 0.35 * box and dense == dense_part > 4 * box
+    if prec != "tc_bf16_split":
+        # Hs x (y: 96 slices, 3 tiles of columns, 48 half-coordinates; x/z: 6 chunks, 48, Ht), 256 flop each
+        assert box % (256 * 48) == 0
+        Hs_terms = box / (256 * 48)
+        assert any(Hs_terms == Hs * (96 * 3 + 6 * Ht) for Hs in range(4, 97) for Ht in range(4, 97))
+
+
+def test_issued_flops_of_a_fit_are_the_pixel_sums():
+    """A split-phase fit sums over the pixels: what it reports is what the same pixels as a list of q report."""
+    import paper_2202_03411_gb300 as sm
+    g = Geometry(96, 96, 96, 1.0, 10.0, 45.0, 256, 256)
+    h = sm.scatman_create(g, "fp32")
+    q = sm.scatman_get_q(h)
+    h.close()
+    s = Shape(SPHERE, r=30.0, delta=0.01, beta=0.001)
+    assert _flops(g, s, "tc_bf16_split", soft=True) == _flops(g, s, "tc_bf16_split", soft=True, q_list=q)
