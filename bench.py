@@ -617,6 +617,19 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
+def forward_path(precision: str):
+    """What bounds a forward pass of the benchmark's workload, its kernels, and what its
+    flops count, by the sums that the precision mode takes."""
+    grid = "fg_xz_kernel, fg_columns_kernel, fg_pixels_out_kernel)"
+    if not precision.startswith("tc_"):
+        return ("alu" if precision == "fp64" else "latency", "forward pass (fg_y_kernel, " + grid,
+                "CUDA-core flops of the folded sums over y and over x and z; the interpolation is not counted")
+    if "split" in precision:
+        return ("latency", "forward pass (msft_tc_kernel in store mode, " + grid,
+                "tensor-core flops of the sums over y; the x/z sums and the interpolation run on the CUDA cores")
+    return ("tensor", "msft_tc_kernel", "tensor-core flops of the sums over every pixel")
+
+
 def launches_per_pattern(precision: str, n_pix: int, sm_count: int) -> int:
     """Kernels one voxelise + forward launches.  Every mode resets the slice boxes
     and voxelises; the split phases list the work units, sum over y on the tensor
@@ -777,25 +790,24 @@ def main():
     clocks = sampler.stop()
     single_stream = world * B * args.steps / (max_over_ranks(sum(step1_ms), dist, "cuda") / 1e3)
 
-    # the forward pass: its tensor-core work (the sums over y at the grid's
-    # directions) over its whole duration, beside the direct sums' work that it
-    # stands for (8 flop per pixel, occupied voxel and phase product)
+    # the forward pass: the flops of its sums over its whole duration, beside the
+    # direct sums' work (8 flop per pixel, occupied voxel and phase product), which the
+    # single-product modes run and the others stand for
     peaks, peak_kind = measured_peaks()
     n_vox = g.nx * g.ny * g.nz
     products = 2 if "split" in args.precision else 1
-    executed = statistics.mean(issued)                 # real flops the tensor cores execute per pattern
+    executed = statistics.mean(issued)                 # real flops the sums execute per pattern
     direct = 8.0 * g.n_pix * statistics.mean(occupied) * products
     fwd_avg_s = statistics.mean(fwd_ms) / 1e3
     peak = float(peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops")))
-    roofline = {"bound": "latency", "achieved": executed / fwd_avg_s / 1e12, "peak": peak, "unit": "TFLOP/s",
+    bound, kernel, basis = forward_path(args.precision)
+    roofline = {"bound": bound, "achieved": executed / fwd_avg_s / 1e12, "peak": peak, "unit": "TFLOP/s",
                 "frac": executed / fwd_avg_s / 1e12 / peak,
                 "traffic": recorded_traffic("msft_tc_kernel", "paper_2202_03411_gb300/csrc/msft_tc.cu"),
-                "kernel": "forward pass (msft_tc_kernel in store mode, fg_xz_kernel, fg_columns_kernel, "
-                          "fg_pixels_out_kernel)",
+                "kernel": kernel,
                 "peak_source": f"{peak_kind} bf16_tflops_sustained (cuBLAS bf16; f16 has the same nominal rate)",
                 "flops_per_launch": executed,
-                "flops_basis": "tensor-core flops of the sums over y; the x/z sums and the interpolation run on the "
-                               "CUDA cores",
+                "flops_basis": basis,
                 "direct_sum_flops": direct,
                 "direct_sum_basis": "8 flop x pixels x occupied voxels x phase products "
                                     f"({statistics.mean(occupied):.0f} occupied voxels of {n_vox} on average)",

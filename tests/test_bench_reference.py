@@ -36,3 +36,14 @@ def test_reference_arm_prints_one_contract_line():
 
 def test_reference_arm_other_ranks_print_nothing():
     assert _run({"RANK": "1", "WORLD_SIZE": "2"}) == []
+
+
+def test_forward_path_names_the_kernels_that_run():
+    """The roofline entry: only the single-product modes sum over every pixel on the
+    tensor cores; the other modes' forward pass goes through the grid of directions."""
+    sys.path.insert(0, ROOT)
+    import bench
+    for prec, bound, kernel in (("tc_bf16", "tensor", "msft_tc_kernel"), ("tc_f16", "tensor", "msft_tc_kernel"),
+                                ("tc_bf16_split", "latency", "store mode"), ("fp32", "latency", "fg_y_kernel")):
+        got = bench.forward_path(prec)
+        assert got[0] == bound and kernel in got[1] and ("fg_pixels_out_kernel" in got[1]) == (bound != "tensor")
