@@ -217,3 +217,25 @@ def test_issued_flops_of_a_fit_are_the_pixel_sums():
     h.close()
     s = Shape(SPHERE, r=30.0, delta=0.01, beta=0.001)
     assert _flops(g, s, "tc_bf16_split", soft=True) == _flops(g, s, "tc_bf16_split", soft=True, q_list=q)
+
+
+@pytest.mark.parametrize("prec,soft,tol", [("fp64", False, 1e-10), ("fp32", False, 1e-5), ("fp32", True, 1e-5)])
+@pytest.mark.parametrize("g", [
+    Geometry(12, 12, 12, 1.0, 6.0, 45.0, 401, 403),                       # flat: a row of pixels per warp, eight warps
+    Geometry(12, 12, 12, 1.0, 6.0, 45.0, 801, 803),                       # flat: four rows a thread
+    Geometry(12, 12, 12, 1.0, 6.0, 40.0, 431, 429, DETECTOR_UNIFORM_Q),   # uniform-q: two columns a thread
+    Geometry(12, 12, 12, 1.0, 6.0, 40.0, 803, 801, DETECTOR_UNIFORM_Q),   # uniform-q: four
+])
+def test_large_odd_detectors(g, prec, soft, tol):
+    """Each form of the interpolation to the pixels, past its last whole tile: the rim,
+    the middle and a sample against the oracle (the modes' tolerances)."""
+    from gpu_helpers import oracle_field
+    s = Shape(ELLIPSOID, a=4.4, b=3.6, c=4.0, delta=0.01, beta=0.001, latitude=20, longitude=50, rotation=10, cx=0.3)
+    I, _ = run_gpu(g, s, prec, soft=soft)
+    v, u = np.divmod(np.arange(g.n_pix), g.det_nx)
+    rim = (u < 2) | (u >= g.det_nx - 3) | (v < 2) | (v >= g.det_ny - 3) | ((u - g.det_nx // 2) ** 2 + (v - g.det_ny // 2) ** 2 < 30)
+    at = np.union1d(np.flatnonzero(rim), np.random.default_rng(4).choice(g.n_pix, 2000, replace=False))
+    ref, _ = oracle_field(g, s, sample=at, soft=soft)
+    assert rel_l2(I[at], ref) < tol
+    edge = np.flatnonzero(rim[at] & ((u[at] - g.det_nx // 2) ** 2 + (v[at] - g.det_ny // 2) ** 2 >= 30))
+    assert rel_l2(I[at][edge], ref[edge]) < 100 * tol                     # (two to four decades below the peak)
