@@ -707,8 +707,13 @@ __global__ void __launch_bounds__(256) fg_columns_kernel(FieldGrid f) {
         const int a = f.uniform ? p1 : p2, b = f.uniform ? p2 : p1;
         const R *src = (const R *)f.Q + ((size_t)a * f.Ht + b) * 8 + c;
         R v = (R)0;
-#pragma unroll 8
-        for (int j = 0; j < f.jc; ++j) v += src[j * chunk];
+        for (int j0 = 0; j0 < f.jc; j0 += 8) {
+            R t[8];                                     // eight chunks' loads in flight, added in order
+#pragma unroll
+            for (int j = 0; j < 8; ++j) t[j] = j0 + j < f.jc ? src[(j0 + j) * chunk] : (R)0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v += t[j];
+        }
         // first parity = that of direction 1: t on the flat detector, s on the uniform-q one
         const int pq = c >> 1, d = f.uniform ? pq : ((pq & 1) << 1) | (pq >> 1);
         q[p1 * 8 + 2 * d + (c & 1)] = v;
@@ -717,18 +722,28 @@ __global__ void __launch_bounds__(256) fg_columns_kernel(FieldGrid f) {
     const R *we = (const R *)f.w1, *wo = we + (size_t)f.H1 * f.n1;
     R acc[8] = {};
     if (i < f.n1) {
-#pragma unroll 4
-        for (int p = warp; p < f.H1; p += 8) {
-            const R e = we[(size_t)p * f.n1 + i], o = wo[(size_t)p * f.n1 + i];
-            const V4 a = *reinterpret_cast<const V4 *>(q + p * 8), b = *reinterpret_cast<const V4 *>(q + p * 8 + 4);
-            acc[0] = fma(e, a.x, acc[0]);
-            acc[1] = fma(e, a.y, acc[1]);
-            acc[2] = fma(e, a.z, acc[2]);
-            acc[3] = fma(e, a.w, acc[3]);
-            acc[4] = fma(o, b.x, acc[4]);
-            acc[5] = fma(o, b.y, acc[5]);
-            acc[6] = fma(o, b.z, acc[6]);
-            acc[7] = fma(o, b.w, acc[7]);
+        for (int p0 = warp; p0 < f.H1; p0 += 32) {
+            R e[4], o[4];                               // four points' weights in flight
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int p = p0 + 8 * m;
+                e[m] = p < f.H1 ? we[(size_t)p * f.n1 + i] : (R)0;
+                o[m] = p < f.H1 ? wo[(size_t)p * f.n1 + i] : (R)0;
+            }
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int p = p0 + 8 * m;
+                if (p >= f.H1) break;
+                const V4 a = *reinterpret_cast<const V4 *>(q + p * 8), b = *reinterpret_cast<const V4 *>(q + p * 8 + 4);
+                acc[0] = fma(e[m], a.x, acc[0]);
+                acc[1] = fma(e[m], a.y, acc[1]);
+                acc[2] = fma(e[m], a.z, acc[2]);
+                acc[3] = fma(e[m], a.w, acc[3]);
+                acc[4] = fma(o[m], b.x, acc[4]);
+                acc[5] = fma(o[m], b.y, acc[5]);
+                acc[6] = fma(o[m], b.z, acc[6]);
+                acc[7] = fma(o[m], b.w, acc[7]);
+            }
         }
     }
 #pragma unroll
