@@ -888,10 +888,7 @@ def main():
     tc_ms = statistics.mean(pat_ms)
     if fp32 is not None:
         fp32["rel_l2_I_vs_fp64_oracle"] = err_fp32
-        # both modes skip the empty parts of each slice, so this ratio compares
-        # the arithmetic (tensor cores vs FP32 CUDA cores) at nearly equal work
         fp32["tc_speedup_per_pattern"] = fp32["ms_per_pattern"] / tc_ms
-        fp32["executed_flops_ratio_fp32_over_tc"] = fp32["executed_flops_per_pattern"] / (executed / products)
     if tc2 is not None:
         tc2["note"] = (f"{args.precision} is the headline because the benchmarked configuration specifies BF16 "
                        "operands; FP16 has the same tensor rate and a finer mantissa (|s| <= 1 and the phases fit "

@@ -24,9 +24,10 @@
 // error over the whole box (plan_points below), not from the shape.
 //
 // Measured (forward pass with the voxeliser, against the direct sums): 128^3 on
-// 512^2 to 60 degrees, BF16 split phases 74 us (1798); 96^3 on 256^2, FP32
-// 28 us (5195), FP64 164 us (73600, the same ellipsoid); 32^3 on 64^2, FP64 31 us
-// (736); uniform-q 30^3 on 512^2, FP32 29 us (125, the separable sums per pixel row).
+// 512^2 to 60 degrees, BF16 split phases 74 us (1800); 96^3 on 256^2, by the size of the
+// ellipsoid, FP32 27-32 us (4750-5800), FP64 160-196 us (73600-115000); 32^3 on 64^2, FP64
+// 30 us (680-740); uniform-q 30^3 on 512^2, FP32 26-32 us (124, the separable sums
+// per pixel row).
 #include <algorithm>
 #include <cmath>
 #include <complex>
@@ -147,8 +148,9 @@ bool plan_field_grid(const scatman_config &c, int elem, FieldGrid *f) {
 // FP32).  A loss near its minimum shows the pattern's rounding many times larger: over
 // 63 fits of 20^3 - 64^3 voxels the FP32 sums left the loss 7.0e-7 off (the direct
 // FP32 sums 5.4e-7), these 3.4e-7, most of it the slices' own FP32; the pattern 2.1e-7
-// (3.1e-7) and 6e-8.  A fit step of 48^3 on 128^2 takes 530 us instead of 515.  Where the
-// points exceed the FP64 plan's limit the sums stay FP32.
+// (3.1e-7) and 6e-8.  The forward pass takes 40 us instead of 17 at 48^3 on 128^2 and 153
+// instead of 25 at 96^3 on 256^2 (direct: 438 and 8660).  Where the points exceed the
+// FP64 plan's limit the sums stay FP32.
 // Patterns in FP32 keep FP32 sums: 2.1e-7 of the intensity off on the flat detector (the
 // direct sums 2.9e-7), 2.0e-7 on the uniform-q one (its separable sums 1.3e-7: the
 // alternating weights of the interpolation; 1.5e-7 at 67 us instead of 31 with only the

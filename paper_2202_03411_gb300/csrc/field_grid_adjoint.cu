@@ -13,7 +13,7 @@
 // meets only cosines or only sines, and two mirror voxels share a sum.
 //
 // Short kernels, bound by their launches and the latency of their loads: 48^3 on
-// 128^2, FP32: pixels 6.2 us, columns 8.9, x/z 5.2, y 6.4 (the direct sums over pixels
+// 128^2, FP32: pixels 6.2 us, columns 9.2, x/z 5.4, y 5.9 (the direct sums over pixels
 // and voxels: 12.4 ms).
 //
 // All sums have a fixed order (chunks of pixels are added in order), so the
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kFaThreads) fa_pixels_kernel(FieldGrid f, Fiel
 // direction's points.  Block: one point of the per-pixel direction; it adds the
 // chunks of kFaCols columns in shared memory, then a warp sums kFaColPts points
 // over them, its lanes along the columns.  (Five points per warp, so that one block
-// adds the chunks for all, took 18 us instead of 13 at 96^3 on 256^2 pixels: the
+// adds the chunks for all: 11.7 us instead of 9.2 at 48^3 on 128^2 pixels, the
 // points' sums are as long a chain as the chunks'.)
 constexpr int kFaCols = 256;
 constexpr int kFaColPts = 2;
